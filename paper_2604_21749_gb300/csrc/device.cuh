@@ -29,7 +29,7 @@ struct ViewDev {             // one view of a frame
     uint64_t *vis;           // W*H visibility words
 };
 
-struct PairDev {             // one (instance, view) pair that survived host culling
+struct alignas(16) PairDev { // one (instance, view) pair that survived host culling
     float mv[12];            // rows 0..2 of view * model, FP32 (the exact transform)
     // conservative tiny-triangle cull: rows giving X'*w, Y'*w and w with FMA,
     // where X' = X - 1/2 and Y' = Y - 1/2 put the pixel centres on integers;
@@ -149,6 +149,7 @@ struct Q2Entry {             // stage 2 -> stage 3: one tile of one sub-triangle
 
 struct Counters {
     unsigned long long work[kMaxRounds];   // stage-1 work grabs of each round
+    unsigned int xwork[kMaxRounds];        // bitmap units the exact kernel has taken of each round
     unsigned long long q1_count, q1_next;
     unsigned long long q2_count, q2_next;
     unsigned long long overflow1, overflow2;

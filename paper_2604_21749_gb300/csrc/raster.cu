@@ -255,6 +255,7 @@ __device__ __forceinline__ int classify(const FrameDev &f, const Rec r[3], const
 }
 
 #include "stage1.cuh"
+#include "stage1_exact.cuh"
 #include "stage1_win.cuh"
 
 // ---------------------------------------------------------------- stage 2 --

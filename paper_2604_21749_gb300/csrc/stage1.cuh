@@ -919,128 +919,3 @@ __global__ void __launch_bounds__(s1::kThreads, (FUSED || INST) ? 3 : s1::kCullB
     }
     if (FUSED && qn > 0) exact_survivor(&f, wq[lane < qn ? lane : 0], lane < qn);
 }
-
-// Stage 1, exact part of round r, from the survivor bitmap of the cull.  A
-// warp walks its share of the bitmap 32 words at a time: each lane decodes
-// its word to (first triangle, pair) -- the segment is found by a forward
-// search from the warp's previous one, since a warp's words only grow --
-// and the set bits are compacted into a shared-memory batch of up to
-// 32 * kExactK survivors.  A full batch is gathered at once (every lane
-// issues the index and position loads of its kExactK survivors before any
-// arithmetic), parked in shared memory, and run through the exact path one
-// survivor a lane at a time.
-__device__ __forceinline__ uint32_t fastdiv(uint32_t n, uint32_t m, uint32_t sh) {   // (fastdiv_consts)
-    const uint32_t t = __umulhi(n, m);
-    return (t + ((n - t) >> 1)) >> sh;
-}
-
-namespace s1 {
-constexpr int kExactWarps = 4;
-constexpr int kExactBlocks = 5;                      // 96 registers a thread
-constexpr int kExactK = 3;                           // survivors a lane gathers together
-constexpr int kBatch = 32 * kExactK;
-}
-template <bool RAY>
-__global__ void __launch_bounds__(32 * s1::kExactWarps, s1::kExactBlocks)
-    k_stage1_exact(const __grid_constant__ FrameDev f, uint32_t r) {
-    using namespace s1;
-    __shared__ uint2 buf[kExactWarps][kBatch];
-    __shared__ float stage[kExactWarps][kExactK][9][32];   // gathered positions, lane-minor
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const RoundDev rd = f.rounds[r];
-    const uint64_t nwords = rd.w1 - rd.w0;
-    const int n_segs = (int)f.hdr->n_segs;
-    const uint32_t G = kConsumerWarps * f.tpt;
-    const uint64_t per_item = (uint64_t)kConsumers * f.tpt;
-    const uint64_t nw = (uint64_t)gridDim.x * kExactWarps;
-    uint64_t c = (uint64_t)blockIdx.x * kExactWarps + warp;   // the next chunk of 32 words
-    uint32_t m_next = 32 * c + lane < nwords ? __ldcs(f.bits + 32 * c + lane) : 0u;
-    uint32_t m = 0;                                 // bits of the lane's word not yet batched
-    uint64_t t0 = 0;
-    uint32_t pair = 0;
-    int seg = 0;                                    // segment of the warp's last word so far
-    bool more = 32 * c < nwords;
-    while (true) {
-        int n = 0;                                  // survivors in the batch (warp-uniform)
-        while (n < kBatch) {
-            if (__ballot_sync(0xffffffffu, m != 0) == 0) {
-                if (!more) break;
-                m = m_next;                         // advance to chunk c
-                const uint64_t gw = rd.w0 + 32 * c + lane;
-                const uint64_t cn = c + nw;
-                m_next = 32 * cn + lane < nwords ? __ldcs(f.bits + 32 * cn + lane) : 0u;
-                if (__ballot_sync(0xffffffffu, m != 0) != 0) {
-                    int sl = seg;
-                    while (sl + 1 < n_segs && f.segs[sl + 1].word0 <= gw) ++sl;
-                    seg = __shfl_sync(0xffffffffu, sl, 31);
-                    if (m) {
-                        const SegDev &sg = f.segs[sl];
-                        const uint64_t local = gw - sg.word0;
-                        const uint32_t per = sg.npairs * G;         // words per item (<= 64 * 32)
-                        uint64_t jb;
-                        uint32_t pi, g;
-                        if (sg.npairs == 1 && local < (1ull << 32)) {   // one pair: item and group
-                            jb = fastdiv((uint32_t)local, f.g_m, f.g_s);
-                            g = (uint32_t)local - (uint32_t)jb * G;
-                            pi = 0;
-                        } else {
-                            jb = local < (1ull << 32) ? (uint64_t)((uint32_t)local / per) : local / per;
-                            const uint32_t rem = (uint32_t)(local - jb * per);
-                            pi = rem / G;
-                            g = rem - pi * G;
-                        }
-                        t0 = jb * per_item + 32ull * g;
-                        pair = sg.pair0 + pi;
-                    }
-                }
-                c = cn;
-                more = 32 * c < nwords;
-                continue;
-            }
-            // append the lowest set bits of every lane's word, as many as fit
-            const int cnt = __popc(m);
-            int incl = cnt;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += v;
-            }
-            const int total = __shfl_sync(0xffffffffu, incl, 31);
-            int at = n + incl - cnt;
-            while (m && at < kBatch) {
-                const int bit = __ffs(m) - 1;
-                m &= m - 1u;
-                buf[warp][at++] = make_uint2((uint32_t)(t0 + (uint64_t)bit), pair);
-            }
-            n = min(n + total, kBatch);
-        }
-        if (n == 0) break;
-        __syncwarp();
-        if (f.stats && lane == 0) stat_add(f, kStatFast, (unsigned long long)n);
-        uint2 e[kExactK];
-        bool live[kExactK];
-        Tri9 p[kExactK];
-#pragma unroll
-        for (int u = 0; u < kExactK; ++u) {
-            live[u] = lane + 32 * u < n;
-            e[u] = buf[warp][live[u] ? lane + 32 * u : 0];
-        }
-#pragma unroll
-        for (int u = 0; u < kExactK; ++u) exact_gather(f, e[u], live[u], p[u]);
-        // the positions wait in shared memory, so the exact path of one
-        // survivor holds no registers for the others
-#pragma unroll
-        for (int u = 0; u < kExactK; ++u)
-#pragma unroll
-            for (int c = 0; c < 9; ++c) stage[warp][u][c][lane] = p[u].v[c];
-        __syncwarp();
-#pragma unroll 1
-        for (int u = 0; u < kExactK; ++u) {
-            if (!__any_sync(0xffffffffu, live[u])) continue;
-            Tri9 q;
-#pragma unroll
-            for (int c = 0; c < 9; ++c) q.v[c] = stage[warp][u][c][lane];
-            exact_compute<RAY>(f, buf[warp][live[u] ? lane + 32 * u : 0], live[u], q);
-        }
-    }
-}

@@ -1,0 +1,380 @@
+// stage1_exact.cuh -- the exact part of stage 1 (Section 4.1), included by raster.cu.
+//
+// A warp takes the survivors that the cull left in the round's bitmap, up to
+// 32 * kExactK at a time, and works in three steps that meet in the warp's
+// shared memory, so that no step holds registers for another:
+//   gather     every lane loads the indices and positions of its kExactK
+//              survivors before any arithmetic;
+//   set up     one survivor a lane: transform, cull, snap, classify; a small
+//              triangle leaves its snapped vertices, 1/depths and pixel range;
+//   rasterize  the pixel ranges of the whole batch laid end to end, 32 pixels
+//              a step, one a lane, whatever triangles they belong to.
+// A lane that walked its own triangle's pixels alone would keep the warp for
+// the largest range of the 32, with the division and the atomic issued at
+// nearly every step for a lane or two.
+#pragma once
+
+namespace s1 {
+constexpr int kExactWarps = 4;
+constexpr int kExactBlocks = 5;                      // 96 registers a thread
+constexpr int kExactK = 3;                           // survivors a lane gathers together
+constexpr int kBatch = 32 * kExactK;
+constexpr uint32_t kUnits = 13;                      // units dealt out of one block of the bitmap
+constexpr int kDenseBits = 12;                       // words with as many survivors are unpacked by the whole warp
+constexpr uint32_t kSegPx = 2048;                    // pixels whose triangle starts are marked at once
+
+// A small triangle ready for the pixel loop, 48 bytes: eight lanes' 16-byte
+// loads of neighbouring records touch every bank once.
+struct __align__(16) SmallTri {
+    int e0, e1, A;             // edge functions 0 and 1 at the centre of pixel (x0, y0); their sum with edge 2
+    uint32_t d0;               // edge 0 (vertex 1 to 2): dx & 0xFFFF | dy << 16, in subpixels
+    uint32_t d1;               // edge 1 (vertex 2 to 0)
+    float iz[3];               // 1/depth of the vertices
+    uint32_t id;               // global id, low word
+    uint32_t idh;              // its 4 high bits | bit 4 + k: edge k is not top-left | view << 8
+    uint32_t at;               // x0 | y0 << 16 of the pixel range
+    uint32_t shape;            // its width w | ceil(2^20 / w) << 11
+};
+
+static_assert(sizeof(SmallTri) == 3 * sizeof(uint4), "a record is three 16-byte words");
+
+struct ExactWarp {
+    uint2 e[kBatch];           // (triangle, pair)
+    uint4 t[kBatch][3];        // the nine gathered floats, overwritten by the SmallTri at set-up
+    uint32_t npx[kBatch];      // pixels of the range (0: nothing to rasterize)
+    uint32_t list[kBatch];     // triangles with pixels: first pixel of the batch | slot << 20
+    uint32_t starts[kSegPx / 32];   // bit i: pixel i of the segment is a triangle's first
+};
+}  // namespace s1
+
+__device__ __forceinline__ uint32_t fastdiv(uint32_t n, uint32_t m, uint32_t sh) {   // (fastdiv_consts)
+    const uint32_t t = __umulhi(n, m);
+    return (t + ((n - t) >> 1)) >> sh;
+}
+
+// Set-up of the survivor in `slot`: its class, and for a small triangle its
+// record in the warp's shared memory, with its number of pixels (else 0).
+// Same decisions and values as outcode, snap and setup_subtri give; what is
+// left out cannot change them:
+//   - inside every plane is decided from w >= near, |x| <= 128 w, |y| <= 128 w,
+//     which have the signs of the five plane values (a sum of two finite
+//     floats rounds to zero only when it is zero; NaN fails both forms; an
+//     infinite 128 w takes the outcodes);
+//   - snap's clamp: inside the guard band |X| < 129 * 8192 * 256 < 2^29, once
+//     1/w is finite; vertices with w < 2^-120 send the triangle to stage 2;
+//   - its two multiplications by H/2 and 256 as one by 128 H (a scaling by a
+//     power of two is exact).
+template <bool RAY>
+__device__ __forceinline__ void exact_setup(const FrameDev &f, s1::ExactWarp &S, int slot, bool live) {
+    uint32_t npx = 0;
+    bool queue = false;
+    uint64_t id = 0;
+    uint2 e = make_uint2(0u, 0u);
+    const MeshDev *mesh = f.meshes;
+    unsigned st = kStatCount;
+    if (live) {
+        e = S.e[slot];
+        const PairDev &pr = f.pairs[e.y];
+        const ViewDev &vw = f.views[pr.view];
+        const float4 pa = reinterpret_cast<const float4 *>(S.t[slot])[0], pb = reinterpret_cast<const float4 *>(S.t[slot])[1];
+        const float p[9] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w, __uint_as_float(S.t[slot][2].x)};
+        // (scalar: the assembler contracts packed mul.rn.f32x2 / add.rn.f32x2 pairs into FMAs)
+        float mv[12];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            const float4 row = reinterpret_cast<const float4 *>(pr.mv)[q];
+            mv[4 * q] = row.x; mv[4 * q + 1] = row.y; mv[4 * q + 2] = row.z; mv[4 * q + 3] = row.w;
+        }
+        CV c[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) c[k] = to_clip(mv, p[3 * k], p[3 * k + 1], p[3 * k + 2], vw.fx, vw.fy);
+        id = pr.base + e.x;
+        mesh = f.meshes + pr.mesh;
+        const float wmin = fmaxf(vw.nearv, 7.5231638e-37f);      // 2^-120
+        bool inside = true;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float gw = __fmul_rn(kGuard, c[k].w);
+            inside &= (c[k].w >= wmin) & (gw < INFINITY) & (fabsf(c[k].x) <= gw) & (fabsf(c[k].y) <= gw);
+        }
+        if (!inside) {
+            // beyond one clip plane, or to be clipped by stage 2
+            queue = (outcode(c[0], vw.nearv) & outcode(c[1], vw.nearv) & outcode(c[2], vw.nearv)) == 0;
+            if (!queue) st = kStatClip;
+        } else {
+            int X[3], Y[3];
+            float iz[3];
+            const float sx = __fmul_rn(vw.hw, 256.0f), sy = __fmul_rn(vw.hh, 256.0f);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                iz[k] = __frcp_rn(c[k].w);
+                X[k] = __float2int_rn(__fmul_rn(__fadd_rn(__fmul_rn(c[k].x, iz[k]), 1.0f), sx));
+                Y[k] = __float2int_rn(__fmul_rn(__fadd_rn(__fmul_rn(c[k].y, iz[k]), 1.0f), sy));
+            }
+            const int minX = min(X[0], min(X[1], X[2])), maxX = max(X[0], max(X[1], X[2]));
+            const int minY = min(Y[0], min(Y[1], Y[2])), maxY = max(Y[0], max(Y[1], Y[2]));
+            const bool big = max(maxX - minX, maxY - minY) >= (1 << 14);
+            const int ux = X[1] - X[0], uy = Y[1] - Y[0], wx = X[2] - X[0], wy = Y[2] - Y[0];
+            const bool front = big ? (int64_t)ux * wy - (int64_t)wx * uy > 0 : ux * wy - wx * uy > 0;
+            int x0, x1, y0, y1;
+            centre_range(minX, maxX, vw.W, x0, x1);
+            centre_range(minY, maxY, vw.H, y0, y1);
+            if (!front) {
+                st = kStatBack;
+            } else if (x0 > x1 || y0 > y1) {
+                st = kStatTiny;
+            } else {
+                const uint32_t w = (uint32_t)(x1 - x0 + 1), n = w * (uint32_t)(y1 - y0 + 1);
+                queue = big || n > f.s1_max;
+                if (!queue) {
+                    npx = n;
+                    // m = ceil(2^20 / w): the approximate quotient is off by less than 1/w, so its
+                    // floor is the true one or, where w divides 2^20, perhaps one less
+                    uint32_t m = (uint32_t)(1048576.0f * rcp_approx((float)w));
+                    m += m * w < (1u << 20) ? 1u : 0u;
+                    // edge k runs from vertex k+1 to vertex k+2; (px, py) is the first pixel's centre
+                    const int px = 256 * x0 + 128, py = 256 * y0 + 128;
+                    const int dx0 = X[2] - X[1], dy0 = Y[2] - Y[1], dx1 = -wx, dy1 = -wy;
+                    const int e0 = dx0 * (py - Y[1]) - dy0 * (px - X[1]), e1 = dx1 * (py - Y[2]) - dy1 * (px - X[2]);
+                    const uint32_t b0 = (dy0 < 0 || (dy0 == 0 && dx0 < 0)) ? 0u : 16u;
+                    const uint32_t b1 = (dy1 < 0 || (dy1 == 0 && dx1 < 0)) ? 0u : 32u;
+                    const uint32_t b2 = (uy < 0 || (uy == 0 && ux < 0)) ? 0u : 64u;
+                    S.t[slot][0] = make_uint4((uint32_t)e0, (uint32_t)e1, (uint32_t)(ux * wy - wx * uy),
+                                              ((uint32_t)dx0 & 0xFFFFu) | (uint32_t)dy0 << 16);
+                    S.t[slot][1] = make_uint4(((uint32_t)dx1 & 0xFFFFu) | (uint32_t)dy1 << 16, __float_as_uint(iz[0]),
+                                              __float_as_uint(iz[1]), __float_as_uint(iz[2]));
+                    S.t[slot][2] = make_uint4((uint32_t)id, (uint32_t)(id >> 32) | b0 | b1 | b2 | pr.view << 8,
+                                              (uint32_t)x0 | (uint32_t)y0 << 16, w | m << 11);
+                }
+            }
+        }
+    }
+    S.npx[slot] = npx;
+    q1_append<RAY>(f, queue, id, e.y, mesh, e.x);
+    if (f.stats && live) {
+        stat_add(f, kStatIn, 1);
+        if (st != kStatCount) stat_add(f, st, 1);
+        if (npx) stat_add(f, kStatS1, 1);
+    }
+}
+
+// Rasterizes the small triangles of a batch: slot s holds npx[s]
+// pixels.  The ranges are laid end to end in the order (lane, u); the
+// triangle of pixel i is the last one to start at or before i, found by
+// counting the marked starts up to it.  The range is walked row by row: pixel
+// k of a range of width w is (k mod w, k / w), the division as a multiplication
+// by m = ceil(2^20 / w), exact for k, w <= 1024 (k (m w - 2^20) < 2^20).  The
+// edge functions are int32: both extents are below 2^14 subpixels, so
+// |E| < 2^30 at every visited sample, and E2 = A - E0 - E1 exactly.
+__device__ __forceinline__ void exact_raster(const FrameDev &f, s1::ExactWarp &S, int lane) {
+    using namespace s1;
+    uint32_t npx[kExactK], own = 0;                  // own: pixels | triangles << 20
+#pragma unroll
+    for (int u = 0; u < kExactK; ++u) npx[u] = S.npx[lane + 32 * u];
+#pragma unroll
+    for (int u = 0; u < kExactK; ++u) own += npx[u] ? npx[u] + (1u << 20) : 0u;
+    uint32_t incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    const uint32_t P = __shfl_sync(0xffffffffu, incl, 31) & 0xFFFFFu;
+    if (P == 0) return;
+    const uint32_t at0 = incl - own;
+    uint32_t at = at0;
+#pragma unroll
+    for (int u = 0; u < kExactK; ++u)
+        if (npx[u]) {
+            S.list[at >> 20] = (at & 0xFFFFFu) | (uint32_t)(lane + 32 * u) << 20;
+            at += npx[u] + (1u << 20);
+        }
+    const uint32_t upto = 0xffffffffu >> (31 - lane);
+    int first = -1;                                  // triangles that start before the window, less one
+    for (uint32_t sb = 0; sb < P; sb += kSegPx) {
+        const uint32_t nwin = (min(P - sb, kSegPx) + 31) / 32;
+        for (uint32_t w = lane; w < nwin; w += 32) S.starts[w] = 0;
+        __syncwarp();
+        at = at0;
+#pragma unroll
+        for (int u = 0; u < kExactK; ++u)
+            if (npx[u]) {
+                const uint32_t i = (at & 0xFFFFFu) - sb;
+                if (i < kSegPx) atomicOr(&S.starts[i >> 5], 1u << (i & 31));
+                at += npx[u] + (1u << 20);
+            }
+        __syncwarp();
+        for (uint32_t w = 0; w < nwin; ++w) {
+            const uint32_t word = S.starts[w], i = sb + 32 * w + lane;
+            const int o = first + __popc(word & upto);
+            first += __popc(word);
+            if (i >= P) continue;
+            const uint32_t L = S.list[o], k = i - (L & 0xFFFFFu);
+            const uint4 *t = S.t[L >> 20];
+            const uint4 ta = t[0], tb = t[1], tc = t[2];
+            const uint32_t dy = (k * (tc.w >> 11)) >> 20, dx = k - dy * (tc.w & 2047u);
+            // one column changes E_k by -256 dy_k and one row by 256 dx_k
+            const int e0 = (int)ta.x + (int)dy * ((int)(ta.w << 16) >> 8) - (int)dx * (((int)ta.w >> 16) << 8);
+            const int e1 = (int)ta.y + (int)dy * ((int)(tb.x << 16) >> 8) - (int)dx * (((int)tb.x >> 16) << 8);
+            const int e2 = (int)ta.z - e0 - e1;
+            const int b0 = (tc.y >> 4) & 1, b1 = (tc.y >> 5) & 1, b2 = (tc.y >> 6) & 1;
+            if (((e0 - b0) | (e1 - b1) | (e2 - b2)) < 0) continue;
+            const float s = __fadd_rn(__fadd_rn(__fmul_rn(__int2float_rn(e0), __uint_as_float(tb.y)),
+                                                __fmul_rn(__int2float_rn(e1), __uint_as_float(tb.z))),
+                                      __fmul_rn(__int2float_rn(e2), __uint_as_float(tb.w)));
+            const float depth = __fdiv_rn(__int2float_rn((int)ta.z), s);
+            const ViewDev &vw = f.views[tc.y >> 8];
+            const uint64_t key = (uint64_t)(__float_as_uint(depth) >> 3) << 36 | (uint64_t)(tc.y & 15u) << 32 | tc.x;
+            depth_min(vw.vis, (size_t)((tc.z >> 16) + dy) * (size_t)vw.W + ((tc.z & 0xFFFFu) + dx), key);
+        }
+        __syncwarp();
+    }
+}
+
+// The exact kernel, round r.  Warps take the bitmap in units from a counter:
+// survivors come in clusters where the view looks closely, and a fixed deal of
+// 32-word chunks left some SMs with twice the average (the ordinary full-HD
+// view of a 4.2 M-triangle mesh: 179 us, 117 us now).  A unit is four words
+// (128 triangles of one pair, a 16-byte load) for each of 2^ll lanes, in runs
+// of eight words kUnits runs apart, so that a cluster spreads over several
+// units.  2^ll is the largest of 1 .. 32 that gives every warp twelve units:
+// one address takes an atomic add every 1.8 ns, which 32-word units would
+// make the bound of the billion-triangle frame (1.75 ms against 0.93).  Frames
+// too small for any of that deal single words, so that all warps work.  The
+// next grab and the words of the next unit are in flight while a batch runs.
+template <bool RAY>
+__global__ void __launch_bounds__(32 * s1::kExactWarps, s1::kExactBlocks)
+    k_stage1_exact(const __grid_constant__ FrameDev f, uint32_t r) {
+    using namespace s1;
+    __shared__ ExactWarp sw[kExactWarps];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    ExactWarp &S = sw[warp];
+    const RoundDev rd = f.rounds[r];
+    const uint64_t nwords = rd.w1 - rd.w0;
+    const int n_segs = (int)f.hdr->n_segs;
+    const uint32_t G = kConsumerWarps * f.tpt;
+    const uint64_t per_item = (uint64_t)kConsumers * f.tpt;
+    const uint32_t nw = gridDim.x * kExactWarps;
+    const bool quad = nwords >= 16ull * nw;         // 16-byte loads (a round's words are a multiple of 8)
+    int ll = quad ? 5 : 0;
+    while (ll > 0 && nwords >> (ll + 2) < 12ull * nw) --ll;
+    // units of single loads follow one another; larger ones take two lanes a run, kUnits units a block
+    const uint32_t block = ll ? kUnits << (ll + 2) : quad ? 4u : 1u;   // words
+    const uint32_t per_block = ll ? kUnits : 1u;
+    const uint32_t nunits = (uint32_t)((nwords + block - 1) / block) * per_block;   // (at most 2^34 words)
+    const uint64_t lane0 = lane >= 1 << ll ? nwords : ll ? (uint64_t)(lane >> 1) * 8 * kUnits + 4 * (lane & 1) : 0;
+    uint32_t next = 0;                              // lane 0: the unit after the one being fetched
+    if (lane == 0) next = atomicAdd(&f.ctr->xwork[r], 1u);
+    uint64_t word = 0;                              // the lane's first word of the unit
+    bool more = true;
+    // moves to the next unit and issues its load
+    auto fetch = [&]() -> uint4 {
+        const uint32_t unit = __shfl_sync(0xffffffffu, next, 0);
+        more = unit < nunits;
+        if (lane == 0 && more) next = atomicAdd(&f.ctr->xwork[r], 1u);
+        const uint32_t b = ll ? unit / kUnits : unit;
+        word = lane0 + (uint64_t)b * block + (ll ? 8 * (unit - b * kUnits) : 0u);
+        uint4 w = make_uint4(0u, 0u, 0u, 0u);
+        if (more && word < nwords) {
+            if (quad) w = __ldcs(reinterpret_cast<const uint4 *>(f.bits + word));
+            else w.x = __ldcs(f.bits + word);
+        }
+        return w;
+    };
+    uint4 w_next = fetch();
+    uint32_t m = 0, m1 = 0, m2 = 0, m3 = 0;         // bits of the lane's words not yet batched
+    uint32_t t0 = 0, pair = 0;                      // the triangle of bit 0 of m, and its pair
+    int seg = 0;                                    // segment of the lane's last run so far
+    const unsigned lt_mask = (1u << lane) - 1u;
+    while (true) {
+        int n = 0;                                  // survivors in the batch (warp-uniform)
+        while (n < kBatch) {
+            if (__ballot_sync(0xffffffffu, m != 0) == 0) {
+                if (__ballot_sync(0xffffffffu, (m1 | m2 | m3) != 0)) {
+                    m = m1; m1 = m2; m2 = m3; m3 = 0;   // the next word of the runs
+                    t0 += 32;
+                    continue;
+                }
+                if (!more) break;
+                m = w_next.x; m1 = w_next.y; m2 = w_next.z; m3 = w_next.w;   // the next unit
+                const uint64_t at = rd.w0 + word;
+                w_next = fetch();
+                if (m | m1 | m2 | m3) {
+                    while (seg + 1 < n_segs && f.segs[seg + 1].word0 <= at) ++seg;
+                    const SegDev &sg = f.segs[seg];
+                    const uint64_t local = at - sg.word0;
+                    const uint32_t per = sg.npairs * G;         // words per item (<= 64 * 32)
+                    uint64_t jb;
+                    uint32_t pi, g;
+                    if (sg.npairs == 1 && local < (1ull << 32)) {   // one pair: item and group
+                        jb = fastdiv((uint32_t)local, f.g_m, f.g_s);
+                        g = (uint32_t)local - (uint32_t)jb * G;
+                        pi = 0;
+                    } else {
+                        jb = local < (1ull << 32) ? (uint64_t)((uint32_t)local / per) : local / per;
+                        const uint32_t rem = (uint32_t)(local - jb * per);
+                        pi = rem / G;
+                        g = rem - pi * G;
+                    }
+                    t0 = (uint32_t)(jb * per_item) + 32u * g;
+                    pair = sg.pair0 + pi;
+                }
+                continue;
+            }
+            const int cnt = __popc(m);
+            const unsigned dense = __ballot_sync(0xffffffffu, cnt >= kDenseBits);
+            if (dense) {
+                // a dense word: its bits a lane each, as many as fit
+                const int l = __ffs(dense) - 1;
+                const uint32_t bits = __shfl_sync(0xffffffffu, m, l), wt = __shfl_sync(0xffffffffu, t0, l),
+                               wp = __shfl_sync(0xffffffffu, pair, l);
+                const bool set = (bits >> lane) & 1u;
+                const int to = n + __popc(bits & lt_mask);
+                if (set && to < kBatch) S.e[to] = make_uint2(wt + lane, wp);
+                const unsigned rest = __ballot_sync(0xffffffffu, set && to >= kBatch);
+                if (lane == l) m = rest;
+                n = min(n + __popc(bits), kBatch);
+                continue;
+            }
+            // sparse words: every lane appends its first bits, as many as fit
+            int incl = cnt;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            const int total = __shfl_sync(0xffffffffu, incl, 31);
+            int to = n + incl - cnt;
+            while (m && to < kBatch) {
+                const int bit = __ffs(m) - 1;
+                m &= m - 1u;
+                S.e[to++] = make_uint2(t0 + (uint32_t)bit, pair);
+            }
+            n = min(n + total, kBatch);
+        }
+        if (n == 0) break;
+        __syncwarp();
+        if (f.stats && lane == 0) stat_add(f, kStatFast, (unsigned long long)n);
+        {
+            Tri9 p[kExactK];
+#pragma unroll
+            for (int u = 0; u < kExactK; ++u) {
+                const bool live = lane + 32 * u < n;
+                exact_gather(f, S.e[live ? lane + 32 * u : 0], live, p[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < kExactK; ++u) {
+                float4 *t = reinterpret_cast<float4 *>(S.t[lane + 32 * u]);
+                t[0] = make_float4(p[u].v[0], p[u].v[1], p[u].v[2], p[u].v[3]);
+                t[1] = make_float4(p[u].v[4], p[u].v[5], p[u].v[6], p[u].v[7]);
+                S.t[lane + 32 * u][2].x = __float_as_uint(p[u].v[8]);
+            }
+        }
+#pragma unroll 1
+        for (int u = 0; u < kExactK; ++u)           // (a lane reads and writes its own slots only)
+            exact_setup<RAY>(f, S, lane + 32 * u, lane + 32 * u < n);
+        __syncwarp();
+        exact_raster(f, S, lane);
+        __syncwarp();
+    }
+}
