@@ -1,4 +1,7 @@
 // raster.cu -- clear, stage 1, stage 2 and stage 3 kernels (Sections 4.1-4.3).
+#include <cstddef>
+#include <type_traits>
+
 #include "internal.h"
 
 namespace curast {
@@ -134,9 +137,10 @@ __device__ __noinline__ void q1_overflow_ray(const FrameDev *fp, uint64_t id, ui
 
 // Warp-aggregated append to queue 1 (ballot + popc + one atomicAdd per warp).
 // Lanes whose slot lies beyond the capacity rasterize their triangle in place.
+// px: the pixels of its visible range (0 where it is to be clipped).
 // f must live in parameter or global memory (its address is passed on).
 template <bool RAY>
-__device__ __forceinline__ void q1_append(const FrameDev &f, bool want, uint64_t id, uint32_t pidx,
+__device__ __forceinline__ void q1_append(const FrameDev &f, bool want, uint32_t px, uint64_t id, uint32_t pidx,
                                           const MeshDev *mesh, uint64_t t) {
     const unsigned active = __activemask();
     const unsigned m = __ballot_sync(active, want);
@@ -147,12 +151,13 @@ __device__ __forceinline__ void q1_append(const FrameDev &f, bool want, uint64_t
     if (lane == leader) base = atomicAdd(&f.ctr->q1_count, (unsigned long long)__popc(m));
     base = __shfl_sync(active, base, leader);
     if (!want) return;
+    if (px) atomicAdd(&f.ctr->q1_px, (unsigned long long)px);
     const unsigned long long slot = base + __popc(m & ((1u << lane) - 1u));
     if (slot < f.q1_cap) {
         Q1Entry e;
         e.id = id;
         e.pair = pidx;
-        e.pad = 0;
+        e.small = 0;
         f.q1[slot] = e;
     } else {
         if (RAY) q1_overflow_ray(&f, id, pidx, mesh, t);
@@ -258,197 +263,112 @@ __device__ __forceinline__ int classify(const FrameDev &f, const Rec r[3], const
 #include "stage1_exact.cuh"
 #include "stage1_win.cuh"
 
-// ---------------------------------------------------------------- stage 2 --
-// Section 4.2: one warp per queued triangle.  The triangle is clipped
-// (Sutherland-Hodgman, near plane and guard band) and fan-triangulated;
-// sub-triangles with a bbox of at most s2_max pixels are rasterized by the
-// warp with the 1D pixel loop, larger ones are split along tile boundaries
-// into stage-3 parts.
-__device__ __forceinline__ void q2_append(const FrameDev &f, bool want, const SubTri &s, uint32_t view, int tx,
-                                          int ty, const ViewDev &vw) {
-    const unsigned active = __activemask();
-    const unsigned m = __ballot_sync(active, want);
-    if (m == 0) return;
-    const int lane = threadIdx.x & 31;
-    const int leader = __ffs(m) - 1;
-    unsigned long long base = 0;
-    if (lane == leader) base = atomicAdd(&f.ctr->q2_count, (unsigned long long)__popc(m));
-    base = __shfl_sync(active, base, leader);
-    if (!want) return;
-    const unsigned long long slot = base + __popc(m & ((1u << lane) - 1u));
-    if (slot < f.q2_cap) {
-        Q2Entry e;
-        for (int k = 0; k < 3; ++k) { e.X[k] = s.X[k]; e.Y[k] = s.Y[k]; e.iz[k] = s.iz[k]; }
-        e.view = view;
-        e.id = s.id;
-        e.tx = (uint32_t)tx;
-        e.ty = (uint32_t)ty;
-        e.pair = 0;
-        e.ray = 0;
-        f.q2[slot] = e;
-        if (f.s3_bin) atomicAdd(&f.tile_cnt[vw.tile0 + (uint32_t)ty * vw.ntx + (uint32_t)tx], 1u);
-    } else {
-        atomicAdd(&f.ctr->overflow2, 1ull);
-        const int ts = 1 << f.tile_log2;
-        raster_range(s, max(s.x0, tx * ts), min(s.x1, tx * ts + ts - 1), max(s.y0, ty * ts),
-                     min(s.y1, ty * ts + ts - 1), 0, 1, vw.vis, vw.W);
-    }
-}
-
-// The same for one tile of a triangle that takes the ray-cast stage 3: the
-// entry names the triangle (id, pair) and its visible pixel range.
-__device__ __forceinline__ void q2_append_ray(const FrameDev &f, bool want, uint64_t id, uint32_t pidx, uint32_t view,
-                                              int x0, int x1, int y0, int y1, int tx, int ty, const ViewDev &vw) {
-    const unsigned active = __activemask();
-    const unsigned m = __ballot_sync(active, want);
-    if (m == 0) return;
-    const int lane = threadIdx.x & 31;
-    const int leader = __ffs(m) - 1;
-    unsigned long long base = 0;
-    if (lane == leader) base = atomicAdd(&f.ctr->q2_count, (unsigned long long)__popc(m));
-    base = __shfl_sync(active, base, leader);
-    if (!want) return;
-    const unsigned long long slot = base + __popc(m & ((1u << lane) - 1u));
-    if (slot < f.q2_cap) {
-        Q2Entry e;
-        e.X[0] = x0; e.X[1] = x1; e.X[2] = 0;
-        e.Y[0] = y0; e.Y[1] = y1; e.Y[2] = 0;
-        e.iz[0] = e.iz[1] = e.iz[2] = 0.0f;
-        e.view = view;
-        e.id = id;
-        e.tx = (uint32_t)tx;
-        e.ty = (uint32_t)ty;
-        e.pair = pidx;
-        e.ray = 1;
-        f.q2[slot] = e;
-        if (f.s3_bin) atomicAdd(&f.tile_cnt[vw.tile0 + (uint32_t)ty * vw.ntx + (uint32_t)tx], 1u);
-    } else {
-        atomicAdd(&f.ctr->overflow2, 1ull);
-        const int ts = 1 << f.tile_log2;
-        RayTri R;
-        if (ray_tri_of(f, pidx, id, R))
-            ray_range(R, max(x0, tx * ts), min(x1, tx * ts + ts - 1), max(y0, ty * ts), min(y1, ty * ts + ts - 1), 0,
-                      1, vw, id);
-    }
-}
-
-__global__ void __launch_bounds__(256) k_stage2(FrameDev f) {
-    const int lane = threadIdx.x & 31;
-    const unsigned long long total = *((volatile unsigned long long *)&f.ctr->q1_count);
-    const unsigned long long n = total < f.q1_cap ? total : f.q1_cap;
-    unsigned long long n_s2 = 0, n_parts = 0;
-    for (;;) {
-        unsigned long long i = 0;
-        if (lane == 0) i = atomicAdd(&f.ctr->q1_next, 1ull);
-        i = __shfl_sync(0xffffffffu, i, 0);
-        if (i >= n) break;
-        const Q1Entry e = f.q1[i];
-        const PairDev &pr = f.pairs[e.pair];
-        const ViewDev vw = f.views[pr.view];
-        const MeshDev mesh = f.meshes[pr.mesh];
-        CV c[3];
-        load_clip(f, mesh, e.pair, e.id - pr.base, vw, c);
-        CV poly[kMaxPoly];
-        int np;
-        if ((outcode(c[0], vw.nearv) | outcode(c[1], vw.nearv) | outcode(c[2], vw.nearv)) == 0) {
-            // inside every plane: Sutherland-Hodgman would return it unchanged
-            poly[0] = c[0]; poly[1] = c[1]; poly[2] = c[2];
-            np = 3;
-        } else {
-            np = clip_polygon(c, vw.nearv, poly);
-        }
-        if (np < 3) continue;
-        int X[kMaxPoly], Y[kMaxPoly];
-        float iz[kMaxPoly];
-        for (int k = 0; k < np; ++k) snap(poly[k], vw.hw, vw.hh, X[k], Y[k], iz[k]);
-        if (f.s3_ray) {
-            // the paper's stage 3: a triangle whose visible bbox holds more
-            // than s2_max pixel centres is ray cast over that range, in tiles
-            int x0, x1, y0, y1;
-            const int64_t cnt = poly_range(X, Y, np, vw.W, vw.H, x0, x1, y0, y1);
-            if (cnt == 0) continue;
-            if (cnt > (int64_t)f.s2_max) {
-                const int tl = (int)f.tile_log2;
-                const int tx0 = x0 >> tl, tx1 = x1 >> tl, ty0 = y0 >> tl, ty1 = y1 >> tl;
-                const int ntx = tx1 - tx0 + 1;
-                const int nt = ntx * (ty1 - ty0 + 1);
-                for (int kb = 0; kb < nt; kb += 32) {
-                    const int k = kb + lane;
-                    const bool want = k < nt;
-                    const int tx = tx0 + (want ? k % ntx : 0), ty = ty0 + (want ? k / ntx : 0);
-                    q2_append_ray(f, want, e.id, e.pair, pr.view, x0, x1, y0, y1, tx, ty, vw);
-                    n_parts += want;
-                }
-                continue;
-            }
-        }
-        for (int j = 1; j + 1 < np; ++j) {
-            SubTri s;
-            s.X[0] = X[0]; s.X[1] = X[j]; s.X[2] = X[j + 1];
-            s.Y[0] = Y[0]; s.Y[1] = Y[j]; s.Y[2] = Y[j + 1];
-            s.iz[0] = iz[0]; s.iz[1] = iz[j]; s.iz[2] = iz[j + 1];
-            s.id = e.id;
-            if (!setup_subtri(s, vw.W, vw.H)) continue;
-            const int64_t cnt = (int64_t)(s.x1 - s.x0 + 1) * (int64_t)(s.y1 - s.y0 + 1);
-            if (cnt <= (int64_t)f.s2_max) {
-                raster_range<4>(s, s.x0, s.x1, s.y0, s.y1, lane, 32, vw.vis, vw.W);
-                n_s2 += (lane == 0);
-            } else {
-                const int tl = (int)f.tile_log2;
-                const int tx0 = s.x0 >> tl, tx1 = s.x1 >> tl, ty0 = s.y0 >> tl, ty1 = s.y1 >> tl;
-                const int ntx = tx1 - tx0 + 1;
-                const int nt = ntx * (ty1 - ty0 + 1);
-                for (int kb = 0; kb < nt; kb += 32) {
-                    const int k = kb + lane;
-                    const bool want = k < nt;
-                    const int tx = tx0 + (want ? k % ntx : 0), ty = ty0 + (want ? k / ntx : 0);
-                    q2_append(f, want, s, pr.view, tx, ty, vw);
-                    n_parts += want;
-                }
-            }
-        }
-    }
-    if (f.stats) {
-        stat_add(f, kStatS2, n_s2);
-        stat_add(f, kStatParts, n_parts);
-    }
-}
+#include "stage2.cuh"
 
 // ---------------------------------------------------------------- stage 3 --
-// Section 4.3: one block per tile part; its threads walk the tile's pixels
-// (restricted to the sub-triangle's bbox) line by line -- with edge
-// functions, or, in the ray-cast mode, with the paper's view-space pixel
-// rays against the whole (unclipped) triangle.
-__global__ void __launch_bounds__(256) k_stage3(FrameDev f) {
+// Section 4.3: one block per tile part -- with edge functions, or, in the
+// ray-cast mode, with the paper's view-space pixel rays against the whole
+// (unclipped) triangle.  A block takes up to kGrab parts at once and sets them
+// up a thread each; parts whose sub-triangle covers no pixel of their tile
+// (half of them where a few huge triangles fill the screen) end there.  Of the
+// others a warp takes every eighth row and a lane every 32nd column, the edge
+// functions stepped from row to row; ranges narrower than 16 pixels are
+// walked end to end instead.
+namespace s3 {
+constexpr int kGrab = 4;
+}
+
+// Whether the sub-triangle covers a pixel of the range: each edge function
+// takes its largest value over the pixel centres at a corner (E_k falls with x
+// where dy_k > 0 and with y where dx_k < 0), and no pixel is covered when one
+// edge's largest value is outside.
+__device__ __forceinline__ bool range_touched(const SubTri &s, int x0, int x1, int y0, int y1) {
+    bool in = true;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const int a = (k + 1) % 3, b = (k + 2) % 3;
+        const int64_t dx = (int64_t)s.X[b] - s.X[a], dy = (int64_t)s.Y[b] - s.Y[a];
+        const int64_t px = 256 * (int64_t)(dy > 0 ? x0 : x1) + 128, py = 256 * (int64_t)(dx < 0 ? y0 : y1) + 128;
+        in &= dx * (py - s.Y[a]) - dy * (px - s.X[a]) >= (int64_t)((s.bias >> k) & 1u);
+    }
+    return in;
+}
+
+__global__ void __launch_bounds__(256) k_stage3(const __grid_constant__ FrameDev f) {
+    __shared__ SubTri part[s3::kGrab];               // x0 .. y1: the range inside the tile, x0 > x1: none
+    __shared__ uint32_t s_view[s3::kGrab], s_ray[s3::kGrab];   // s_ray: pair + 1 of a ray-cast part
     __shared__ unsigned long long s_i;
     const unsigned long long total = *((volatile unsigned long long *)&f.ctr->q2_count);
     const unsigned long long n = total < f.q2_cap ? total : f.q2_cap;
     const int ts = 1 << f.tile_log2;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t per = (uint32_t)max(1ull, min((unsigned long long)s3::kGrab, n / (2ull * gridDim.x)));
     for (;;) {
-        if (threadIdx.x == 0) s_i = atomicAdd(&f.ctr->q2_next, 1ull);
+        if (tid == 0) s_i = atomicAdd(&f.ctr->q2_next, (unsigned long long)per);
         __syncthreads();
-        const unsigned long long i = s_i;
-        __syncthreads();
-        if (i >= n) break;
-        const Q2Entry e = f.q2[i];
-        const ViewDev vw = f.views[e.view];
-        if (e.ray) {
-            RayTri R;
-            if (!ray_tri_of(f, e.pair, e.id, R)) continue;
-            const int x0 = max(e.X[0], (int)e.tx * ts), x1 = min(e.X[1], (int)e.tx * ts + ts - 1);
-            const int y0 = max(e.Y[0], (int)e.ty * ts), y1 = min(e.Y[1], (int)e.ty * ts + ts - 1);
-            if (x0 > x1 || y0 > y1) continue;
-            ray_range(R, x0, x1, y0, y1, threadIdx.x, blockDim.x, vw, e.id);
-            continue;
+        const unsigned long long i0 = s_i;
+        if (i0 >= n) break;
+        const int g = (int)min((unsigned long long)per, n - i0);
+        if (tid < g) {
+            const Q2Entry e = f.q2[i0 + tid];
+            const ViewDev &vw = f.views[e.view];
+            SubTri s;
+            s.id = e.id;
+            int x0, x1, y0, y1;
+            bool ok = true;
+            if (e.ray) {
+                x0 = e.X[0]; x1 = e.X[1]; y0 = e.Y[0]; y1 = e.Y[1];
+            } else {
+                for (int k = 0; k < 3; ++k) { s.X[k] = e.X[k]; s.Y[k] = e.Y[k]; s.iz[k] = e.iz[k]; }
+                ok = setup_subtri(s, vw.W, vw.H);
+                x0 = s.x0; x1 = s.x1; y0 = s.y0; y1 = s.y1;
+            }
+            s.x0 = max(x0, (int)e.tx * ts); s.x1 = min(x1, (int)e.tx * ts + ts - 1);
+            s.y0 = max(y0, (int)e.ty * ts); s.y1 = min(y1, (int)e.ty * ts + ts - 1);
+            if (ok && !e.ray) ok = s.x0 <= s.x1 && s.y0 <= s.y1 && range_touched(s, s.x0, s.x1, s.y0, s.y1);
+            if (!ok) s.x0 = 1, s.x1 = 0;
+            part[tid] = s;
+            s_view[tid] = e.view;
+            s_ray[tid] = e.ray ? e.pair + 1 : 0u;
         }
-        SubTri s;
-        for (int k = 0; k < 3; ++k) { s.X[k] = e.X[k]; s.Y[k] = e.Y[k]; s.iz[k] = e.iz[k]; }
-        s.id = e.id;
-        if (!setup_subtri(s, vw.W, vw.H)) continue;
-        const int x0 = max(s.x0, (int)e.tx * ts), x1 = min(s.x1, (int)e.tx * ts + ts - 1);
-        const int y0 = max(s.y0, (int)e.ty * ts), y1 = min(s.y1, (int)e.ty * ts + ts - 1);
-        if (x0 > x1 || y0 > y1) continue;
-        raster_range(s, x0, x1, y0, y1, threadIdx.x, blockDim.x, vw.vis, vw.W);
+        __syncthreads();
+        for (int p = 0; p < g; ++p) {
+            const SubTri &s = part[p];
+            const int x0 = s.x0, x1 = s.x1, y0 = s.y0, y1 = s.y1;
+            if (x0 > x1 || y0 > y1) continue;
+            const ViewDev &vw = f.views[s_view[p]];
+            if (s_ray[p]) {
+                RayTri R;
+                if (ray_tri_of(f, s_ray[p] - 1, s.id, R)) ray_range(R, x0, x1, y0, y1, tid, 256, vw, s.id);
+                continue;
+            }
+            const int W = vw.W;
+            uint64_t *vis = vw.vis;
+            if (x1 - x0 < 15) {
+                raster_range(s, x0, x1, y0, y1, tid, 256, vis, W);
+                continue;
+            }
+            const int64_t dx0 = (int64_t)s.X[2] - s.X[1], dy0 = (int64_t)s.Y[2] - s.Y[1];
+            const int64_t dx1 = (int64_t)s.X[0] - s.X[2], dy1 = (int64_t)s.Y[0] - s.Y[2];
+            const int64_t dx2 = (int64_t)s.X[1] - s.X[0], dy2 = (int64_t)s.Y[1] - s.Y[0];
+            const int64_t b0 = s.bias & 1u, b1 = (s.bias >> 1) & 1u, b2 = (s.bias >> 2) & 1u;
+            const float fA = nonneg_to_float(s.A);
+            const float iz[3] = {s.iz[0], s.iz[1], s.iz[2]};
+            const uint64_t id = s.id;
+            for (int x = x0 + lane; x <= x1; x += 32) {
+                const int64_t px = 256 * (int64_t)x + 128, py = 256 * (int64_t)(y0 + warp) + 128;
+                // less the bias, so that the sign alone decides
+                int64_t E0 = dx0 * (py - s.Y[1]) - dy0 * (px - s.X[1]) - b0;
+                int64_t E1 = dx1 * (py - s.Y[2]) - dy1 * (px - s.X[2]) - b1;
+                int64_t E2 = dx2 * (py - s.Y[0]) - dy2 * (px - s.X[0]) - b2;
+                uint64_t *at = vis + (size_t)(y0 + warp) * (size_t)W + (size_t)x;
+                for (int y = y0 + warp; y <= y1; y += 8, at += 8 * (size_t)W) {
+                    if ((E0 | E1 | E2) >= 0) depth_min(at, 0, frag_key(E0 + b0, E1 + b1, E2 + b2, fA, iz, id));
+                    E0 += 2048 * dx0; E1 += 2048 * dx1; E2 += 2048 * dx2;
+                }
+            }
+        }
+        __syncthreads();
     }
 }
 
@@ -622,9 +542,10 @@ __global__ void __launch_bounds__(256) k_stage3_tiles(FrameDev f) {
                 int64_t E2 = dx2 * (py - s.Y[0]) - dy2 * (px - s.X[0]);
                 const int64_t st = 256 * (int64_t)dyr;
                 const int64_t b0 = s.bias & 1u, b1 = (s.bias >> 1) & 1u, b2 = (s.bias >> 2) & 1u;
+                const float fA = nonneg_to_float(s.A);
                 for (; y <= ry1; y += dyr) {
                     if (((E0 - b0) | (E1 - b1) | (E2 - b2)) >= 0) {
-                        const uint64_t key = frag_key(E0, E1, E2, s.A, s.iz, s.id);
+                        const uint64_t key = frag_key(E0, E1, E2, fA, s.iz, s.id);
                         if (key < tw[(y << tl) + lx]) tw[(y << tl) + lx] = key;
                     }
                     E0 += dx0 * st; E1 += dx1 * st; E2 += dx2 * st;
@@ -639,7 +560,7 @@ __global__ void __launch_bounds__(256) k_stage3_tiles(FrameDev f) {
             for (; y <= uy1; y += dyr) {
                 const uint64_t key = tw[(y << tl) + lx];
                 if (key != kEmpty) {
-                    depth_test_write(vw.vis, (size_t)(by + y) * (size_t)vw.W + (size_t)(bx + lx), key);
+                    depth_min(vw.vis, (size_t)(by + y) * (size_t)vw.W + (size_t)(bx + lx), key);
                     tw[(y << tl) + lx] = kEmpty;
                 }
             }
@@ -726,11 +647,14 @@ cudaError_t query_launch_shape(LaunchShape *o, int device) {
         if (e != cudaSuccess) return e;
         o->stage1_blocks_per_sm[1][3] = o->stage1_blocks_per_sm[0][3];
     }
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o->stage1x_blocks_per_sm, k_stage1_exact<false>,
-                                                      32 * s1::kExactWarps, 0);
-
+    e = cudaFuncSetAttribute(k_stage1_exact<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)exact_smem_bytes());
     if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o->stage2_blocks_per_sm, k_stage2, 256, 0);
+    e = cudaFuncSetAttribute(k_stage1_exact<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)exact_smem_bytes());
+    if (e != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o->stage1x_blocks_per_sm, k_stage1_exact<false>,
+                                                      32 * s1::kExactWarps, exact_smem_bytes());
+    if (e != cudaSuccess) return e;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o->stage2_blocks_per_sm, k_stage2, 32 * s2::kWarps, 0);
     if (e != cudaSuccess) return e;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o->stage3_blocks_per_sm, k_stage3, 256, 0);
     if (e != cudaSuccess) return e;
@@ -775,13 +699,13 @@ cudaError_t launch_stage1(const FrameDev &f, bool instanced, int variant, uint32
 }
 
 cudaError_t launch_stage1_exact(const FrameDev &f, uint32_t r, int blocks, cudaStream_t s) {
-    if (f.s3_ray) k_stage1_exact<true><<<blocks, 32 * s1::kExactWarps, 0, s>>>(f, r);
-    else k_stage1_exact<false><<<blocks, 32 * s1::kExactWarps, 0, s>>>(f, r);
+    if (f.s3_ray) k_stage1_exact<true><<<blocks, 32 * s1::kExactWarps, exact_smem_bytes(), s>>>(f, r);
+    else k_stage1_exact<false><<<blocks, 32 * s1::kExactWarps, exact_smem_bytes(), s>>>(f, r);
     return cudaGetLastError();
 }
 
 cudaError_t launch_stage2(const FrameDev &f, int blocks, cudaStream_t s) {
-    k_stage2<<<blocks, 256, 0, s>>>(f);
+    k_stage2<<<blocks, 32 * s2::kWarps, 0, s>>>(f);
     return cudaGetLastError();
 }
 

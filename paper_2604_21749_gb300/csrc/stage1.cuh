@@ -325,7 +325,7 @@ __device__ __forceinline__ void exact_compute(const FrameDev &f, uint2 e, bool l
         cls = classify(f, r, vw, x0, x1, y0, y1, A, st);
     }
     const uint64_t id = pr.base + t;
-    q1_append<RAY>(f, cls == kQueue, id, pidx, mesh, t);
+    q1_append<RAY>(f, cls == kQueue, (uint32_t)(max(x1 - x0 + 1, 0) * max(y1 - y0 + 1, 0)), id, pidx, mesh, t);
     if (cls == kSmall) {
         const int X[3] = {r[0].X, r[1].X, r[2].X}, Y[3] = {r[0].Y, r[1].Y, r[2].Y};
         const float iz[3] = {r[0].iz, r[1].iz, r[2].iz};

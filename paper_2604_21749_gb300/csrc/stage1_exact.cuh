@@ -15,8 +15,7 @@
 #pragma once
 
 namespace s1 {
-constexpr int kExactWarps = 4;
-constexpr int kExactBlocks = 5;                      // 96 registers a thread
+constexpr int kExactWarps = 20;                      // one block an SM, 96 registers a thread
 constexpr int kExactK = 3;                           // survivors a lane gathers together
 constexpr int kBatch = 32 * kExactK;
 constexpr uint32_t kUnits = 13;                      // units dealt out of one block of the bitmap
@@ -38,18 +37,46 @@ struct __align__(16) SmallTri {
 
 static_assert(sizeof(SmallTri) == 3 * sizeof(uint4), "a record is three 16-byte words");
 
-struct ExactWarp {
-    uint2 e[kBatch];           // (triangle, pair)
-    uint4 t[kBatch][3];        // the nine gathered floats, overwritten by the SmallTri at set-up
-    uint32_t npx[kBatch];      // pixels of the range (0: nothing to rasterize)
-    uint32_t list[kBatch];     // triangles with pixels: first pixel of the batch | slot << 20
+// Up to 32 K small triangles of one warp, K a lane, and the pixel loop's marks.
+template <int K>
+struct SmallBatch {
+    uint4 t[32 * K][3];        // the SmallTri of each slot
+    uint32_t npx[32 * K];      // pixels of its range (0: nothing to rasterize)
+    uint32_t list[32 * K];     // triangles with pixels: first pixel of the batch | slot << 20
     uint32_t starts[kSegPx / 32];   // bit i: pixel i of the segment is a triangle's first
+};
+
+struct ExactWarp : SmallBatch<kExactK> {             // (t first holds the nine gathered floats)
+    uint2 e[kBatch];           // (triangle, pair)
 };
 }  // namespace s1
 
 __device__ __forceinline__ uint32_t fastdiv(uint32_t n, uint32_t m, uint32_t sh) {   // (fastdiv_consts)
     const uint32_t t = __umulhi(n, m);
     return (t + ((n - t) >> 1)) >> sh;
+}
+
+// The record of a front-facing triangle with both extents below 2^14
+// subpixels and at most 1024 pixels, w of them a row, from (x0, y0) on.
+__device__ __forceinline__ void put_small(uint4 (&t)[3], const int (&X)[3], const int (&Y)[3], const float (&iz)[3],
+                                          uint64_t id, uint32_t view, int x0, int y0, uint32_t w) {
+    // m = ceil(2^20 / w): the approximate quotient is off by less than 1/w, so its floor is the true one or,
+    // where w divides 2^20, perhaps one less
+    uint32_t m = (uint32_t)(1048576.0f * rcp_approx((float)w));
+    m += m * w < (1u << 20) ? 1u : 0u;
+    // edge k runs from vertex k+1 to vertex k+2; (px, py) is the first pixel's centre
+    const int px = 256 * x0 + 128, py = 256 * y0 + 128;
+    const int dx0 = X[2] - X[1], dy0 = Y[2] - Y[1], dx1 = X[0] - X[2], dy1 = Y[0] - Y[2], dx2 = X[1] - X[0], dy2 = Y[1] - Y[0];
+    const int e0 = dx0 * (py - Y[1]) - dy0 * (px - X[1]), e1 = dx1 * (py - Y[2]) - dy1 * (px - X[2]);
+    const uint32_t b0 = (dy0 < 0 || (dy0 == 0 && dx0 < 0)) ? 0u : 16u;
+    const uint32_t b1 = (dy1 < 0 || (dy1 == 0 && dx1 < 0)) ? 0u : 32u;
+    const uint32_t b2 = (dy2 < 0 || (dy2 == 0 && dx2 < 0)) ? 0u : 64u;
+    t[0] = make_uint4((uint32_t)e0, (uint32_t)e1, (uint32_t)(dx1 * dy2 - dx2 * dy1),
+                      ((uint32_t)dx0 & 0xFFFFu) | (uint32_t)dy0 << 16);
+    t[1] = make_uint4(((uint32_t)dx1 & 0xFFFFu) | (uint32_t)dy1 << 16, __float_as_uint(iz[0]), __float_as_uint(iz[1]),
+                      __float_as_uint(iz[2]));
+    t[2] = make_uint4((uint32_t)id, (uint32_t)(id >> 32) | b0 | b1 | b2 | view << 8, (uint32_t)x0 | (uint32_t)y0 << 16,
+                      w | m << 11);
 }
 
 // Set-up of the survivor in `slot`: its class, and for a small triangle its
@@ -66,7 +93,7 @@ __device__ __forceinline__ uint32_t fastdiv(uint32_t n, uint32_t m, uint32_t sh)
 //     power of two is exact).
 template <bool RAY>
 __device__ __forceinline__ void exact_setup(const FrameDev &f, s1::ExactWarp &S, int slot, bool live) {
-    uint32_t npx = 0;
+    uint32_t npx = 0, px = 0;                        // px: pixels of a triangle for stage 2
     bool queue = false;
     uint64_t id = 0;
     uint2 e = make_uint2(0u, 0u);
@@ -126,31 +153,17 @@ __device__ __forceinline__ void exact_setup(const FrameDev &f, s1::ExactWarp &S,
             } else {
                 const uint32_t w = (uint32_t)(x1 - x0 + 1), n = w * (uint32_t)(y1 - y0 + 1);
                 queue = big || n > f.s1_max;
-                if (!queue) {
+                if (queue) {
+                    px = n;
+                } else {
                     npx = n;
-                    // m = ceil(2^20 / w): the approximate quotient is off by less than 1/w, so its
-                    // floor is the true one or, where w divides 2^20, perhaps one less
-                    uint32_t m = (uint32_t)(1048576.0f * rcp_approx((float)w));
-                    m += m * w < (1u << 20) ? 1u : 0u;
-                    // edge k runs from vertex k+1 to vertex k+2; (px, py) is the first pixel's centre
-                    const int px = 256 * x0 + 128, py = 256 * y0 + 128;
-                    const int dx0 = X[2] - X[1], dy0 = Y[2] - Y[1], dx1 = -wx, dy1 = -wy;
-                    const int e0 = dx0 * (py - Y[1]) - dy0 * (px - X[1]), e1 = dx1 * (py - Y[2]) - dy1 * (px - X[2]);
-                    const uint32_t b0 = (dy0 < 0 || (dy0 == 0 && dx0 < 0)) ? 0u : 16u;
-                    const uint32_t b1 = (dy1 < 0 || (dy1 == 0 && dx1 < 0)) ? 0u : 32u;
-                    const uint32_t b2 = (uy < 0 || (uy == 0 && ux < 0)) ? 0u : 64u;
-                    S.t[slot][0] = make_uint4((uint32_t)e0, (uint32_t)e1, (uint32_t)(ux * wy - wx * uy),
-                                              ((uint32_t)dx0 & 0xFFFFu) | (uint32_t)dy0 << 16);
-                    S.t[slot][1] = make_uint4(((uint32_t)dx1 & 0xFFFFu) | (uint32_t)dy1 << 16, __float_as_uint(iz[0]),
-                                              __float_as_uint(iz[1]), __float_as_uint(iz[2]));
-                    S.t[slot][2] = make_uint4((uint32_t)id, (uint32_t)(id >> 32) | b0 | b1 | b2 | pr.view << 8,
-                                              (uint32_t)x0 | (uint32_t)y0 << 16, w | m << 11);
+                    put_small(S.t[slot], X, Y, iz, id, pr.view, x0, y0, w);
                 }
             }
         }
     }
     S.npx[slot] = npx;
-    q1_append<RAY>(f, queue, id, e.y, mesh, e.x);
+    q1_append<RAY>(f, queue, px, id, e.y, mesh, e.x);
     if (f.stats && live) {
         stat_add(f, kStatIn, 1);
         if (st != kStatCount) stat_add(f, st, 1);
@@ -158,49 +171,23 @@ __device__ __forceinline__ void exact_setup(const FrameDev &f, s1::ExactWarp &S,
     }
 }
 
-// Rasterizes the small triangles of a batch: slot s holds npx[s]
-// pixels.  The ranges are laid end to end in the order (lane, u); the
-// triangle of pixel i is the last one to start at or before i, found by
-// counting the marked starts up to it.  The range is walked row by row: pixel
-// k of a range of width w is (k mod w, k / w), the division as a multiplication
-// by m = ceil(2^20 / w), exact for k, w <= 1024 (k (m w - 2^20) < 2^20).  The
-// edge functions are int32: both extents are below 2^14 subpixels, so
-// |E| < 2^30 at every visited sample, and E2 = A - E0 - E1 exactly.
-__device__ __forceinline__ void exact_raster(const FrameDev &f, s1::ExactWarp &S, int lane) {
+// The pixels p0 .. p1 - 1 of a batch, 32 a step.  own / at0: the scan of
+// small_raster; first: triangles that start before p0, less one.
+template <int K>
+__device__ __forceinline__ void small_span(const FrameDev &f, s1::SmallBatch<K> &S, const uint32_t (&npx)[K], uint32_t at0,
+                                           uint32_t p0, uint32_t p1, int first, int lane) {
     using namespace s1;
-    uint32_t npx[kExactK], own = 0;                  // own: pixels | triangles << 20
-#pragma unroll
-    for (int u = 0; u < kExactK; ++u) npx[u] = S.npx[lane + 32 * u];
-#pragma unroll
-    for (int u = 0; u < kExactK; ++u) own += npx[u] ? npx[u] + (1u << 20) : 0u;
-    uint32_t incl = own;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += v;
-    }
-    const uint32_t P = __shfl_sync(0xffffffffu, incl, 31) & 0xFFFFFu;
-    if (P == 0) return;
-    const uint32_t at0 = incl - own;
-    uint32_t at = at0;
-#pragma unroll
-    for (int u = 0; u < kExactK; ++u)
-        if (npx[u]) {
-            S.list[at >> 20] = (at & 0xFFFFFu) | (uint32_t)(lane + 32 * u) << 20;
-            at += npx[u] + (1u << 20);
-        }
     const uint32_t upto = 0xffffffffu >> (31 - lane);
-    int first = -1;                                  // triangles that start before the window, less one
-    for (uint32_t sb = 0; sb < P; sb += kSegPx) {
-        const uint32_t nwin = (min(P - sb, kSegPx) + 31) / 32;
+    for (uint32_t sb = p0; sb < p1; sb += kSegPx) {
+        const uint32_t nwin = (min(p1 - sb, kSegPx) + 31) / 32;
         for (uint32_t w = lane; w < nwin; w += 32) S.starts[w] = 0;
         __syncwarp();
-        at = at0;
+        uint32_t at = at0;
 #pragma unroll
-        for (int u = 0; u < kExactK; ++u)
+        for (int u = 0; u < K; ++u)
             if (npx[u]) {
                 const uint32_t i = (at & 0xFFFFFu) - sb;
-                if (i < kSegPx) atomicOr(&S.starts[i >> 5], 1u << (i & 31));
+                if (i < 32 * nwin) atomicOr(&S.starts[i >> 5], 1u << (i & 31));
                 at += npx[u] + (1u << 20);
             }
         __syncwarp();
@@ -208,7 +195,7 @@ __device__ __forceinline__ void exact_raster(const FrameDev &f, s1::ExactWarp &S
             const uint32_t word = S.starts[w], i = sb + 32 * w + lane;
             const int o = first + __popc(word & upto);
             first += __popc(word);
-            if (i >= P) continue;
+            if (i >= p1) continue;
             const uint32_t L = S.list[o], k = i - (L & 0xFFFFFu);
             const uint4 *t = S.t[L >> 20];
             const uint4 ta = t[0], tb = t[1], tc = t[2];
@@ -231,24 +218,93 @@ __device__ __forceinline__ void exact_raster(const FrameDev &f, s1::ExactWarp &S
     }
 }
 
-// The exact kernel, round r.  Warps take the bitmap in units from a counter:
-// survivors come in clusters where the view looks closely, and a fixed deal of
-// 32-word chunks left some SMs with twice the average (the ordinary full-HD
-// view of a 4.2 M-triangle mesh: 179 us, 117 us now).  A unit is four words
-// (128 triangles of one pair, a 16-byte load) for each of 2^ll lanes, in runs
-// of eight words kUnits runs apart, so that a cluster spreads over several
-// units.  2^ll is the largest of 1 .. 32 that gives every warp twelve units:
-// one address takes an atomic add every 1.8 ns, which 32-word units would
-// make the bound of the billion-triangle frame (1.75 ms against 0.93).  Frames
-// too small for any of that deal single words, so that all warps work.  The
-// next grab and the words of the next unit are in flight while a batch runs.
+// Rasterizes the small triangles of a batch: slot s holds npx[s] pixels.  The
+// ranges are laid end to end in the order (lane, u); the
+// triangle of pixel i is the last one to start at or before i, found by
+// counting the marked starts up to it.  The range is walked row by row: pixel
+// k of a range of width w is (k mod w, k / w), the division as a multiplication
+// by m = ceil(2^20 / w), exact for k, w <= 1024 (k (m w - 2^20) < 2^20).  The
+// edge functions are int32: both extents are below 2^14 subpixels, so
+// |E| < 2^30 at every visited sample, and E2 = A - E0 - E1 exactly.
+// give(want, slot): where the batch holds more than 2 kSegPx pixels, hands
+// over the triangles that start past pixel kSegPx, the lanes' `want`ed ones in
+// lane order, and returns false to those it has no room for (the last ones);
+// nullptr keeps them all.
+template <int K, class Give>
+__device__ __forceinline__ void small_raster(const FrameDev &f, s1::SmallBatch<K> &S, int lane, Give give) {
+    using namespace s1;
+    uint32_t npx[K], own = 0;                        // own: pixels | triangles << 20
+#pragma unroll
+    for (int u = 0; u < K; ++u) npx[u] = S.npx[lane + 32 * u];
+#pragma unroll
+    for (int u = 0; u < K; ++u) own += npx[u] ? npx[u] + (1u << 20) : 0u;
+    uint32_t incl = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += v;
+    }
+    const uint32_t all = __shfl_sync(0xffffffffu, incl, 31), P = all & 0xFFFFFu;
+    if (P == 0) return;
+    const uint32_t at0 = incl - own;
+    uint32_t at = at0;
+#pragma unroll
+    for (int u = 0; u < K; ++u)
+        if (npx[u]) {
+            S.list[at >> 20] = (at & 0xFFFFFu) | (uint32_t)(lane + 32 * u) << 20;
+            at += npx[u] + (1u << 20);
+        }
+    uint32_t pa = P, pb = P;                         // pixels pa .. pb - 1 are handed over
+    int fb = 0;
+    if constexpr (!std::is_same<Give, std::nullptr_t>::value) {
+        if (P > 2 * kSegPx) {
+            __syncwarp();
+            const int nt = (int)(all >> 20);
+            int g0 = 0;                              // the first triangle to start at or past kSegPx
+            for (int b = 0; b < nt; b += 32)
+                g0 += __popc(__ballot_sync(0xffffffffu, b + lane < nt && (S.list[min(b + lane, nt - 1)] & 0xFFFFFu) < kSegPx));
+            int kept = nt;                           // triangles from here on found no room
+            for (int b = g0; b < nt && kept == nt; b += 32) {
+                const bool want = b + lane < nt;
+                const bool ok = give(want, (int)(S.list[want ? b + lane : nt - 1] >> 20));
+                const unsigned bad = __ballot_sync(0xffffffffu, want && !ok);
+                if (bad) kept = b + __ffs(bad) - 1;
+            }
+            if (g0 < nt) pa = S.list[g0] & 0xFFFFFu;
+            if (kept < nt) pb = S.list[kept] & 0xFFFFFu;
+            fb = kept - 1;
+        }
+    }
+    small_span(f, S, npx, at0, 0u, pa, -1, lane);
+    if (pb < P) small_span(f, S, npx, at0, pb, P, fb, lane);
+}
+
+size_t exact_smem_bytes() { return sizeof(s1::ExactWarp) * s1::kExactWarps; }
+
+// The exact kernel, round r, one block of 20 warps an SM.  Warps take the
+// bitmap in units: survivors come in clusters where the view looks closely,
+// and a fixed deal of 32-word chunks to warps left some SMs with twice the
+// average (the full-HD view of a 4.2 M-triangle mesh: 179 us, 106 us now).
+// The SM's share of the first 7/8 of the units is taken from a counter in
+// shared memory, the rest from one in global memory, which evens the SMs out:
+// one global address takes an atomic add every 1.8 ns, too slow for every unit
+// (4-word units of that mesh: 59 of 117 us; 32-word units of the billion-
+// triangle frame: 1.75 ms against 0.91).  A unit is four words (128 triangles
+// of one pair, a 16-byte load) for each of 2^ll lanes, in runs of eight words
+// kUnits runs apart, so that a cluster spreads over several units; 2^ll is the
+// largest of 1 .. 32 that gives every warp twelve units.  Frames too small for
+// any of that deal single words, so that all warps work.  The words of the
+// next unit are in flight while a batch runs.
 template <bool RAY>
-__global__ void __launch_bounds__(32 * s1::kExactWarps, s1::kExactBlocks)
+__global__ void __launch_bounds__(32 * s1::kExactWarps, 1)
     k_stage1_exact(const __grid_constant__ FrameDev f, uint32_t r) {
     using namespace s1;
-    __shared__ ExactWarp sw[kExactWarps];
+    extern __shared__ __align__(128) unsigned char exact_smem[];
+    __shared__ uint32_t s_taken;                    // units the SM has taken of its share
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    ExactWarp &S = sw[warp];
+    ExactWarp &S = reinterpret_cast<ExactWarp *>(exact_smem)[warp];
+    if (threadIdx.x == 0) s_taken = 0;
+    __syncthreads();
     const RoundDev rd = f.rounds[r];
     const uint64_t nwords = rd.w1 - rd.w0;
     const int n_segs = (int)f.hdr->n_segs;
@@ -263,15 +319,20 @@ __global__ void __launch_bounds__(32 * s1::kExactWarps, s1::kExactBlocks)
     const uint32_t per_block = ll ? kUnits : 1u;
     const uint32_t nunits = (uint32_t)((nwords + block - 1) / block) * per_block;   // (at most 2^34 words)
     const uint64_t lane0 = lane >= 1 << ll ? nwords : ll ? (uint64_t)(lane >> 1) * 8 * kUnits + 4 * (lane & 1) : 0;
-    uint32_t next = 0;                              // lane 0: the unit after the one being fetched
-    if (lane == 0) next = atomicAdd(&f.ctr->xwork[r], 1u);
+    // the SM's share of the first 7/8 of the units, then whatever is left of the rest
+    const uint32_t shared_out = nunits - nunits / 8;
+    auto grab = [&]() -> uint32_t {
+        const uint32_t u = blockIdx.x + atomicAdd(&s_taken, 1u) * gridDim.x;
+        return u < shared_out ? u : shared_out + atomicAdd(&f.ctr->xwork[r], 1u);
+    };
+    uint32_t next = lane == 0 ? grab() : 0u;        // lane 0: the unit after the one being fetched
     uint64_t word = 0;                              // the lane's first word of the unit
     bool more = true;
     // moves to the next unit and issues its load
     auto fetch = [&]() -> uint4 {
         const uint32_t unit = __shfl_sync(0xffffffffu, next, 0);
         more = unit < nunits;
-        if (lane == 0 && more) next = atomicAdd(&f.ctr->xwork[r], 1u);
+        if (lane == 0 && more) next = grab();
         const uint32_t b = ll ? unit / kUnits : unit;
         word = lane0 + (uint64_t)b * block + (ll ? 8 * (unit - b * kUnits) : 0u);
         uint4 w = make_uint4(0u, 0u, 0u, 0u);
@@ -374,7 +435,21 @@ __global__ void __launch_bounds__(32 * s1::kExactWarps, s1::kExactBlocks)
         for (int u = 0; u < kExactK; ++u)           // (a lane reads and writes its own slots only)
             exact_setup<RAY>(f, S, lane + 32 * u, lane + 32 * u < n);
         __syncwarp();
-        exact_raster(f, S, lane);
+        // a batch of heavy triangles (a near surface, up to 128 pixels each) would keep its warp long after
+        // the others: what starts past kSegPx pixels goes to stage 2, which deals triangles out finely (a
+        // close 4K view of a 100 M-triangle scan: exact kernel and stage 2 521 + 67 us, 453 + 41 us with it)
+        small_raster<kExactK>(f, S, lane, [&](bool want, int slot) -> bool {
+            unsigned long long base = 0;
+            const unsigned all = __ballot_sync(0xffffffffu, want);
+            if (lane == 0) base = atomicAdd(&f.ctr->q1_count, (unsigned long long)__popc(all));
+            const uint32_t px = __reduce_add_sync(0xffffffffu, want ? S.npx[slot] : 0u);
+            if (lane == 0) atomicAdd(&f.ctr->q1_px, (unsigned long long)px);
+            base = __shfl_sync(0xffffffffu, base, 0) + __popc(all & lt_mask);
+            if (!want || base >= f.q1_cap) return false;
+            const uint2 e = S.e[slot];
+            f.q1[base] = Q1Entry{f.pairs[e.y].base + e.x, e.y, 1u};
+            return true;
+        });
         __syncwarp();
     }
 }

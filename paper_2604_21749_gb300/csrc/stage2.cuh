@@ -1,0 +1,219 @@
+// stage2.cuh -- stage 2 (Section 4.2), included by raster.cu.
+//
+// A warp takes up to 32 queued triangles at a time.  Each lane sets one up:
+// transform, clip (Sutherland-Hodgman, near plane and guard band) where it
+// reaches beyond a plane, snap, visible pixel range.  Most of the clipped
+// ones end there with no pixel on the screen; whole triangles of at most
+// 1024 pixels go through the small triangles' pixel loop together; the warp
+// works through the rest one by one, rasterizing sub-triangles of at most
+// s2_max pixels itself and splitting larger ones along tile boundaries into
+// stage-3 parts.
+#pragma once
+
+namespace s2 {
+constexpr int kWarps = 4;
+constexpr unsigned long long kGrabPx = 2048;
+}
+
+// The tiles of [x0, x1] x [y0, y1] as stage-3 parts, with one reservation of
+// queue 2.  RAY: the whole triangle is ray cast, s holds its id alone.  Parts
+// past the queue's capacity are rasterized in place.  Returns their number.
+template <bool RAY>
+__device__ __forceinline__ uint32_t append_parts(const FrameDev &f, const SubTri &s, uint32_t pidx, uint32_t view,
+                                                 const ViewDev &vw, int x0, int x1, int y0, int y1, int lane) {
+    const int tl = (int)f.tile_log2, ts = 1 << tl;
+    const int tx0 = x0 >> tl, ty0 = y0 >> tl, ntx = (x1 >> tl) - tx0 + 1;
+    const int nt = ntx * ((y1 >> tl) - ty0 + 1);
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(&f.ctr->q2_count, (unsigned long long)nt);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    // the entry but for its tile, as the four 16-byte words it is stored in
+    static_assert(sizeof(Q2Entry) == 64, "a part is four 16-byte words");
+    uint4 w0, w1, w2;
+    if (RAY) {
+        w0 = make_uint4((uint32_t)x0, (uint32_t)x1, 0u, (uint32_t)y0);
+        w1 = make_uint4((uint32_t)y1, 0u, 0u, 0u);
+        w2 = make_uint4(0u, view, (uint32_t)s.id, (uint32_t)(s.id >> 32));
+    } else {
+        w0 = make_uint4((uint32_t)s.X[0], (uint32_t)s.X[1], (uint32_t)s.X[2], (uint32_t)s.Y[0]);
+        w1 = make_uint4((uint32_t)s.Y[1], (uint32_t)s.Y[2], __float_as_uint(s.iz[0]), __float_as_uint(s.iz[1]));
+        w2 = make_uint4(__float_as_uint(s.iz[2]), view, (uint32_t)s.id, (uint32_t)(s.id >> 32));
+    }
+    int tx = lane % ntx, ty = ty0 + lane / ntx;      // stepped by 32 tiles: sy rows and sx columns
+    const int sx = 32 % ntx, sy = 32 / ntx;
+    for (int k = lane; k < nt; k += 32) {
+        const uint32_t ex = (uint32_t)(tx0 + tx), ey = (uint32_t)ty;
+        tx += sx;
+        ty += sy;
+        if (tx >= ntx) tx -= ntx, ++ty;
+        if (base + k < f.q2_cap) {
+            uint4 *e = reinterpret_cast<uint4 *>(f.q2 + base + k);
+            e[0] = w0; e[1] = w1; e[2] = w2;
+            e[3] = make_uint4(ex, ey, RAY ? pidx : 0u, RAY ? 1u : 0u);
+            if (f.s3_bin) atomicAdd(&f.tile_cnt[vw.tile0 + ey * vw.ntx + ex], 1u);
+        } else {
+            atomicAdd(&f.ctr->overflow2, 1ull);
+            const int rx0 = max(x0, (int)ex * ts), rx1 = min(x1, (int)ex * ts + ts - 1);
+            const int ry0 = max(y0, (int)ey * ts), ry1 = min(y1, (int)ey * ts + ts - 1);
+            if (RAY) {
+                RayTri R;
+                if (ray_tri_of(f, pidx, s.id, R)) ray_range(R, rx0, rx1, ry0, ry1, 0, 1, vw, s.id);
+            } else {
+                raster_range(s, rx0, rx1, ry0, ry1, 0, 1, vw.vis, vw.W);
+            }
+        }
+    }
+    return (uint32_t)nt;
+}
+
+// One sub-triangle by the whole warp.
+__device__ __forceinline__ void stage2_subtri(const FrameDev &f, SubTri &s, uint32_t view, const ViewDev &vw, int lane,
+                                              unsigned long long &n_s2, unsigned long long &n_parts) {
+    if (!setup_subtri(s, vw.W, vw.H)) return;
+    const int64_t cnt = (int64_t)(s.x1 - s.x0 + 1) * (int64_t)(s.y1 - s.y0 + 1);
+    if (cnt <= (int64_t)f.s2_max) {
+        raster_range(s, s.x0, s.x1, s.y0, s.y1, lane, 32, vw.vis, vw.W);
+        ++n_s2;
+    } else {
+        n_parts += append_parts<false>(f, s, 0u, view, vw, s.x0, s.x1, s.y0, s.y1, lane);
+    }
+}
+
+// One queued triangle that reaches beyond a plane, by the whole warp.
+__device__ __noinline__ void stage2_clipped(const FrameDev *fp, const Q1Entry *ep, unsigned long long *n_s2,
+                                            unsigned long long *n_parts) {
+    const FrameDev &f = *fp;
+    const int lane = threadIdx.x & 31;
+    const Q1Entry e = *ep;
+    const PairDev &pr = f.pairs[e.pair];
+    const ViewDev vw = f.views[pr.view];
+    CV c[3];
+    load_clip(f, f.meshes[pr.mesh], e.pair, e.id - pr.base, vw, c);
+    CV poly[kMaxPoly];
+    const int np = clip_polygon(c, vw.nearv, poly);
+    if (np < 3) return;
+    int X[kMaxPoly], Y[kMaxPoly];
+    float iz[kMaxPoly];
+    for (int k = 0; k < np; ++k) snap(poly[k], vw.hw, vw.hh, X[k], Y[k], iz[k]);
+    SubTri s;
+    s.id = e.id;
+    if (f.s3_ray) {
+        // the paper's stage 3: a triangle whose visible bbox holds more
+        // than s2_max pixel centres is ray cast over that range, in tiles
+        int x0, x1, y0, y1;
+        const int64_t cnt = poly_range(X, Y, np, vw.W, vw.H, x0, x1, y0, y1);
+        if (cnt == 0) return;
+        if (cnt > (int64_t)f.s2_max) {
+            *n_parts += append_parts<true>(f, s, e.pair, pr.view, vw, x0, x1, y0, y1, lane);
+            return;
+        }
+    }
+    unsigned long long a = 0, b = 0;
+    for (int j = 1; j + 1 < np; ++j) {
+        s.X[0] = X[0]; s.X[1] = X[j]; s.X[2] = X[j + 1];
+        s.Y[0] = Y[0]; s.Y[1] = Y[j]; s.Y[2] = Y[j + 1];
+        s.iz[0] = iz[0]; s.iz[1] = iz[j]; s.iz[2] = iz[j + 1];
+        stage2_subtri(f, s, pr.view, vw, lane, a, b);
+    }
+    *n_s2 += a;
+    *n_parts += b;
+}
+
+// Whether a triangle beyond some plane covers anything: false when its
+// clipped polygon holds no pixel centre of the screen.
+__device__ __noinline__ bool clipped_visible(const CV *c, const ViewDev *vw) {
+    CV poly[kMaxPoly];
+    const int np = clip_polygon(c, vw->nearv, poly);
+    if (np < 3) return false;
+    int X[kMaxPoly], Y[kMaxPoly];
+    float iz;
+    for (int k = 0; k < np; ++k) snap(poly[k], vw->hw, vw->hh, X[k], Y[k], iz);
+    int x0, x1, y0, y1;
+    return poly_range(X, Y, np, vw->W, vw->H, x0, x1, y0, y1) > 0;
+}
+
+// per: triangles a warp takes at once.  Big triangles are dealt out finely,
+// kGrabPx pixels a grab by the queue's average, or the last warps to get some
+// would work long after the others; a short queue is dealt out singly, so that
+// all warps share it.  (A 100 M-triangle view whose queue is half clipped
+// triangles without a pixel and half small ones handed over: 67 us singly,
+// 35 us in sevens.)
+__global__ void __launch_bounds__(32 * s2::kWarps) k_stage2(const __grid_constant__ FrameDev f) {
+    using namespace s2;
+    __shared__ s1::SmallBatch<1> sw[kWarps];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    s1::SmallBatch<1> &S = sw[warp];
+    const unsigned long long total = *((volatile unsigned long long *)&f.ctr->q1_count);
+    const unsigned long long n = total < f.q1_cap ? total : f.q1_cap;
+    const unsigned long long nw = (unsigned long long)gridDim.x * kWarps;
+    const unsigned long long fair = max(n / (2 * nw), n < nw ? 1ull : 4ull);
+    const unsigned long long light = kGrabPx * total / (*((volatile unsigned long long *)&f.ctr->q1_px) + 1);
+    const uint32_t per = (uint32_t)max(1ull, min(32ull, min(fair, light)));
+    unsigned long long n_s2 = 0, n_parts = 0;
+    for (;;) {
+        unsigned long long i0 = 0;
+        if (lane == 0) i0 = atomicAdd(&f.ctr->q1_next, (unsigned long long)per);
+        i0 = __shfl_sync(0xffffffffu, i0, 0);
+        if (i0 >= n) break;
+        const uint32_t g = (uint32_t)min((unsigned long long)per, n - i0);
+        uint32_t npx = 0, view = 0;
+        bool whole = false, clip = false;             // for the warp: unclipped, clipped
+        int X[3] = {0, 0, 0}, Y[3] = {0, 0, 0};
+        float iz[3] = {0.0f, 0.0f, 0.0f};
+        Q1Entry e{0, 0, 0};
+        if (lane < g) {
+            e = f.q1[i0 + lane];
+            const PairDev &pr = f.pairs[e.pair];
+            view = pr.view;
+            const ViewDev &vw = f.views[view];
+            CV c[3];
+            load_clip(f, f.meshes[pr.mesh], e.pair, e.id - pr.base, vw, c);
+            if ((outcode(c[0], vw.nearv) | outcode(c[1], vw.nearv) | outcode(c[2], vw.nearv)) == 0) {
+                // inside every plane: Sutherland-Hodgman would return it unchanged
+#pragma unroll
+                for (int k = 0; k < 3; ++k) snap(c[k], vw.hw, vw.hh, X[k], Y[k], iz[k]);
+                int x0, x1, y0, y1;
+                const int64_t cnt = poly_range(X, Y, 3, vw.W, vw.H, x0, x1, y0, y1);
+                const int ex = max(X[0], max(X[1], X[2])) - min(X[0], min(X[1], X[2]));
+                const int ey = max(Y[0], max(Y[1], Y[2])) - min(Y[0], min(Y[1], Y[2]));
+                if (cnt > 1024 || max(ex, ey) >= (1 << 14) || (!e.small && cnt > (int64_t)f.s2_max)) {
+                    whole = true;
+                } else if (cnt > 0 && (X[1] - X[0]) * (Y[2] - Y[0]) - (X[2] - X[0]) * (Y[1] - Y[0]) > 0) {
+                    npx = (uint32_t)cnt;
+                    put_small(S.t[lane], X, Y, iz, e.id, view, x0, y0, (uint32_t)(x1 - x0 + 1));
+                }
+            } else {
+                clip = per == 1 || clipped_visible(c, &vw);
+            }
+        }
+        S.npx[lane] = npx;
+        __syncwarp();
+        small_raster<1>(f, S, lane, nullptr);
+        n_s2 += __popc(__ballot_sync(0xffffffffu, npx != 0));
+        for (unsigned m = __ballot_sync(0xffffffffu, whole); m; m &= m - 1) {
+            const int l = __ffs(m) - 1;
+            SubTri s;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+                s.X[k] = __shfl_sync(0xffffffffu, X[k], l);
+                s.Y[k] = __shfl_sync(0xffffffffu, Y[k], l);
+                s.iz[k] = __shfl_sync(0xffffffffu, iz[k], l);
+            }
+            s.id = __shfl_sync(0xffffffffu, e.id, l);
+            const uint32_t v = __shfl_sync(0xffffffffu, view, l), pair = __shfl_sync(0xffffffffu, e.pair, l);
+            const ViewDev &vw = f.views[v];
+            int x0, x1, y0, y1;
+            if (f.s3_ray && poly_range(s.X, s.Y, 3, vw.W, vw.H, x0, x1, y0, y1) > (int64_t)f.s2_max)
+                n_parts += append_parts<true>(f, s, pair, v, vw, x0, x1, y0, y1, lane);
+            else
+                stage2_subtri(f, s, v, vw, lane, n_s2, n_parts);
+        }
+        for (unsigned m = __ballot_sync(0xffffffffu, clip); m; m &= m - 1)
+            stage2_clipped(&f, f.q1 + i0 + (__ffs(m) - 1), &n_s2, &n_parts);
+        __syncwarp();
+    }
+    if (f.stats && lane == 0) {
+        stat_add(f, kStatS2, n_s2);
+        stat_add(f, kStatParts, n_parts);
+    }
+}

@@ -1,5 +1,6 @@
 """The exact kernel of stage 1 at the edges of its pixel loop and of its deal
-of the survivor bitmap, against the oracle (bit-exact words)."""
+of the survivor bitmap, and stages 2 and 3 behind it, against the oracle
+(bit-exact words)."""
 import numpy as np
 import pytest
 import torch
@@ -20,11 +21,13 @@ def api():
     return A
 
 
-def _slivers(n, W, H, seed):
+SHAPES = [(1, 1), (2, 1), (1, 3), (31, 1), (32, 1), (33, 2), (8, 16), (32, 32), (1024, 1), (1, 1024), (341, 3), (64, 16)]
+
+
+def _slivers(n, W, H, seed, shapes=SHAPES):
     """Triangles in the plane z = -1 of a camera at the origin whose pixel boxes
     are 1 x 1 .. 1024 x 1, 1 x 1024 and 32 x 32 pixels, some across the border."""
     rng = np.random.default_rng(seed)
-    shapes = [(1, 1), (2, 1), (1, 3), (31, 1), (32, 1), (33, 2), (8, 16), (32, 32), (1024, 1), (1, 1024), (341, 3), (64, 16)]
     pos = []
     for k in range(n):
         w, h = shapes[k % len(shapes)]
@@ -68,4 +71,52 @@ def test_bitmap_deal(api, n):
     vis = r.render(cam.view, cam.proj, W, H)
     r.sync()
     assert_vis_equal(vis, oracle_vis(scene, cam), f"{n} x {n} cells")
+    del keep
+
+
+@pytest.mark.parametrize("capacity", [1, 50, 1 << 20])
+def test_heavy_batches_are_handed_over(api, capacity):
+    """Batches of up to 96 x 1024 pixels: what stage 1 hands to stage 2, and what
+    queue 1 has no room for, lands in the buffer all the same."""
+    scene = _slivers(700, 1100, 1060, seed=5, shapes=[(32, 32), (31, 33), (1024, 1), (40, 25)])
+    cam = scene.cameras[0]
+    r = api.Renderer(0)
+    r.set_config(stage1_max_pixels=1024, stage1_exact_all=1, queue1_capacity=capacity)
+    keep = upload(r, scene, with_colour=False)
+    vis = r.render(cam.view, cam.proj, cam.W, cam.H)
+    st = r.sync()
+    assert st["queued_stage2"] > 0
+    assert_vis_equal(vis, oracle_vis(scene, cam), f"queue 1 of {capacity}")
+    del keep
+
+
+@pytest.mark.parametrize("s2", [32, 1023, 1024, 4096, 1 << 20])
+@pytest.mark.parametrize("n", [1, 31, 700, 20000])
+def test_stage2_sizes(api, n, s2):
+    """Queues dealt out singly and in groups, ranges about the 1024 pixels of the
+    shared pixel loop and about the stage-2 limit, tiles with and without a
+    covered pixel."""
+    scene = _slivers(n, 1100, 1060, seed=100 + n, shapes=[(1, 1), (32, 32), (1025, 1), (33, 32), (300, 200), (15, 70),
+                                                          (900, 900) if n < 1000 else (64, 64)])
+    cam = scene.cameras[0]
+    r = api.Renderer(0)
+    r.set_config(stage1_max_pixels=1, stage2_max_pixels=s2, stage1_exact_all=1)
+    keep = upload(r, scene, with_colour=False)
+    vis = r.render(cam.view, cam.proj, cam.W, cam.H)
+    r.sync()
+    assert_vis_equal(vis, oracle_vis(scene, cam), f"{n} triangles, stage-2 limit {s2}")
+    del keep
+
+
+@pytest.mark.parametrize("size", [(3840, 2160), (1921, 1081), (8000, 37)])
+def test_room_large(api, size):
+    """Clipped triangles as wide as the screen: edge functions far beyond 32 bits."""
+    W, H = size
+    scene = S.scene_room()
+    cam = Camera(scene.cameras[0].view, S.perspective(80.0, W / H, 0.05, 100.0), W, H)
+    r = api.Renderer(0)
+    keep = upload(r, scene, with_colour=False)
+    vis = r.render(cam.view, cam.proj, W, H)
+    r.sync()
+    assert_vis_equal(vis, oracle_vis(scene, cam), f"room {W} x {H}")
     del keep
