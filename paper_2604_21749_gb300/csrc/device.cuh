@@ -446,11 +446,14 @@ __device__ __forceinline__ float dot3(float3 a, float3 b) {
 }
 
 // Pixel-centre ray through (x, y): (ndx / fx, ndy / fy, -1) with
-// ndx = (2x + 1) / W - 1 (camera at the origin of view space).
+// ndx = (2x + 1) / W - 1 (camera at the origin of view space); one of its
+// first two coordinates, and all three.
+__device__ __forceinline__ float ray_axis(int i, int n, float f) {
+    return __fdiv_rn(__fsub_rn(__fdiv_rn(__int2float_rn(2 * i + 1), __int2float_rn(n)), 1.0f), f);
+}
+
 __device__ __forceinline__ float3 pixel_ray(int x, int y, int W, int H, float fx, float fy) {
-    const float ndx = __fsub_rn(__fdiv_rn(__int2float_rn(2 * x + 1), __int2float_rn(W)), 1.0f);
-    const float ndy = __fsub_rn(__fdiv_rn(__int2float_rn(2 * y + 1), __int2float_rn(H)), 1.0f);
-    return make_float3(__fdiv_rn(ndx, fx), __fdiv_rn(ndy, fy), -1.0f);
+    return make_float3(ray_axis(x, W, fx), ray_axis(y, H, fy), -1.0f);
 }
 
 // Pixel centres 256 i + 128 inside the snapped range [mn, mx] (1/256 px) of
@@ -478,8 +481,7 @@ __device__ __forceinline__ RayTri ray_setup(float3 v0, float3 v1, float3 v2) {
     return R;
 }
 
-__device__ __forceinline__ bool ray_key(const RayTri &R, int x, int y, const ViewDev &vw, uint64_t id, uint64_t &key) {
-    const float3 r = pixel_ray(x, y, vw.W, vw.H, vw.fx, vw.fy);
+__device__ __forceinline__ bool ray_key(const RayTri &R, float3 r, float nearv, uint64_t id, uint64_t &key) {
     const float3 pv = cross3(r, R.e2);
     const float det = dot3(R.e1, pv);
     if (!(det > 0.0f)) return false;
@@ -487,14 +489,15 @@ __device__ __forceinline__ bool ray_key(const RayTri &R, int x, int y, const Vie
     const float w = __fdiv_rn(dot3(r, R.qv), det);
     const float b0 = __fsub_rn(__fsub_rn(1.0f, u), w);
     const float t = __fdiv_rn(dot3(R.e2, R.qv), det);
-    if (!(u >= 0.0f && w >= 0.0f && b0 >= 0.0f && t >= vw.nearv)) return false;
+    if (!(u >= 0.0f && w >= 0.0f && b0 >= 0.0f && t >= nearv)) return false;
     key = ((uint64_t)(__float_as_uint(t) >> 3) << 36) | (id & kIdMask);
     return true;
 }
 
 __device__ __forceinline__ void ray_pixel(const RayTri &R, int x, int y, const ViewDev &vw, uint64_t id) {
     uint64_t key;
-    if (ray_key(R, x, y, vw, id, key)) depth_min(vw.vis, (size_t)y * (size_t)vw.W + (size_t)x, key);
+    if (ray_key(R, pixel_ray(x, y, vw.W, vw.H, vw.fx, vw.fy), vw.nearv, id, key))
+        depth_min(vw.vis, (size_t)y * (size_t)vw.W + (size_t)x, key);
 }
 
 // Pixels i = start, start + stride, ... of [x0, x1] x [y0, y1] by ray cast.

@@ -339,7 +339,15 @@ __global__ void __launch_bounds__(256) k_stage3(const __grid_constant__ FrameDev
             const ViewDev &vw = f.views[s_view[p]];
             if (s_ray[p]) {
                 RayTri R;
-                if (ray_tri_of(f, s_ray[p] - 1, s.id, R)) ray_range(R, x0, x1, y0, y1, tid, 256, vw, s.id);
+                if (!ray_tri_of(f, s_ray[p] - 1, s.id, R)) continue;
+                for (int x = x0 + lane; x <= x1; x += 32) {
+                    const float rx = ray_axis(x, vw.W, vw.fx);
+                    for (int y = y0 + warp; y <= y1; y += 8) {
+                        uint64_t key;
+                        if (ray_key(R, make_float3(rx, ray_axis(y, vw.H, vw.fy), -1.0f), vw.nearv, s.id, key))
+                            depth_min(vw.vis, (size_t)y * (size_t)vw.W + (size_t)x, key);
+                    }
+                }
                 continue;
             }
             const int W = vw.W;
@@ -528,7 +536,8 @@ __global__ void __launch_bounds__(256) k_stage3_tiles(FrameDev f) {
                 const uint64_t id = pr[j].s.id;
                 for (; y <= ry1; y += dyr) {
                     uint64_t key;
-                    if (ray_key(R, x, by + y, vw, id, key) && key < tw[(y << tl) + lx]) tw[(y << tl) + lx] = key;
+                    if (ray_key(R, pixel_ray(x, by + y, vw.W, vw.H, vw.fx, vw.fy), vw.nearv, id, key) &&
+                        key < tw[(y << tl) + lx]) tw[(y << tl) + lx] = key;
                 }
             } else {
                 const SubTri s = pr[j].s;

@@ -181,9 +181,18 @@ __device__ __forceinline__ void xform2(const FastPair &fp, float2 x, float2 y, f
 // from their vertices' bounds: the margin m, the widened bounds, the
 // pixel-centre test on each axis, the region where the bound holds and, with
 // NEAR, every vertex beyond the near plane.
-template <bool NEAR>
+// BACK: and a triangle that surely faces away.  area is the estimated doubled
+// area in its listed order.  With every exact snapped vertex within m of its
+// estimate on each axis, a difference of two vertices is off by at most 2m,
+// and with the differences at most (dX, dY) the exact area lies within
+// 4m (dX + dY) + 8m^2 of the estimated one (taken as 4.01 and 8.01, for the
+// rounding of the bound), whose own rounding is below 16 ulps of dX dY: an
+// area below minus that sum is negative in the exact path, which drops the
+// triangle.  Seen to pay where the survivors are many: half of what reaches
+// the exact kernel from closed surfaces faces away.
+template <bool NEAR, bool BACK>
 __device__ __forceinline__ void cull_tail2(const FastPair &fp, float2 xmn, float2 xmx, float2 ymn, float2 ymx,
-                                           float2 wmn, float2 wmx, float2 rmx, bool &cp, bool &cq) {
+                                           float2 wmn, float2 wmx, float2 rmx, float2 area, bool &cp, bool &cq) {
     const float4 k = fp.k, lim = fp.lim;
     const float2 a = make_float2(max3f(fabsf(xmn.x), fabsf(xmx.x), fmaxf(fabsf(ymn.x), fabsf(ymx.x))),
                                  max3f(fabsf(xmn.y), fabsf(xmx.y), fmaxf(fabsf(ymn.y), fabsf(ymx.y))));
@@ -192,19 +201,33 @@ __device__ __forceinline__ void cull_tail2(const FastPair &fp, float2 xmn, float
     const bool sp = (wmn.x > lim.x) & (a.x < lim.y), sq = (wmn.y > lim.x) & (a.y < lim.y);
     const bool nxp = floorf(fminf(xh.x, lim.z)) < fmaxf(xl.x, 0.0f), nxq = floorf(fminf(xh.y, lim.z)) < fmaxf(xl.y, 0.0f);
     const bool nyp = floorf(fminf(yh.x, lim.w)) < fmaxf(yl.x, 0.0f), nyq = floorf(fminf(yh.y, lim.w)) < fmaxf(yl.y, 0.0f);
-    cp = sp & (nxp | nyp);
-    cq = sq & (nxq | nyq);
+    bool op = nxp | nyp, oq = nxq | nyq;
+    if (BACK) {
+        const float2 dX = sub_x2(xmx, xmn), dY = sub_x2(ymx, ymn);
+        const float2 t = fma_x2(m, fma_x2(dup(8.01f), m, mul_x2(dup(4.01f), add_x2(dX, dY))),
+                                mul_x2(mul_x2(dup(9.5367431640625e-7f), dX), dY));
+        op |= area.x < -t.x;
+        oq |= area.y < -t.y;
+    }
+    cp = sp & op;
+    cq = sq & oq;
     if (NEAR) {                                       // or every vertex beyond the near plane
         cp |= wmx.x < fp.sl.w;
         cq |= wmx.y < fp.sl.w;
     }
 }
 
+// The doubled areas of two triangles (one per half) from their vertices.
+__device__ __forceinline__ float2 area2(float2 ax, float2 ay, float2 bx, float2 by, float2 cx, float2 cy) {
+    const float2 ux = sub_x2(bx, ax), uy = sub_x2(by, ay), vx = sub_x2(cx, ax), vy = sub_x2(cy, ay);
+    return sub_x2(mul_x2(ux, vy), mul_x2(uy, vx));
+}
+
 // fast_cull for two triangles of the same pair at once: the same arithmetic,
 // with the FMA rows, the products by 1/w, the margin and the widened bounds
 // evaluated on packed pairs (one triangle per half).  NEAR = false leaves the
 // near-plane test out (frames where no vertex can lie near that plane).
-template <bool NEAR = true>
+template <bool NEAR, bool BACK>
 __device__ __forceinline__ void fast_cull2(const FastPair &fp, const Tri9 &p, const Tri9 &q, bool &cp, bool &cq) {
     float2 X[3], Y[3], w[3], r[3];
 #pragma unroll
@@ -220,7 +243,9 @@ __device__ __forceinline__ void fast_cull2(const FastPair &fp, const Tri9 &p, co
     const float2 rmx = make_float2(max3f(r[0].x, r[1].x, r[2].x), max3f(r[0].y, r[1].y, r[2].y));
     float2 wmx = wmn;
     if (NEAR) wmx = make_float2(max3f(w[0].x, w[1].x, w[2].x), max3f(w[0].y, w[1].y, w[2].y));
-    cull_tail2<NEAR>(fp, xmn, xmx, ymn, ymx, wmn, wmx, rmx, cp, cq);
+    float2 area = make_float2(0.0f, 0.0f);
+    if (BACK) area = area2(X[0], Y[0], X[1], Y[1], X[2], Y[2]);
+    cull_tail2<NEAR, BACK>(fp, xmn, xmx, ymn, ymx, wmn, wmx, rmx, area, cp, cq);
 }
 
 // The bounds of two triangles of a strip (one per half) whose vertices are
@@ -360,7 +385,6 @@ constexpr int kItem = kConsumers * kMaxTpt;          // 1024 triangles, 12 KB of
 constexpr int kSlots = 4;
 constexpr int kQueue = 64;                           // per-warp survivors (fused kernel)
 constexpr int kMaxPairs = 64;                        // pairs of one segment (pairs_per_segment <= 64)
-constexpr int kNT = 2;                               // triangles a lane loads together
 constexpr int kCullBlocks = 3;                       // cull blocks per SM: 72 registers a thread (at 4 blocks
                                                      // and 56 registers the four-triangle cull spills)
 
@@ -520,14 +544,13 @@ __device__ __forceinline__ void decode_pair(const MeshDev &mesh, const uint32_t 
     }
 }
 
-// The four triangles of a lane in strip order, (s0 s1 s2) (s2 s1 s3)
-// (s2 s3 s4) (s4 s3 s5) with sv = s0 .. s5: the six vertices loaded and
-// transformed once, each triangle culled from the bounds of its three.
-template <bool NEAR, bool COMP>
-__device__ __forceinline__ void strip_cull(const FastPair &fp, const MeshDev &mesh, const float *pos,
-                                           const uint32_t (&sv)[6], bool (&cull)[4]) {
-    // vertex pairs (s0, s1), (s2, s3), (s4, s5)
-    float2 X[3], Y[3], w[3], r[3];
+// The positions of a lane's six strip vertices, as the packed pairs (s0, s1),
+// (s2, s3), (s4, s5).  Compressed meshes: the 16-bit values, converted exactly
+// (as u16_to_float) and dequantized as fma(q, step, lo).
+struct Strip { float2 x[3], y[3], z[3]; };
+
+template <bool COMP>
+__device__ __forceinline__ void strip_load(const MeshDev &mesh, const float *pos, const uint32_t (&sv)[6], Strip &p) {
     if constexpr (!COMP) {
         float v[18];
 #pragma unroll
@@ -536,12 +559,12 @@ __device__ __forceinline__ void strip_cull(const FastPair &fp, const MeshDev &me
             v[3 * c] = __ldg(q); v[3 * c + 1] = __ldg(q + 1); v[3 * c + 2] = __ldg(q + 2);
         }
 #pragma unroll
-        for (int c = 0; c < 3; ++c)
-            xform2(fp, make_float2(v[6 * c], v[6 * c + 3]), make_float2(v[6 * c + 1], v[6 * c + 4]),
-                   make_float2(v[6 * c + 2], v[6 * c + 5]), X[c], Y[c], w[c], r[c]);
+        for (int c = 0; c < 3; ++c) {
+            p.x[c] = make_float2(v[6 * c], v[6 * c + 3]);
+            p.y[c] = make_float2(v[6 * c + 1], v[6 * c + 4]);
+            p.z[c] = make_float2(v[6 * c + 2], v[6 * c + 5]);
+        }
     } else {
-        // the 16-bit values, converted exactly (as u16_to_float) and
-        // dequantized as fma(q, step, lo), two vertices a packed pair
         uint32_t fb[18];   // bits of the floats 2^23 + value
 #pragma unroll
         for (int c = 0; c < 6; ++c) {
@@ -551,33 +574,80 @@ __device__ __forceinline__ void strip_cull(const FastPair &fp, const MeshDev &me
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            float2 p[3];
+            float2 q[3];
 #pragma unroll
             for (int a = 0; a < 3; ++a)
-                p[a] = fma_x2(sub_x2(make_float2(__int_as_float(fb[6 * c + a]), __int_as_float(fb[6 * c + 3 + a])),
+                q[a] = fma_x2(sub_x2(make_float2(__int_as_float(fb[6 * c + a]), __int_as_float(fb[6 * c + 3 + a])),
                                      dup(8388608.0f)),
                               dup(mesh.step[a]), dup(mesh.lo[a]));
-            xform2(fp, p[0], p[1], p[2], X[c], Y[c], w[c], r[c]);
+            p.x[c] = q[0]; p.y[c] = q[1]; p.z[c] = q[2];
         }
     }
+}
+
+// The four triangles of a strip, triangle k of the vertices s_k, s_k+1, s_k+2:
+// the six vertices transformed once, each triangle culled from the bounds of
+// its three.  BACK: sign is 1 where the triangles are listed with the winding
+// of (s0 s1 s2), (s2 s1 s3), (s2 s3 s4), (s4 s3 s5), else -1.
+template <bool NEAR, bool BACK>
+__device__ __forceinline__ void strip_cull(const FastPair &fp, const Strip &p, float sign, bool (&cull)[4]) {
+    float2 X[3], Y[3], w[3], r[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) xform2(fp, p.x[c], p.y[c], p.z[c], X[c], Y[c], w[c], r[c]);
     // triangles (t0, t1) from the pairs (s0, s1), (s2, s3); (t2, t3) from (s2, s3), (s4, s5)
 #pragma unroll
-    for (int h = 0; h < 2; ++h)
-        cull_tail2<NEAR>(fp, strip_min(X[h], X[h + 1]), strip_max(X[h], X[h + 1]), strip_min(Y[h], Y[h + 1]),
-                         strip_max(Y[h], Y[h + 1]), strip_min(w[h], w[h + 1]),
-                         NEAR ? strip_max(w[h], w[h + 1]) : make_float2(0.0f, 0.0f),
-                         strip_max(r[h], r[h + 1]), cull[2 * h], cull[2 * h + 1]);
+    for (int h = 0; h < 2; ++h) {
+        float2 area = make_float2(0.0f, 0.0f);
+        if (BACK)
+            area = mul_x2(make_float2(sign, -sign),
+                          area2(X[h], Y[h], make_float2(X[h].y, X[h + 1].x), make_float2(Y[h].y, Y[h + 1].x), X[h + 1], Y[h + 1]));
+        cull_tail2<NEAR, BACK>(fp, strip_min(X[h], X[h + 1]), strip_max(X[h], X[h + 1]), strip_min(Y[h], Y[h + 1]),
+                               strip_max(Y[h], Y[h + 1]), strip_min(w[h], w[h + 1]),
+                               NEAR ? strip_max(w[h], w[h + 1]) : make_float2(0.0f, 0.0f),
+                               strip_max(r[h], r[h + 1]), area, cull[2 * h], cull[2 * h + 1]);
+    }
+}
+
+// Whether the four triangles of every lane of the warp are a strip, in one of
+// the orders in which a row of grid cells is commonly listed (two triangles a
+// cell): as (s0 s1 s2) (s2 s1 s3) (s2 s3 s4) (s4 s3 s5) ...
+__device__ __forceinline__ bool strip_rows(const uint32_t (&ix)[12], bool usable, bool all_valid, uint32_t v32) {
+    const uint32_t smax = max(max(ix[0], max(ix[1], ix[2])), max(ix[5], max(ix[8], ix[11])));
+    const bool strip = usable & (all_valid | (smax < v32)) & (ix[3] == ix[2]) & (ix[4] == ix[1]) & (ix[6] == ix[2]) &
+                       (ix[7] == ix[5]) & (ix[9] == ix[8]) & (ix[10] == ix[5]);
+    return __all_sync(0xffffffffu, strip);
+}
+
+// ... or, a lane each in any of the three, the same facing the other way
+// (s0 s2 s1) (s2 s3 s1) ..., or split along the other diagonal
+// (s1 s0 s2) (s1 s2 s3) (s3 s2 s4) (s3 s4 s5).  sv: the six vertices; sign as
+// in strip_cull.
+__device__ __forceinline__ bool strip_other(const uint32_t (&ix)[12], bool usable, bool all_valid, uint32_t v32,
+                                            uint32_t (&sv)[6], float &sign) {
+    const bool a = (ix[3] == ix[2]) & (ix[4] == ix[1]) & (ix[6] == ix[2]) & (ix[7] == ix[5]) & (ix[9] == ix[8]) &
+                   (ix[10] == ix[5]);
+    const bool b = (ix[3] == ix[1]) & (ix[5] == ix[2]) & (ix[6] == ix[1]) & (ix[8] == ix[4]) & (ix[9] == ix[7]) &
+                   (ix[11] == ix[4]);
+    const bool c = (ix[3] == ix[0]) & (ix[4] == ix[2]) & (ix[6] == ix[5]) & (ix[7] == ix[2]) & (ix[9] == ix[5]) &
+                   (ix[10] == ix[8]);
+    sign = a ? 1.0f : -1.0f;
+    sv[0] = c ? ix[1] : ix[0];
+    sv[1] = c ? ix[0] : b ? ix[2] : ix[1];
+    sv[2] = b ? ix[1] : ix[2];
+    sv[3] = b ? ix[4] : ix[5];
+    sv[4] = b ? ix[7] : ix[8];
+    sv[5] = b ? ix[10] : ix[11];
+    const uint32_t smax = max(max(sv[0], max(sv[1], sv[2])), max(sv[3], max(sv[4], sv[5])));
+    return __all_sync(0xffffffffu, usable & (a | b | c) & (all_valid | (smax < v32)));
 }
 
 // Single-pair items of plain meshes, four consecutive triangles a lane: a
 // warp takes the 128-triangle groups g = warp, warp + 8, ... of the item and
 // lane l the triangles 128 g + 4 l .. 128 g + 4 l + 3, whose twelve index
-// words are three 16-byte loads from shared memory.  Where the four are in
-// strip order -- the list a triangle strip s0 s1 s2 s3 s4 s5 unrolls to,
-// (s0 s1 s2) (s2 s1 s3) (s2 s3 s4) (s4 s3 s5), which is how a row-major grid
-// mesh lists a row of cells -- triangle k has the vertices s_k, s_k+1 and
-// s_k+2; when every lane's four are, the warp loads and transforms the six
-// vertices once for the four triangles.  The cull's bounds are symmetric in
+// words are three 16-byte loads from shared memory.  Where the four are a
+// strip (strip_rows, strip_other: a row-major grid mesh lists a row of cells so), triangle
+// k has the vertices s_k, s_k+1 and s_k+2; when every lane's four are, the
+// warp loads and transforms the six vertices once for the four triangles.  The cull's bounds are symmetric in
 // a triangle's vertices, so each triangle gets the decision fast_cull2 would
 // give it.  Other orders run fast_cull2 on the two pairs of triangles.  The
 // 128 decisions are the bitmap words 4 g .. 4 g + 3 of the item (word h:
@@ -612,7 +682,9 @@ __device__ __forceinline__ void cull_quads(const FrameDev &f, const uint32_t *id
             bit += mesh.bits;
             const uint32_t s1 = mesh.imin + (__funnelshift_r(idx[bit >> 5], idx[(bit >> 5) + 1], bit & 31u) & mesh.mask);
             const uint32_t sv[6] = {s0, s1, s0 + 1, s1 + 1, s0 + 2, s1 + 2};
-            strip_cull<NEAR, COMP>(fp, mesh, pos, sv, cull);
+            Strip p;
+            strip_load<COMP>(mesh, pos, sv, p);
+            strip_cull<NEAR, false>(fp, p, 1.0f, cull);
         } else {
             uint32_t ix[12];
             if constexpr (!COMP) {
@@ -627,12 +699,17 @@ __device__ __forceinline__ void cull_quads(const FrameDev &f, const uint32_t *id
                 for (int k = 0; k < 12; ++k, bit += mesh.bits)
                     ix[k] = mesh.imin + (__funnelshift_r(idx[bit >> 5], idx[(bit >> 5) + 1], bit & 31u) & mesh.mask);
             }
-            const uint32_t smax = max(max(ix[0], max(ix[1], ix[2])), max(ix[5], max(ix[8], ix[11])));
-            const bool strip = (lt + 3 < d.n) & (all_valid | (smax < v32)) & (ix[3] == ix[2]) & (ix[4] == ix[1]) &
-                               (ix[6] == ix[2]) & (ix[7] == ix[5]) & (ix[9] == ix[8]) & (ix[10] == ix[5]);
-            if (__all_sync(0xffffffffu, strip)) {
-                const uint32_t sv[6] = {ix[0], ix[1], ix[2], ix[5], ix[8], ix[11]};
-                strip_cull<NEAR, COMP>(fp, mesh, pos, sv, cull);
+            uint32_t sv[6];
+            float sign;
+            if (strip_rows(ix, lt + 3 < d.n, all_valid, v32)) {
+                const uint32_t rv[6] = {ix[0], ix[1], ix[2], ix[5], ix[8], ix[11]};
+                Strip p;
+                strip_load<COMP>(mesh, pos, rv, p);
+                strip_cull<NEAR, false>(fp, p, 1.0f, cull);
+            } else if (!COMP && strip_other(ix, lt + 3 < d.n, all_valid, v32, sv, sign)) {
+                Strip p;
+                strip_load<COMP>(mesh, pos, sv, p);
+                strip_cull<NEAR, false>(fp, p, sign, cull);
             } else {
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
@@ -664,7 +741,7 @@ __device__ __forceinline__ void cull_quads(const FrameDev &f, const uint32_t *id
                             for (int c = 0; c < 9; ++c) p[u].v[c] = 0.0f;
                         }
                     }
-                    fast_cull2<NEAR>(fp, p[0], p[1], cull[2 * h], cull[2 * h + 1]);
+                    fast_cull2<NEAR, false>(fp, p[0], p[1], cull[2 * h], cull[2 * h + 1]);
                 }
             }
         }
@@ -683,6 +760,209 @@ __device__ __forceinline__ void cull_quads(const FrameDev &f, const uint32_t *id
         wd.w = __reduce_or_sync(0xffffffffu, h == 3 ? sh : 0u);
         // 16-byte aligned: the item's words start at a multiple of 8 tpt
         if (lane == 0) *reinterpret_cast<uint4 *>(f.bits + d.wbase + 4 * g) = wd;
+    }
+}
+
+// The box of a group of triangles from each lane's bounds, over the lanes
+// whose index differs in the bits below `lanes`: centre and half extent.
+template <int LANES>
+__device__ __forceinline__ void group_box(float (&lo)[3], float (&hi)[3], float3 &gc, float3 &ge) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int o = LANES / 2; o > 0; o >>= 1) {
+            lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
+            hi[a] = fmaxf(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
+        }
+    gc = make_float3(0.5f * (lo[0] + hi[0]), 0.5f * (lo[1] + hi[1]), 0.5f * (lo[2] + hi[2]));
+    ge = make_float3(fmaxf(hi[0] - gc.x, gc.x - lo[0]), fmaxf(hi[1] - gc.y, gc.y - lo[1]),
+                     fmaxf(hi[2] - gc.z, gc.z - lo[2]));
+}
+
+// One 128-triangle group of an instanced item in strip order: a lane holds
+// the six vertices of its four triangles for all pairs.  Each half warp has a
+// box of its own 64 triangles and tests it against 16 pairs a step; the pairs
+// it cannot reject it then walks one by one, the two halves each at their own
+// pair (the rejected ones' words are zeroed in bulk).  bits: word 0 of the
+// group under pair 0, G words from pair to pair.
+template <bool NEAR>
+__device__ __forceinline__ void cull_strips(const FrameDev &f, const Strip &p, float sign, const FastPair *fps, uint32_t np,
+                                            uint32_t *bits, uint32_t G, int lane) {
+    const uint32_t half = (uint32_t)lane >> 4;
+    uint64_t keep = np >= 64 ? ~0ull : (1ull << np) - 1;       // pairs my half has to walk
+    if (f.group_min != 0 && np >= f.group_min) {
+        float lo[3], hi[3];
+        lo[0] = min3f(fminf(p.x[0].x, p.x[0].y), fminf(p.x[1].x, p.x[1].y), fminf(p.x[2].x, p.x[2].y));
+        hi[0] = max3f(fmaxf(p.x[0].x, p.x[0].y), fmaxf(p.x[1].x, p.x[1].y), fmaxf(p.x[2].x, p.x[2].y));
+        lo[1] = min3f(fminf(p.y[0].x, p.y[0].y), fminf(p.y[1].x, p.y[1].y), fminf(p.y[2].x, p.y[2].y));
+        hi[1] = max3f(fmaxf(p.y[0].x, p.y[0].y), fmaxf(p.y[1].x, p.y[1].y), fmaxf(p.y[2].x, p.y[2].y));
+        lo[2] = min3f(fminf(p.z[0].x, p.z[0].y), fminf(p.z[1].x, p.z[1].y), fminf(p.z[2].x, p.z[2].y));
+        hi[2] = max3f(fmaxf(p.z[0].x, p.z[0].y), fmaxf(p.z[1].x, p.z[1].y), fmaxf(p.z[2].x, p.z[2].y));
+        float3 gc, ge;
+        group_box<16>(lo, hi, gc, ge);
+        uint64_t failed = 0;
+        for (uint32_t pb = 0; pb < np; pb += 16) {
+            const uint32_t q = pb + ((uint32_t)lane & 15u);
+            const bool g = q < np && group_cull<NEAR>(fps[q < np ? q : 0], gc, ge);
+            const unsigned b = __ballot_sync(0xffffffffu, q < np && !g);
+            failed |= (uint64_t)((b >> (16 * half)) & 0xFFFFu) << pb;
+        }
+        // the rejected pairs' words, a pair a lane of the half
+        for (uint32_t q = (uint32_t)lane & 15u; q < np; q += 16)
+            if (!((failed >> q) & 1u)) *reinterpret_cast<uint2 *>(bits + q * G + 2 * half) = make_uint2(0u, 0u);
+        if (f.stats && failed != keep) {
+            const uint32_t rejected = np - (uint32_t)__popcll(failed);
+            stat_add(f, kStatIn, 4 * rejected), stat_add(f, kStatTiny, 4 * rejected);
+        }
+        keep = failed;
+    }
+    while (__any_sync(0xffffffffu, keep != 0)) {
+        const bool has = keep != 0;
+        const uint32_t pi = has ? (uint32_t)__ffsll((long long)keep) - 1 : 0u;
+        keep &= keep - 1;
+        bool cull[4];
+        strip_cull<NEAR, true>(fps[pi], p, sign, cull);
+        uint32_t nib = 0;
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            if (f.stats && has && cull[u]) stat_add(f, kStatIn, 1), stat_add(f, kStatTiny, 1);
+            nib |= (uint32_t)!cull[u] << u;
+        }
+        uint32_t word = nib << (4 * (lane & 7));
+        word |= __shfl_xor_sync(0xffffffffu, word, 1);
+        word |= __shfl_xor_sync(0xffffffffu, word, 2);
+        word |= __shfl_xor_sync(0xffffffffu, word, 4);
+        if (has && (lane & 7) == 0) bits[pi * G + ((uint32_t)lane >> 3)] = word;
+    }
+}
+
+// Instanced items (Section 4.5, extended to several views): a warp takes the
+// 128-triangle groups warp, warp + 8, ... of the item and loops every pair of
+// the item over each.  Where the lanes' triangles are strips (cull_quads),
+// cull_strips holds their six vertices; other orders take two 32-triangle runs
+// of the group at a time, a lane one triangle of each.  Items with group_min
+// pairs or more first test the step's triangles as one box per pair, one pair
+// a lane; the rejected pairs get zero words in bulk and only the others run
+// the per-triangle test.
+template <bool NEAR, bool COMP>
+__device__ __forceinline__ void cull_instanced(const FrameDev &f, const uint32_t *idx, const FastPair *fps,
+                                               const MeshDev &mesh, const s1::Desc &d, uint32_t np, uint32_t tpt, int warp,
+                                               int lane) {
+    using namespace s1;
+    const bool all_valid = mesh.V > 0xFFFFFFFFull;   // every uint32 index is below V
+    const uint32_t v32 = (uint32_t)mesh.V;
+    const uint32_t G = kConsumerWarps * tpt;
+    for (uint32_t g = warp; g < 2 * tpt; g += kConsumerWarps) {   // the warp stays converged
+        const uint32_t lt = 128 * g + 4 * lane;
+        uint32_t *bits = f.bits + d.wbase + 4 * g;
+        {
+            uint32_t ix[12], sv[6];
+            float sign;
+            if constexpr (!COMP) {
+                const uint4 *src = reinterpret_cast<const uint4 *>(idx + 3 * lt);
+                const uint4 ia = src[0], ib = src[1], ic = src[2];
+                ix[0] = ia.x; ix[1] = ia.y; ix[2] = ia.z; ix[3] = ia.w; ix[4] = ib.x; ix[5] = ib.y;
+                ix[6] = ib.z; ix[7] = ib.w; ix[8] = ic.x; ix[9] = ic.y; ix[10] = ic.z; ix[11] = ic.w;
+            } else {
+                uint32_t bit = 3 * lt * mesh.bits;
+#pragma unroll
+                for (int k = 0; k < 12; ++k, bit += mesh.bits)
+                    ix[k] = mesh.imin + (__funnelshift_r(idx[bit >> 5], idx[(bit >> 5) + 1], bit & 31u) & mesh.mask);
+            }
+            if (strip_other(ix, lt + 3 < d.n, all_valid, v32, sv, sign)) {
+                Strip p;
+                strip_load<COMP>(mesh, mesh.pos, sv, p);
+                cull_strips<NEAR>(f, p, sign, fps, np, bits, G, lane);
+                continue;
+            }
+        }
+#pragma unroll 1
+        for (uint32_t run = 0; run < 4; run += 2) {
+            bool valid[2];
+            uint32_t ix[2][3];
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const uint32_t t = 128 * g + 32 * (run + u) + lane;
+                valid[u] = t < d.n;
+                ix[u][0] = ix[u][1] = ix[u][2] = 0;
+                if (valid[u]) {
+                    if (!COMP) {
+                        ix[u][0] = idx[3 * t]; ix[u][1] = idx[3 * t + 1]; ix[u][2] = idx[3 * t + 2];
+                    } else {
+#pragma unroll
+                        for (int c = 0; c < 3; ++c) {
+                            const uint32_t bit = (3 * t + c) * mesh.bits;
+                            ix[u][c] = mesh.imin +
+                                       (__funnelshift_r(idx[bit >> 5], idx[(bit >> 5) + 1], bit & 31u) & mesh.mask);
+                        }
+                    }
+                    if (max(ix[u][0], max(ix[u][1], ix[u][2])) >= v32 && !all_valid) {
+                        if (f.check) atomicOr(f.err, kErrIndex);
+                        valid[u] = false;
+                    }
+                }
+            }
+            Tri9 p[2];
+            if constexpr (COMP) {
+                decode_pair(mesh, ix, valid, p);
+            } else
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                if (valid[u]) {
+#pragma unroll
+                    for (int c = 0; c < 3; ++c) {
+                        const float *q = mesh.pos + 3 * (uint64_t)ix[u][c];
+                        p[u].v[3 * c] = __ldg(q); p[u].v[3 * c + 1] = __ldg(q + 1); p[u].v[3 * c + 2] = __ldg(q + 2);
+                    }
+                } else {
+#pragma unroll
+                    for (int c = 0; c < 9; ++c) p[u].v[c] = 0.0f;
+                }
+            }
+            uint64_t keep = np >= 64 ? ~0ull : (1ull << np) - 1;   // pairs whose group test failed
+            if (f.group_min != 0 && np >= f.group_min) {
+                float lo[3], hi[3];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    lo[a] = INFINITY, hi[a] = -INFINITY;
+#pragma unroll
+                    for (int u = 0; u < 2; ++u)
+                        if (valid[u])
+#pragma unroll
+                            for (int c = 0; c < 3; ++c)
+                                lo[a] = fminf(lo[a], p[u].v[3 * c + a]), hi[a] = fmaxf(hi[a], p[u].v[3 * c + a]);
+                }
+                float3 gc, ge;
+                group_box<32>(lo, hi, gc, ge);
+                keep = 0;
+                for (uint32_t pb = 0; pb < np; pb += 32) {
+                    const uint32_t q = pb + lane;
+                    const bool gq = q < np && group_cull<NEAR>(fps[q < np ? q : 0], gc, ge);
+                    keep |= (uint64_t)__ballot_sync(0xffffffffu, q < np && !gq) << pb;
+                }
+                for (uint32_t q = lane; q < np; q += 32)
+                    if (!((keep >> q) & 1u)) *reinterpret_cast<uint2 *>(bits + q * G + run) = make_uint2(0u, 0u);
+                if (f.stats) {
+                    const uint32_t rejected = np - (uint32_t)__popcll(keep);
+                    const uint32_t nvalid = (uint32_t)valid[0] + (uint32_t)valid[1];
+                    if (rejected && nvalid) stat_add(f, kStatIn, rejected * nvalid), stat_add(f, kStatTiny, rejected * nvalid);
+                }
+            }
+            while (keep) {
+                const uint32_t pi = (uint32_t)__ffsll((long long)keep) - 1;
+                keep &= keep - 1;
+                bool cull[2];
+                fast_cull2<NEAR, true>(fps[pi], p[0], p[1], cull[0], cull[1]);
+                uint2 m;
+                m.x = __ballot_sync(0xffffffffu, valid[0] && !cull[0]);
+                m.y = __ballot_sync(0xffffffffu, valid[1] && !cull[1]);
+                if (f.stats) {
+                    const uint32_t gone = (uint32_t)(valid[0] && cull[0]) + (uint32_t)(valid[1] && cull[1]);
+                    stat_add(f, kStatIn, gone), stat_add(f, kStatTiny, gone);
+                }
+                if (lane == 0) *reinterpret_cast<uint2 *>(bits + pi * G + run) = m;
+            }
+        }
     }
 }
 
@@ -743,133 +1023,10 @@ __global__ void __launch_bounds__(s1::kThreads, (FUSED || INST) ? 3 : s1::kCullB
         const uint32_t v32 = (uint32_t)mesh.V;
         const uint32_t np = INST ? d.npairs : 1u;
         if (!FUSED) {
-            // NT triangles per lane are loaded together (more loads in flight),
-            // then culled for every pair of the item; the pair constants are
-            // read from shared memory, which leaves the registers to the loads
-            constexpr int NT = kNT;
-            constexpr bool comp = COMP;                   // rounds hold one kind of mesh
             if constexpr (!INST) {
                 cull_quads<NEAR, COMP>(f, idx, S.fp[slot][0], mesh, d, tpt, warp, lane);
             } else {
-                // Instanced items: a lane takes one triangle of each of nv
-                // 32-triangle runs a step, the adjacent runs k * 8 + nv * warp
-                // + u (the group test wants the step's triangles together);
-                // the warp's ballot over run q is bitmap word q of the pair.
-                for (uint32_t k = 0; k < tpt; k += NT) {   // uniform trip count: the warp stays converged
-                    bool valid[NT];
-                    uint32_t ix[NT][3];
-#pragma unroll
-                    for (int u = 0; u < NT; ++u) {
-                        const uint32_t lt = 32 * (k * kConsumerWarps + min((uint32_t)NT, tpt - k) * warp + u) + lane;
-                        valid[u] = k + u < tpt && lt < d.n;
-                        ix[u][0] = ix[u][1] = ix[u][2] = 0;
-                        if (valid[u]) {
-                            if (!comp) {
-                                ix[u][0] = idx[3 * lt]; ix[u][1] = idx[3 * lt + 1]; ix[u][2] = idx[3 * lt + 2];
-                            } else {
-#pragma unroll
-                                for (int c = 0; c < 3; ++c) {
-                                    const uint32_t bit = (3 * lt + c) * mesh.bits;
-                                    ix[u][c] = mesh.imin +
-                                               (__funnelshift_r(idx[bit >> 5], idx[(bit >> 5) + 1], bit & 31u) & mesh.mask);
-                                }
-                            }
-                            if (max(ix[u][0], max(ix[u][1], ix[u][2])) >= v32 && !all_valid) {
-                                if (f.check) atomicOr(f.err, kErrIndex);
-                                valid[u] = false;
-                            }
-                        }
-                    }
-                    Tri9 p[NT];
-                    if (comp) {
-                        decode_pair(mesh, ix, valid, p);
-                    } else
-#pragma unroll
-                    for (int u = 0; u < NT; ++u) {
-                        if (valid[u]) {
-#pragma unroll
-                            for (int c = 0; c < 3; ++c) {
-                                const float *q = mesh.pos + 3 * (uint64_t)ix[u][c];
-                                p[u].v[3 * c] = __ldg(q); p[u].v[3 * c + 1] = __ldg(q + 1); p[u].v[3 * c + 2] = __ldg(q + 2);
-                            }
-                        } else {
-#pragma unroll
-                            for (int c = 0; c < 9; ++c) p[u].v[c] = 0.0f;
-                        }
-                    }
-                    static_assert(NT == 2, "the cull evaluates triangles in packed pairs");
-                    if (f.group_min != 0 && np >= f.group_min) {
-                        const uint32_t nv = min((uint32_t)NT, tpt - k);
-                        const uint32_t run0 = k * kConsumerWarps + nv * warp;
-                        // Instanced items first test the step's triangles as one
-                        // group per pair, one pair a lane; the rejected pairs get
-                        // zero words in bulk and only the others run the
-                        // per-triangle test.
-                        float3 gc, ge;                     // the group's box: centre, half extent
-                        {
-                            float lo[3], hi[3];
-#pragma unroll
-                            for (int a = 0; a < 3; ++a) {
-                                lo[a] = INFINITY, hi[a] = -INFINITY;
-#pragma unroll
-                                for (int u = 0; u < NT; ++u)
-                                    if (valid[u])
-#pragma unroll
-                                        for (int c = 0; c < 3; ++c)
-                                            lo[a] = fminf(lo[a], p[u].v[3 * c + a]), hi[a] = fmaxf(hi[a], p[u].v[3 * c + a]);
-#pragma unroll
-                                for (int o = 16; o > 0; o >>= 1) {
-                                    lo[a] = fminf(lo[a], __shfl_xor_sync(0xffffffffu, lo[a], o));
-                                    hi[a] = fmaxf(hi[a], __shfl_xor_sync(0xffffffffu, hi[a], o));
-                                }
-                            }
-                            gc = make_float3(0.5f * (lo[0] + hi[0]), 0.5f * (lo[1] + hi[1]), 0.5f * (lo[2] + hi[2]));
-                            ge = make_float3(fmaxf(hi[0] - gc.x, gc.x - lo[0]), fmaxf(hi[1] - gc.y, gc.y - lo[1]),
-                                             fmaxf(hi[2] - gc.z, gc.z - lo[2]));
-                        }
-                        uint64_t keep = 0;                 // pairs whose group test failed
-                        for (uint32_t pb = 0; pb < np; pb += 32) {
-                            const uint32_t q = pb + lane;
-                            const bool g = q < np && group_cull<NEAR>(S.fp[slot][q < np ? q : 0], gc, ge);
-                            keep |= (uint64_t)__ballot_sync(0xffffffffu, q < np && !g) << pb;
-                        }
-                        for (uint32_t i0 = 0; i0 < 2 * np; i0 += 32) {
-                            const uint32_t i = i0 + lane, pi = i >> 1, u = i & 1u;
-                            if (i < 2 * np && u < nv && !((keep >> pi) & 1u)) f.bits[d.wbase + pi * G + run0 + u] = 0u;
-                        }
-                        if (f.stats) {
-                            const uint32_t rejected = np - (uint32_t)__popcll(keep);
-                            const uint32_t nvalid = (uint32_t)valid[0] + (uint32_t)valid[1];
-                            if (rejected && nvalid) stat_add(f, kStatIn, rejected * nvalid), stat_add(f, kStatTiny, rejected * nvalid);
-                        }
-                        while (keep) {
-                            const uint32_t pi = (uint32_t)__ffsll((long long)keep) - 1;
-                            keep &= keep - 1;
-                            bool cull[NT];
-                            fast_cull2<NEAR>(S.fp[slot][pi], p[0], p[1], cull[0], cull[1]);
-#pragma unroll
-                            for (int u = 0; u < NT; ++u) {
-                                const bool live = valid[u] && !cull[u];
-                                if (f.stats && valid[u] && !live) stat_add(f, kStatIn, 1), stat_add(f, kStatTiny, 1);
-                                const unsigned m = __ballot_sync(0xffffffffu, live);
-                                if (u < nv && lane == 0) f.bits[d.wbase + pi * G + run0 + u] = m;
-                            }
-                        }
-                    } else {
-                        for (uint32_t pi = 0; pi < np; ++pi) {
-                            bool cull[NT];
-                            fast_cull2<NEAR>(S.fp[slot][pi], p[0], p[1], cull[0], cull[1]);
-#pragma unroll
-                            for (int u = 0; u < NT; ++u) {
-                                const bool live = valid[u] && !cull[u];
-                                if (f.stats && valid[u] && !live) stat_add(f, kStatIn, 1), stat_add(f, kStatTiny, 1);
-                                const unsigned m = __ballot_sync(0xffffffffu, live);
-                                const uint32_t word = k * kConsumerWarps + min((uint32_t)NT, tpt - k) * warp + u;
-                                if (k + u < tpt && lane == 0) f.bits[d.wbase + pi * G + word] = m;
-                            }
-                        }
-                    }
-                }
+                cull_instanced<NEAR, COMP>(f, idx, S.fp[slot], mesh, d, np, tpt, warp, lane);
             }
         } else
         for (uint32_t k = 0; k < tpt; ++k) {          // uniform trip count: the warp stays converged
