@@ -45,15 +45,20 @@ cudaError_t launch_quantize_positions(const float *pos, uint64_t V, const double
 cudaError_t launch_count_diff(const uint64_t *a, const uint64_t *b, uint64_t n, unsigned long long *out,
                               cudaStream_t s);
 
+struct InstDev {                // an instance of the screen passes
+    uint64_t base;              // global id of its triangle 0
+    uint32_t mesh, pad;
+};
+
 struct ShadeArgs {
     const uint64_t *vis;
     int W, H;
     float fx, fy;
     const float *inst_mv;       // n_inst x 12
-    const uint64_t *base;       // n_inst + 1
-    const uint32_t *inst_mesh;  // n_inst
+    const InstDev *inst;        // n_inst + 1, the last one's base is the total
     const MeshDev *meshes;
     int n_inst;
+    int rows;                   // pixel rows a thread walks (set by the launchers)
     // resolve
     float *rgba_f32;
     uint8_t *rgba8;
@@ -70,12 +75,12 @@ struct ShadeArgs {
     float *grad_pos;
 };
 
-cudaError_t launch_resolve(const ShadeArgs &a, cudaStream_t s);
+cudaError_t launch_resolve(ShadeArgs a, cudaStream_t s);
 // a.W, a.H: the super-sampled buffer (ss W x ss H); W, H: the output
 cudaError_t launch_resolve_ss(const ShadeArgs &a, int W, int H, cudaStream_t s);
 // resolve with textures and the 4-ray mip-level choice (Section 4.4)
-cudaError_t launch_resolve_textured(const ShadeArgs &a, cudaStream_t s);
-cudaError_t launch_interpolate(const ShadeArgs &a, cudaStream_t s);
+cudaError_t launch_resolve_textured(ShadeArgs a, cudaStream_t s);
+cudaError_t launch_interpolate(ShadeArgs a, cudaStream_t s);
 cudaError_t launch_interpolate_backward(const ShadeArgs &a, cudaStream_t s);
 
 }  // namespace curast

@@ -285,8 +285,7 @@ struct curast_ctx {
     bool inst_dirty = true, meshes_dirty = true;
 
     DevBuf<MeshDev> d_meshes;
-    DevBuf<uint64_t> d_base;
-    DevBuf<uint32_t> d_inst_mesh;
+    DevBuf<InstDev> d_inst;               // n_inst + 1 entries
     DevBuf<float> d_inst_mv;
     PinBuf<float> h_inst_mv;
     cudaEvent_t ev_inst_mv = nullptr;
@@ -394,12 +393,10 @@ curast_status sync_scene(curast_ctx *c, cudaStream_t s) {
     }
     if (c->inst_dirty) {
         const size_t n = c->insts.size();
-        CU(c->d_base.reserve(n + 1));
-        CU(c->d_inst_mesh.reserve(std::max<size_t>(n, 1)));
-        std::vector<uint32_t> im(n);
-        for (size_t i = 0; i < n; ++i) im[i] = c->insts[i].mesh;
-        CU(cudaMemcpyAsync(c->d_base.p, c->base.data(), (n + 1) * sizeof(uint64_t), cudaMemcpyHostToDevice, s));
-        if (n) CU(cudaMemcpyAsync(c->d_inst_mesh.p, im.data(), n * sizeof(uint32_t), cudaMemcpyHostToDevice, s));
+        CU(c->d_inst.reserve(n + 1));
+        std::vector<InstDev> id(n + 1);
+        for (size_t i = 0; i <= n; ++i) id[i] = InstDev{c->base[i], i < n ? c->insts[i].mesh : 0u, 0u};
+        CU(cudaMemcpyAsync(c->d_inst.p, id.data(), (n + 1) * sizeof(InstDev), cudaMemcpyHostToDevice, s));
         c->mesh_insts.assign(c->meshes.size(), {});
         for (size_t i = 0; i < n; ++i) c->mesh_insts[c->insts[i].mesh].push_back((uint32_t)i);
         c->inst_dirty = false;
@@ -738,8 +735,7 @@ curast_status shade_setup(curast_ctx *c, const float *view, const float *proj, i
     a->fx = cam.fx;
     a->fy = cam.fy;
     a->inst_mv = c->d_inst_mv.p;
-    a->base = c->d_base.p;
-    a->inst_mesh = c->d_inst_mesh.p;
+    a->inst = c->d_inst.p;
     a->meshes = c->d_meshes.p;
     a->n_inst = (int)c->insts.size();
     return CURAST_OK;
@@ -914,7 +910,7 @@ curast_status curast_create(curast_ctx **out, int device) {
     if (st == CURAST_OK) st = cuda_status(cudaEventCreateWithFlags(&c->ev_tab, cudaEventDisableTiming));
     if (st == CURAST_OK) st = cuda_status(cudaEventCreateWithFlags(&c->ev_inst_mv, cudaEventDisableTiming));
     if (st == CURAST_OK) st = alloc_queues(c);
-    if (st == CURAST_OK) st = cuda_status(c->d_base.reserve(1));
+    if (st == CURAST_OK) st = cuda_status(c->d_inst.reserve(1));
     if (st != CURAST_OK) {
         curast_destroy(c);
         return st;
@@ -930,8 +926,7 @@ void curast_destroy(curast_ctx *c) {
     invalidate_graph(c);
     for (MeshRec &m : c->meshes) free_compressed(m);
     c->d_meshes.release();
-    c->d_base.release();
-    c->d_inst_mesh.release();
+    c->d_inst.release();
     c->d_inst_mv.release();
     c->h_inst_mv.release();
     c->d_tab.release();
