@@ -117,8 +117,8 @@ typedef struct {
                                     parts of a tile meet there, and each covered pixel takes
                                     one global atomic minimum; 0 (default, faster on most of
                                     the workloads measured): every covered pixel of every
-                                    part goes to the global buffer after a plain read (the
-                                    result is the same)                                      */
+                                    part goes straight to the global buffer (the result is
+                                    the same)                                                */
     uint32_t reserved;           /* 0                                                        */
 } curast_config;
 
@@ -396,8 +396,9 @@ curast_status curast_autotune(curast_ctx *ctx, const curast_view *views, int n_v
  *     CURAST_OK;
  *   - the call works on the current CUDA device, which must hold pos, idx,
  *     vis and the stream;
- *   - the stage-1 cull runs its exact path for every triangle (no mesh
- *     bounds are computed), so it is slower than curast_render.
+ *   - the mesh's bounds, which the stage-1 cull needs, are found anew in every
+ *     call (frames of 2^17 (triangle, instance)s or more), so it is slower
+ *     than curast_render.
  * Fails with CURAST_ERR_TOO_LARGE for n_instances outside 1..32 or V, T at
  * or above 2^32. */
 #define CURAST_STATIC_MAX_INSTANCES 32

@@ -181,7 +181,7 @@ struct FrameDev {
     const MeshDev *meshes;
     Q1Entry *q1;
     Q2Entry *q2;
-    uint32_t *bits;          // survivor bitmap of the current round (nullptr: fused stage 1)
+    uint32_t *bits;          // survivor bitmap of the current round
     Counters *ctr;
     unsigned *err;           // sticky error bits, cleared by curast_sync
     uint64_t q1_cap, q2_cap;

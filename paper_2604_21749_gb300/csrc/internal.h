@@ -7,8 +7,8 @@
 namespace curast {
 
 struct LaunchShape {
-    int stage1_blocks_per_sm[2][4];   // [instanced][variant: 0 cull, 1 fused, 2 cull of compressed meshes,
-                                      //  3 single-pair cull with vertex windows (not instanced)]
+    int stage1_blocks_per_sm[2][3];   // [instanced][variant: 0 plain meshes, 1 compressed ones,
+                                      //  2 single-pair cull with vertex windows (not instanced)]
     int stage1x_blocks_per_sm;        // exact kernel of stage 1
     int stage2_blocks_per_sm;
     int stage3_blocks_per_sm;
@@ -19,10 +19,9 @@ struct LaunchShape {
 cudaError_t query_launch_shape(LaunchShape *out, int device);
 
 cudaError_t launch_clear(uint64_t *vis, uint64_t n, cudaStream_t s);
-// Stage 1 of round r: the cull kernel (fused: it runs the exact path itself
-// and needs no bitmap), then the exact kernel over the round's bitmap.
-// near = false launches the cull (not the fused form) without its near-plane
-// test (valid when no pair's mesh bounds reach the near plane).
+// Stage 1 of round r: the cull kernel, then the exact kernel over the round's
+// bitmap.  near = false launches the cull without its near-plane test (valid
+// when no pair's mesh bounds reach the near plane).
 cudaError_t launch_stage1(const FrameDev &f, bool instanced, int variant, uint32_t r, int blocks, bool near,
                           cudaStream_t s);
 cudaError_t launch_stage1_exact(const FrameDev &f, uint32_t r, int blocks, cudaStream_t s);

@@ -166,99 +166,6 @@ __device__ __forceinline__ void q1_append(const FrameDev &f, bool want, uint32_t
 }
 
 // ---------------------------------------------------------------- stage 1 --
-// Small-triangle rasterizer of Section 4.1: one thread per triangle, y outer
-// / x inner over the bounding box with incrementally updated edge functions.
-// int32 is exact here because both bbox extents are below 2^14 subpixels,
-// so |E| < 2^30 at every visited sample.
-__device__ __forceinline__ void raster_small(const int X[3], const int Y[3], const float iz[3], int64_t A, int x0,
-                                             int x1, int y0, int y1, uint64_t id, uint64_t *vis, int W) {
-    const int px0 = 256 * x0 + 128, py0 = 256 * y0 + 128;
-    // edge k runs from vertex k+1 to vertex k+2
-    const int ax0 = X[1], ay0 = Y[1], dx0 = X[2] - X[1], dy0 = Y[2] - Y[1];
-    const int ax1 = X[2], ay1 = Y[2], dx1 = X[0] - X[2], dy1 = Y[0] - Y[2];
-    const int ax2 = X[0], ay2 = Y[0], dx2 = X[1] - X[0], dy2 = Y[1] - Y[0];
-    int e0 = dx0 * (py0 - ay0) - dy0 * (px0 - ax0);
-    int e1 = dx1 * (py0 - ay1) - dy1 * (px0 - ax1);
-    int e2 = dx2 * (py0 - ay2) - dy2 * (px0 - ax2);
-    const int b0 = (dy0 < 0 || (dy0 == 0 && dx0 < 0)) ? 0 : 1;
-    const int b1 = (dy1 < 0 || (dy1 == 0 && dx1 < 0)) ? 0 : 1;
-    const int b2 = (dy2 < 0 || (dy2 == 0 && dx2 < 0)) ? 0 : 1;
-    const float fA = __ll2float_rn(A);
-    for (int y = y0; y <= y1; ++y) {
-        int r0 = e0, r1 = e1, r2 = e2;
-        uint64_t *row = vis + (size_t)y * (size_t)W;
-        for (int x = x0; x <= x1; ++x) {
-            if (((r0 - b0) | (r1 - b1) | (r2 - b2)) >= 0) {
-                float s = __fadd_rn(__fadd_rn(__fmul_rn(__int2float_rn(r0), iz[0]), __fmul_rn(__int2float_rn(r1), iz[1])),
-                                    __fmul_rn(__int2float_rn(r2), iz[2]));
-                float depth = __fdiv_rn(fA, s);
-                uint64_t key = ((uint64_t)(__float_as_uint(depth) >> 3) << 36) | (id & kIdMask);
-                depth_min(row, (size_t)x, key);
-            }
-            r0 -= dy0 * 256; r1 -= dy1 * 256; r2 -= dy2 * 256;
-        }
-        e0 += dx0 * 256; e1 += dx1 * 256; e2 += dx2 * 256;
-    }
-}
-
-// Per-vertex record of one (instance, view): the snapped screen position and
-// 1/depth, or X = INT_MIN with Y = the clip outcode when the vertex lies
-// outside the near plane or the guard band.
-struct Rec { int X, Y; float iz; };
-constexpr int kOutside = (int)0x80000000;
-
-__device__ __forceinline__ Rec make_rec(CV c, const ViewDev &vw) {
-    Rec r;
-    // Inside every plane, decided without the five plane values: w >= near,
-    // |x| <= 128 w and |y| <= 128 w give the same answers as the signs of
-    // w - near, x + 128 w, ... (a sum of two finite floats rounds to zero only
-    // when it is zero; no flush to zero here), NaN fails both forms, and an
-    // infinite 128 w takes the full outcode (inf - inf is NaN there).
-    const float gw = __fmul_rn(kGuard, c.w);
-    const bool inside = (c.w >= vw.nearv) & (gw < INFINITY) & (fabsf(c.x) <= gw) & (fabsf(c.y) <= gw);
-    const unsigned oc = inside ? 0u : outcode(c, vw.nearv);
-    if (oc) {
-        r.X = kOutside;
-        r.Y = (int)oc;
-        r.iz = 0.0f;
-    } else {
-        snap(c, vw.hw, vw.hh, r.X, r.Y, r.iz);
-    }
-    return r;
-}
-
-enum Class { kDrop = 0, kQueue = 1, kSmall = 2 };
-
-// Cull tests of one triangle of one (instance, view) from its vertex records:
-// beyond one clip plane -> drop; crossing the near plane or the guard band
-// -> stage 2 (clipping); back-facing or degenerate -> drop; bbox without a
-// pixel centre on screen (frustum and tiny-triangle cull) -> drop; bbox over
-// the stage-1 limit -> stage 2; else rasterize here.
-__device__ __forceinline__ int classify(const FrameDev &f, const Rec r[3], const ViewDev &vw, int &x0, int &x1,
-                                        int &y0, int &y1, int64_t &A, unsigned &stat) {
-    if (r[0].X == kOutside || r[1].X == kOutside || r[2].X == kOutside) {
-        const unsigned o0 = r[0].X == kOutside ? (unsigned)r[0].Y : 0u;
-        const unsigned o1 = r[1].X == kOutside ? (unsigned)r[1].Y : 0u;
-        const unsigned o2 = r[2].X == kOutside ? (unsigned)r[2].Y : 0u;
-        if (o0 & o1 & o2) { stat = kStatClip; return kDrop; }
-        return kQueue;
-    }
-    A = (int64_t)(r[1].X - r[0].X) * (int64_t)(r[2].Y - r[0].Y) - (int64_t)(r[2].X - r[0].X) * (int64_t)(r[1].Y - r[0].Y);
-    if (A <= 0) { stat = kStatBack; return kDrop; }
-    const int minX = min(r[0].X, min(r[1].X, r[2].X)), maxX = max(r[0].X, max(r[1].X, r[2].X));
-    const int minY = min(r[0].Y, min(r[1].Y, r[2].Y)), maxY = max(r[0].Y, max(r[1].Y, r[2].Y));
-    // pixel centres 256 x + 128 inside [min, max] (arithmetic shifts are
-    // floor divisions), clamped to the screen
-    x0 = max(-((128 - minX) >> 8), 0);
-    x1 = min((maxX - 128) >> 8, vw.W - 1);
-    y0 = max(-((128 - minY) >> 8), 0);
-    y1 = min((maxY - 128) >> 8, vw.H - 1);
-    if (x0 > x1 || y0 > y1) { stat = kStatTiny; return kDrop; }
-    if (maxX - minX >= (1 << 14) || maxY - minY >= (1 << 14)) return kQueue;
-    if ((uint32_t)((x1 - x0 + 1) * (y1 - y0 + 1)) > f.s1_max) return kQueue;
-    return kSmall;
-}
-
 #include "stage1.cuh"
 #include "stage1_exact.cuh"
 #include "stage1_win.cuh"
@@ -623,38 +530,35 @@ __global__ void k_aabb_final(const float *part, int n, float *out) {
 }
 
 // -------------------------------------------------------------- launchers --
-template <bool INST, bool FUSED, bool COMP, bool NEAR = true>
+template <bool INST, bool COMP, bool NEAR>
 cudaError_t stage1_shape(int *blocks) {
-    const size_t sm = stage1_smem_bytes<INST, FUSED>();
-    cudaError_t e = cudaFuncSetAttribute(k_stage1<INST, FUSED, COMP, NEAR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)sm);
+    const size_t sm = stage1_smem_bytes<INST>();
+    cudaError_t e = cudaFuncSetAttribute(k_stage1<INST, COMP, NEAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k_stage1<INST, FUSED, COMP, NEAR>, s1::kThreads, sm);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k_stage1<INST, COMP, NEAR>, s1::kThreads, sm);
 }
 
 cudaError_t query_launch_shape(LaunchShape *o, int device) {
     cudaError_t e = cudaDeviceGetAttribute(&o->num_sms, cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess) return e;
-    if ((e = stage1_shape<false, false, false>(&o->stage1_blocks_per_sm[0][0])) != cudaSuccess) return e;
     {   // the forms without the near-plane test run at the same shape
         int b = 0;
-        if ((e = stage1_shape<false, false, false, false>(&b)) != cudaSuccess) return e;
-        if ((e = stage1_shape<false, false, true, false>(&b)) != cudaSuccess) return e;
-        if ((e = stage1_shape<true, false, false, false>(&b)) != cudaSuccess) return e;
-        if ((e = stage1_shape<true, false, true, false>(&b)) != cudaSuccess) return e;
+        if ((e = stage1_shape<false, false, false>(&b)) != cudaSuccess) return e;
+        if ((e = stage1_shape<false, true, false>(&b)) != cudaSuccess) return e;
+        if ((e = stage1_shape<true, false, false>(&b)) != cudaSuccess) return e;
+        if ((e = stage1_shape<true, true, false>(&b)) != cudaSuccess) return e;
     }
-    if ((e = stage1_shape<false, true, false>(&o->stage1_blocks_per_sm[0][1])) != cudaSuccess) return e;
-    if ((e = stage1_shape<false, false, true>(&o->stage1_blocks_per_sm[0][2])) != cudaSuccess) return e;
-    if ((e = stage1_shape<true, false, false>(&o->stage1_blocks_per_sm[1][0])) != cudaSuccess) return e;
-    if ((e = stage1_shape<true, true, false>(&o->stage1_blocks_per_sm[1][1])) != cudaSuccess) return e;
-    if ((e = stage1_shape<true, false, true>(&o->stage1_blocks_per_sm[1][2])) != cudaSuccess) return e;
+    if ((e = stage1_shape<false, false, true>(&o->stage1_blocks_per_sm[0][0])) != cudaSuccess) return e;
+    if ((e = stage1_shape<false, true, true>(&o->stage1_blocks_per_sm[0][1])) != cudaSuccess) return e;
+    if ((e = stage1_shape<true, false, true>(&o->stage1_blocks_per_sm[1][0])) != cudaSuccess) return e;
+    if ((e = stage1_shape<true, true, true>(&o->stage1_blocks_per_sm[1][1])) != cudaSuccess) return e;
     {
         const size_t sw = stage1_win_smem_bytes();
         e = cudaFuncSetAttribute(k_stage1_win, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sw);
         if (e != cudaSuccess) return e;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o->stage1_blocks_per_sm[0][3], k_stage1_win, s1::kThreads, sw);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o->stage1_blocks_per_sm[0][2], k_stage1_win, s1::kThreads, sw);
         if (e != cudaSuccess) return e;
-        o->stage1_blocks_per_sm[1][3] = o->stage1_blocks_per_sm[0][3];
+        o->stage1_blocks_per_sm[1][2] = o->stage1_blocks_per_sm[0][2];
     }
     e = cudaFuncSetAttribute(k_stage1_exact<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)exact_smem_bytes());
     if (e != cudaSuccess) return e;
@@ -688,21 +592,18 @@ cudaError_t launch_clear(uint64_t *vis, uint64_t n, cudaStream_t s) {
 
 cudaError_t launch_stage1(const FrameDev &f, bool instanced, int variant, uint32_t r, int blocks, bool near,
                           cudaStream_t s) {
-    const size_t s0 = stage1_smem_bytes<false, false>(), s1f = stage1_smem_bytes<false, true>();
-    const size_t i0 = stage1_smem_bytes<true, false>(), i1f = stage1_smem_bytes<true, true>();
+    const size_t s0 = stage1_smem_bytes<false>(), si = stage1_smem_bytes<true>();
     if (instanced) {
-        if (variant == 1) k_stage1<true, true, false><<<blocks, s1::kThreads, i1f, s>>>(f, r);
-        else if (variant == 2 && near) k_stage1<true, false, true, true><<<blocks, s1::kThreads, i0, s>>>(f, r);
-        else if (variant == 2) k_stage1<true, false, true, false><<<blocks, s1::kThreads, i0, s>>>(f, r);
-        else if (near) k_stage1<true, false, false, true><<<blocks, s1::kThreads, i0, s>>>(f, r);
-        else k_stage1<true, false, false, false><<<blocks, s1::kThreads, i0, s>>>(f, r);
+        if (variant == 1 && near) k_stage1<true, true, true><<<blocks, s1::kThreads, si, s>>>(f, r);
+        else if (variant == 1) k_stage1<true, true, false><<<blocks, s1::kThreads, si, s>>>(f, r);
+        else if (near) k_stage1<true, false, true><<<blocks, s1::kThreads, si, s>>>(f, r);
+        else k_stage1<true, false, false><<<blocks, s1::kThreads, si, s>>>(f, r);
     } else {
-        if (variant == 3) k_stage1_win<<<blocks, s1::kThreads, stage1_win_smem_bytes(), s>>>(f, r);
-        else if (variant == 1) k_stage1<false, true, false><<<blocks, s1::kThreads, s1f, s>>>(f, r);
-        else if (variant == 2 && near) k_stage1<false, false, true, true><<<blocks, s1::kThreads, s0, s>>>(f, r);
-        else if (variant == 2) k_stage1<false, false, true, false><<<blocks, s1::kThreads, s0, s>>>(f, r);
-        else if (near) k_stage1<false, false, false, true><<<blocks, s1::kThreads, s0, s>>>(f, r);
-        else k_stage1<false, false, false, false><<<blocks, s1::kThreads, s0, s>>>(f, r);
+        if (variant == 2) k_stage1_win<<<blocks, s1::kThreads, stage1_win_smem_bytes(), s>>>(f, r);
+        else if (variant == 1 && near) k_stage1<false, true, true><<<blocks, s1::kThreads, s0, s>>>(f, r);
+        else if (variant == 1) k_stage1<false, true, false><<<blocks, s1::kThreads, s0, s>>>(f, r);
+        else if (near) k_stage1<false, false, true><<<blocks, s1::kThreads, s0, s>>>(f, r);
+        else k_stage1<false, false, false><<<blocks, s1::kThreads, s0, s>>>(f, r);
     }
     return cudaGetLastError();
 }

@@ -12,6 +12,7 @@
 #include <new>
 #include <vector>
 
+#include "cull_constants.h"
 #include "curast.h"
 #include "internal.h"
 
@@ -146,90 +147,6 @@ bool instance_visible(const float *mv, const MeshRec &m, const Cam &cam) {
         all_b = all_b && (-cy - (1 + eps) * cw > e);
     }
     return !(all_near || all_l || all_r || all_b || all_t);
-}
-
-// Constants of the conservative tiny-triangle cull of one (instance, view).
-// The estimate X'_f = (fn_x . p) / (fn_w . p) uses FMA rows and an
-// approximate reciprocal; the exact path is the FP32 sequence of the
-// projection (Eq. 2) and the snap.  Forward error analysis of both, with
-// S_r = sum_j |m_rj a_j| + |m_r3| (a_j the largest |coordinate| of the mesh
-// bounds), bounds their distance by max(1/w) (ka + kb |X'|) + kc |X'| + kd
-// pixels (the terms are listed below).  wsafe keeps the exact depth of every
-// vertex above the near plane.
-void fast_constants(PairDev &p, const MeshRec &m, const ViewDev &v) {
-    std::memset(p.fn, 0, sizeof(p.fn));
-    std::memset(p.fk, 0, sizeof(p.fk));
-    std::memset(p.fs, 0, sizeof(p.fs));
-    p.nlo = -INFINITY;
-    p.wsafe = INFINITY;
-    p.win = 0.0f;
-    if (!m.bounded) return;
-    // u: FP32 unit roundoff; rho: relative error assumed for rcp.approx.ftz.f32
-    // (8x the documented one ulp)
-    const double u = std::ldexp(1.0, -24), rho = std::ldexp(1.0, -20);
-    double amax[3], S[3];
-    for (int j = 0; j < 3; ++j) amax[j] = std::max(std::fabs(m.lo[j]), std::fabs(m.hi[j]));
-    for (int r = 0; r < 3; ++r) {
-        S[r] = std::fabs((double)p.mv[4 * r + 3]);
-        for (int j = 0; j < 3; ++j) S[r] += std::fabs((double)p.mv[4 * r + j]) * amax[j];
-    }
-    const double hw = v.hw, hh = v.hh, fx = v.fx, fy = v.fy;
-    const double ax = hw * fx, bx = hw - 0.5, ay = hh * fy, by = hh - 0.5;
-    for (int j = 0; j < 4; ++j) {
-        const double wr = -(double)p.mv[8 + j];
-        p.fn[j] = (float)(ax * (double)p.mv[j] + bx * wr);
-        p.fn[4 + j] = (float)(ay * (double)p.mv[4 + j] + by * wr);
-        p.fn[8 + j] = (float)wr;
-    }
-    // Near plane: the w row holds the exact path's own coefficients, negated,
-    // so the FMA estimate and the exact path's w (three products and sums
-    // without FMA) are each within 3.01 u S_z of the true value; a vertex
-    // whose estimate lies below near - 8 u S_z is beyond the near plane in
-    // the exact path, and a triangle with all three there is dropped by it.
-    {
-        const double nl = (double)v.nearv - 8 * u * S[2];
-        float f = (float)nl;
-        if ((double)f > nl) f = std::nextafter(f, -INFINITY);
-        p.nlo = f;
-    }
-    // Error budget per coordinate (pixels), exact path plus estimate:
-    //   (9.002u a S_axis + 4.001u b S_z + 4.001u h S_z + 7.002u (|X'| + 1) S_z) / w
-    //   + (|X'| + 1)(rho + 7.01u) + 5.01u (h + 1) + 1/512 (the snap),
-    // with 1/w <= max(1/w~) (1 + 4u S_z / wsafe) / (1 - rho) for the estimated w~.
-    double ws = v.nearv * (1 + 1e-3) + 8 * u * S[2];
-    const double F = 1.01 * (1 + 4 * u * S[2] / ws) / (1 - rho);
-    const double kax = 9.002 * ax * S[0] + 4.001 * bx * S[2] + 4.001 * hw * S[2] + 7.002 * S[2];
-    const double kay = 9.002 * ay * S[1] + 4.001 * by * S[2] + 4.001 * hh * S[2] + 7.002 * S[2];
-    const double ka = F * u * std::max(kax, kay);
-    const double kb = F * u * 7.002 * S[2];
-    const double kc = 1.01 * (rho + 7.01 * u);
-    const double kd = 1.01 * (5.01 * u * (std::max(hw, hh) + 1) + rho + 7.01 * u) + 1.0 / 512;
-    // The test applies where w > wsafe and |X'|, |Y'| < win = 100 min(W/2,
-    // H/2).  wsafe is raised until the margin stays below 20 min(W/2, H/2)
-    // there (the reciprocal may read 1 + rho high), so every exact vertex of a
-    // tested triangle has |X'|, |Y'| < 120 min(W/2, H/2): well inside the
-    // guard band (|X - W/2| <= 128 W/2, likewise for Y), where the exact path
-    // snaps it and never clips.  The bound is linear in |X'| and holds at any
-    // size of the margin; a margin of many pixels only culls less.
-    const double hm = std::min(hw, hh);
-    const double win = 100.0 * hm;
-    const double room = 20.0 * hm - kc * win - kd;
-    if (!(room > 0.0)) return;
-    ws = std::max(ws, 1.01 * (1 + rho) * (ka + kb * win) / room);
-    if (!std::isfinite(ka) || !std::isfinite(ws) || ka > 1e30 || ws > 1e30) return;
-    // round the constants up (the window down) so the float copies stay conservative
-    p.fk[0] = (float)(ka * (1 + 1e-6));
-    p.fk[1] = (float)(kb * (1 + 1e-6));
-    p.fk[2] = (float)(kc * (1 + 1e-6));
-    p.fk[3] = (float)(kd * (1 + 1e-6));
-    // the rows' magnitude over the mesh bounds is at most ax S_0 + bx S_2,
-    // ay S_1 + by S_2 and S_2; 2^-19 of it covers the rounding of the group
-    // test's box arithmetic (centre, half extent, row sums: a few u each)
-    p.fs[0] = (float)(std::ldexp(ax * S[0] + bx * S[2], -19) * (1 + 1e-6));
-    p.fs[1] = (float)(std::ldexp(ay * S[1] + by * S[2], -19) * (1 + 1e-6));
-    p.fs[2] = (float)(std::ldexp(S[2], -19) * (1 + 1e-6));
-    p.wsafe = (float)(ws * (1 + 1e-6));
-    p.win = (float)win;
 }
 
 // Whether the near-plane test of the stage-1 cull could fire for a pair: w is
@@ -450,7 +367,7 @@ curast_status build_frame(curast_ctx *c, const curast_view *views, int nv, long 
                 p.base = c->base[i];
                 p.view = (uint32_t)v;
                 p.mesh = (uint32_t)m;
-                fast_constants(p, mr, c->hv[v]);
+                cull_constants(p, mr.bounded, mr.lo, mr.hi, c->hv[v]);
                 if (c->cfg.stage1_exact_all) p.wsafe = INFINITY, p.nlo = -INFINITY;   // no conservative cull
                 c->near_needed = c->near_needed || may_reach_near(p, mr, cams[v]);
                 c->hp.push_back(p);
@@ -646,7 +563,7 @@ curast_status enqueue_stages(curast_ctx *c, bool clear, bool timing, cudaStream_
     // kernel empties it (ev[2] falls after the last round's cull)
     const uint32_t nr = (uint32_t)c->rounds.size();
     for (uint32_t r = 0; r < nr; ++r) {
-        const int variant = c->round_comp[r] ? 2 : (!c->instanced && c->cfg.stage1_vertex_reuse ? 3 : 0);
+        const int variant = c->round_comp[r] ? 1 : (!c->instanced && c->cfg.stage1_vertex_reuse ? 2 : 0);
         CU(launch_stage1(f, c->instanced, variant, r, sms * c->shape.stage1_blocks_per_sm[c->instanced ? 1 : 0][variant],
                          c->near_needed, s));
         if (timing && r + 1 == nr) CU(cudaEventRecord(c->ev[2], s));

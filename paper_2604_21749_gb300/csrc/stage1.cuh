@@ -75,45 +75,6 @@ struct __align__(16) FastPair {
 
 struct Tri9 { float v[9]; };    // the three vertices of a triangle
 
-// The "bbox holds no pixel centre" test of Section 4.1, done before the
-// exact arithmetic: the estimated bbox widened by the error bound must hold
-// no pixel centre of the screen while every vertex lies safely in front of
-// the near plane and inside the window -- then the exact snapped bbox holds
-// none either and the exact path would drop the triangle as well.
-// Evaluated without branches.
-__device__ __forceinline__ bool fast_cull(const FastPair &fp, const Tri9 &p) {
-    // vertex by vertex into running bounds (few live registers); the host
-    // chose wsafe so that every w > wsafe keeps each exact vertex of a
-    // tested triangle inside the guard band (no clipping in the exact path)
-    float xmn, xmx, ymn, ymx, wmn, wmx, rmx;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        const float x = p.v[3 * c], y = p.v[3 * c + 1], z = p.v[3 * c + 2];
-        const float4 rx = fp.rx, ry = fp.ry, rw = fp.rw;
-        const float xw = __fmaf_rn(rx.x, x, __fmaf_rn(rx.y, y, __fmaf_rn(rx.z, z, rx.w)));
-        const float yw = __fmaf_rn(ry.x, x, __fmaf_rn(ry.y, y, __fmaf_rn(ry.z, z, ry.w)));
-        const float w = __fmaf_rn(rw.x, x, __fmaf_rn(rw.y, y, __fmaf_rn(rw.z, z, rw.w)));
-        const float r = rcp_approx(w);
-        const float X = xw * r, Y = yw * r;
-        if (c == 0) {
-            xmn = xmx = X; ymn = ymx = Y; wmn = wmx = w; rmx = r;
-        } else {
-            xmn = fminf(xmn, X); xmx = fmaxf(xmx, X);
-            ymn = fminf(ymn, Y); ymx = fmaxf(ymx, Y);
-            wmn = fminf(wmn, w); wmx = fmaxf(wmx, w); rmx = fmaxf(rmx, r);
-        }
-    }
-    const float4 k = fp.k, lim = fp.lim;
-    const float a = fmaxf(fmaxf(fabsf(xmn), fabsf(xmx)), fmaxf(fabsf(ymn), fabsf(ymx)));
-    const float m = __fmaf_rn(rmx, __fmaf_rn(k.y, a, k.x), __fmaf_rn(k.z, a, k.w));
-    const bool safe = (wmn > lim.x) & (a < lim.y);
-    // no integer in [lo, hi] within [0, last] on one axis: floor(min(hi, last)) < max(lo, 0)
-    const bool nx = floorf(fminf(xmx + m, lim.z)) < fmaxf(xmn - m, 0.0f);
-    const bool ny = floorf(fminf(ymx + m, lim.w)) < fmaxf(ymn - m, 0.0f);
-    // or every vertex beyond the near plane
-    return (safe & (nx | ny)) | (wmx < fp.sl.w);
-}
-
 // Packed FP32 pairs (Blackwell f32x2): two independent operations in one
 // instruction, each half rounded exactly like the scalar __fmaf_rn,
 // __fmul_rn, __fadd_rn and __fsub_rn.
@@ -223,8 +184,13 @@ __device__ __forceinline__ float2 area2(float2 ax, float2 ay, float2 bx, float2 
     return sub_x2(mul_x2(ux, vy), mul_x2(uy, vx));
 }
 
-// fast_cull for two triangles of the same pair at once: the same arithmetic,
-// with the FMA rows, the products by 1/w, the margin and the widened bounds
+// The conservative "bbox holds no pixel centre" test of Section 4.1, done
+// before the exact arithmetic, for two triangles of the same pair: the
+// estimated bbox widened by the error bound must hold no pixel centre of the
+// screen while every vertex lies safely in front of the near plane and inside
+// the window -- then the exact snapped bbox holds none either and the exact
+// path would drop the triangle as well (the host chose wsafe so that no vertex
+// of a tested triangle is clipped there).  Evaluated without branches, with the FMA rows, the products by 1/w, the margin and the widened bounds
 // evaluated on packed pairs (one triangle per half).  NEAR = false leaves the
 // near-plane test out (frames where no vertex can lie near that plane).
 template <bool NEAR, bool BACK>
@@ -327,54 +293,6 @@ __device__ __forceinline__ void exact_gather(const FrameDev &f, uint2 e, bool li
     }
 }
 
-// The exact path given the triangle's positions (from exact_gather).
-template <bool RAY>
-__device__ __forceinline__ void exact_compute(const FrameDev &f, uint2 e, bool live, const Tri9 &p) {
-    const uint32_t pidx = live ? e.y : 0u;
-    const uint64_t t = live ? e.x : 0u;
-    const PairDev &pr = f.pairs[pidx];
-    const MeshDev *mesh = f.meshes + pr.mesh;
-    const ViewDev vw = f.views[pr.view];
-    Rec r[3];
-    int x0 = 0, x1 = 0, y0 = 0, y1 = 0;
-    int64_t A = 0;
-    unsigned st = kStatCount;
-    int cls = kDrop;
-    if (live) {
-        float mv[12];
-#pragma unroll
-        for (int q = 0; q < 12; ++q) mv[q] = pr.mv[q];
-#pragma unroll
-        for (int k = 0; k < 3; ++k)
-            r[k] = make_rec(to_clip(mv, p.v[3 * k], p.v[3 * k + 1], p.v[3 * k + 2], vw.fx, vw.fy), vw);
-        cls = classify(f, r, vw, x0, x1, y0, y1, A, st);
-    }
-    const uint64_t id = pr.base + t;
-    q1_append<RAY>(f, cls == kQueue, (uint32_t)(max(x1 - x0 + 1, 0) * max(y1 - y0 + 1, 0)), id, pidx, mesh, t);
-    if (cls == kSmall) {
-        const int X[3] = {r[0].X, r[1].X, r[2].X}, Y[3] = {r[0].Y, r[1].Y, r[2].Y};
-        const float iz[3] = {r[0].iz, r[1].iz, r[2].iz};
-        raster_small(X, Y, iz, A, x0, x1, y0, y1, id, vw.vis, vw.W);
-    }
-    if (f.stats && live) {
-        stat_add(f, kStatIn, 1);
-        if (st != kStatCount) stat_add(f, st, 1);
-        if (cls == kSmall) stat_add(f, kStatS1, 1);
-    }
-}
-
-// (the fused kernel serves the no-allocation entry point, which has no
-// ray-cast mode)
-__device__ __forceinline__ void exact_body(const FrameDev &f, uint2 e, bool live) {
-    Tri9 p;
-    exact_gather(f, e, live, p);
-    exact_compute<false>(f, e, live, p);
-}
-
-// Out-of-line copy for the fused cull kernel (no survivor bitmap), which
-// runs the exact path itself.
-__device__ __noinline__ void exact_survivor(const FrameDev *f, uint2 e, bool live) { exact_body(*f, e, live); }
-
 // ----------------------------------------------------------- the kernel --
 namespace s1 {
 constexpr int kConsumerWarps = 8;
@@ -383,7 +301,6 @@ constexpr int kThreads = kConsumers + 32;            // + one producer warp
 constexpr int kMaxTpt = 4;                           // triangles per consumer per item
 constexpr int kItem = kConsumers * kMaxTpt;          // 1024 triangles, 12 KB of index triples
 constexpr int kSlots = 4;
-constexpr int kQueue = 64;                           // per-warp survivors (fused kernel)
 constexpr int kMaxPairs = 64;                        // pairs of one segment (pairs_per_segment <= 64)
 constexpr int kCullBlocks = 3;                       // cull blocks per SM: 72 registers a thread (at 4 blocks
                                                      // and 56 registers the four-triangle cull spills)
@@ -396,27 +313,26 @@ struct Desc {
     uint32_t mesh, pair0, npairs;
 };
 
-template <bool INST, bool FUSED>
+template <bool INST>
 struct Smem {
     uint32_t idx[kSlots][3 * kItem + 4];             // index triples, or packed index bits (+1 word read ahead)
     FastPair fp[kSlots][INST ? kMaxPairs : 1];
     MeshDev mesh[kSlots];
     Desc desc[kSlots];
     uint64_t full[kSlots], empty[kSlots];
-    uint2 wq[FUSED ? kConsumerWarps : 1][FUSED ? kQueue : 1];   // (triangle, pair) survivors
 };
 }  // namespace s1
 
-template <bool INST, bool FUSED>
-size_t stage1_smem_bytes() { return sizeof(s1::Smem<INST, FUSED>); }
+template <bool INST>
+size_t stage1_smem_bytes() { return sizeof(s1::Smem<INST>); }
 
 // Producer warp: work grabs (Section 4.1 "Looping Through Batches": a
 // global counter hands out items until all triangles are done; the counter
 // is read one grab ahead), the forward search for the item's segment, the
 // item's pair constants, and the TMA copy of its index triples.  Items
 // [rd.b0, rd.b1) form round r of the frame.
-template <bool INST, bool FUSED, bool COMP>
-__device__ __forceinline__ void stage1_producer(const FrameDev &f, s1::Smem<INST, FUSED> &S, const RoundDev &rd,
+template <bool INST, bool COMP>
+__device__ __forceinline__ void stage1_producer(const FrameDev &f, s1::Smem<INST> &S, const RoundDev &rd,
                                                 uint32_t r, int n_segs, uint64_t per_item, uint32_t G) {
     using namespace s1;
     const int lane = threadIdx.x & 31;
@@ -969,21 +885,17 @@ __device__ __forceinline__ void cull_instanced(const FrameDev &f, const uint32_t
 // Persistent stage-1 cull kernel, round r of the frame.  Consumers read
 // index words from shared memory and position floats from global memory,
 // then run the conservative tiny-triangle cull for every pair of the item
-// (single-pair items: four consecutive triangles a lane, cull_quads;
-// instanced items: two a lane, looped over the pairs).  The warp's
-// decisions are stored as words of the survivor bitmap (32 consecutive
-// triangles of one pair a word), which k_stage1_exact works through
-// afterwards; the cull stays free of the exact path's registers.  The FUSED form (no
-// bitmap) queues the survivors per warp and runs the exact path itself,
-// 32 at a time.  INST blocks loop over many pairs (Section 4.5, extended to
-// several views): a triangle's data is loaded once for all of them.
-template <bool INST, bool FUSED, bool COMP, bool NEAR = true>
-__global__ void __launch_bounds__(s1::kThreads, (FUSED || INST) ? 3 : s1::kCullBlocks)
+// (cull_quads, cull_instanced).  The warp's decisions are stored as words of
+// the survivor bitmap (32 consecutive triangles of one pair a word), which
+// k_stage1_exact works through afterwards; the cull stays free of the exact
+// path's registers.  INST blocks loop over many pairs (Section 4.5, extended
+// to several views): a triangle's data is loaded once for all of them.
+template <bool INST, bool COMP, bool NEAR>
+__global__ void __launch_bounds__(s1::kThreads, s1::kCullBlocks)
     k_stage1(const __grid_constant__ FrameDev f, uint32_t r) {
-    static_assert(!(FUSED && COMP), "the fused kernel reads uncompressed meshes only");
     using namespace s1;
     extern __shared__ __align__(128) unsigned char smem_raw[];
-    Smem<INST, FUSED> &S = *reinterpret_cast<Smem<INST, FUSED> *>(smem_raw);
+    Smem<INST> &S = *reinterpret_cast<Smem<INST> *>(smem_raw);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const RoundDev rd = f.rounds[r];
     const int n_segs = (int)f.hdr->n_segs;
@@ -1001,13 +913,10 @@ __global__ void __launch_bounds__(s1::kThreads, (FUSED || INST) ? 3 : s1::kCullB
     __syncthreads();
 
     if (warp == kConsumerWarps) {
-        stage1_producer<INST, FUSED, COMP>(f, S, rd, r, n_segs, per_item, G);
+        stage1_producer<INST, COMP>(f, S, rd, r, n_segs, per_item, G);
         return;
     }
 
-    uint2 *wq = S.wq[FUSED ? warp : 0];
-    const unsigned lt_mask = (1u << lane) - 1u;
-    int qn = 0;
     for (int j = 0;; ++j) {
         const int slot = j % kSlots;
         if (!mbar_wait(&S.full[slot], (j / kSlots) & 1u)) {
@@ -1018,61 +927,10 @@ __global__ void __launch_bounds__(s1::kThreads, (FUSED || INST) ? 3 : s1::kCullB
         if (d.b >= rd.b1) break;
         const MeshDev &mesh = S.mesh[slot];   // read in place: the slot is ours until we release it
         const uint32_t *idx = S.idx[slot];
-        // index bound as a 32-bit compare: every uint32 index is below V >= 2^32
-        const bool all_valid = mesh.V > 0xFFFFFFFFull;
-        const uint32_t v32 = (uint32_t)mesh.V;
-        const uint32_t np = INST ? d.npairs : 1u;
-        if (!FUSED) {
-            if constexpr (!INST) {
-                cull_quads<NEAR, COMP>(f, idx, S.fp[slot][0], mesh, d, tpt, warp, lane);
-            } else {
-                cull_instanced<NEAR, COMP>(f, idx, S.fp[slot], mesh, d, np, tpt, warp, lane);
-            }
-        } else
-        for (uint32_t k = 0; k < tpt; ++k) {          // uniform trip count: the warp stays converged
-            // three index words from shared memory, nine position floats from
-            // global memory; an index >= V skips the triangle (reported when checking)
-            const uint32_t lt = k * kConsumers + tid;
-            bool valid = lt < d.n;
-            uint32_t i0 = 0, i1 = 0, i2 = 0;
-            if (valid) {
-                i0 = idx[3 * lt]; i1 = idx[3 * lt + 1]; i2 = idx[3 * lt + 2];
-                if (i0 >= mesh.V || i1 >= mesh.V || i2 >= mesh.V) {
-                    if (f.check) atomicOr(f.err, kErrIndex);
-                    valid = false;
-                }
-            }
-            Tri9 p;
-            if (valid) {
-                const float *q0 = mesh.pos + 3 * (uint64_t)i0, *q1 = mesh.pos + 3 * (uint64_t)i1,
-                            *q2 = mesh.pos + 3 * (uint64_t)i2;
-                p.v[0] = __ldg(q0); p.v[1] = __ldg(q0 + 1); p.v[2] = __ldg(q0 + 2);
-                p.v[3] = __ldg(q1); p.v[4] = __ldg(q1 + 1); p.v[5] = __ldg(q1 + 2);
-                p.v[6] = __ldg(q2); p.v[7] = __ldg(q2 + 1); p.v[8] = __ldg(q2 + 2);
-            } else {
-#pragma unroll
-                for (int c = 0; c < 9; ++c) p.v[c] = 0.0f;
-            }
-            for (uint32_t pi = 0; pi < np; ++pi) {
-                const bool live = valid && !fast_cull(S.fp[slot][pi], p);
-                if (f.stats && valid && !live) stat_add(f, kStatIn, 1), stat_add(f, kStatTiny, 1);
-                const unsigned m = __ballot_sync(0xffffffffu, live);
-                if (m) {                               // fused: queue the survivors, run 32 at a time
-                    if (f.stats && live) stat_add(f, kStatFast, 1);
-                    if (live) wq[qn + __popc(m & lt_mask)] = make_uint2((uint32_t)(d.t0 + lt), d.pair0 + pi);
-                    qn += __popc(m);
-                    __syncwarp();
-                    if (qn >= 32) {
-                        qn -= 32;
-                        exact_survivor(&f, wq[qn + lane], true);
-                        __syncwarp();
-                    }
-                }
-            }
-        }
+        if constexpr (INST) cull_instanced<NEAR, COMP>(f, idx, S.fp[slot], mesh, d, d.npairs, tpt, warp, lane);
+        else cull_quads<NEAR, COMP>(f, idx, S.fp[slot][0], mesh, d, tpt, warp, lane);
         // the slot is free once every consumer warp is done with it
         __syncwarp();
         if (lane == 0) mbar_arrive(&S.empty[slot]);
     }
-    if (FUSED && qn > 0) exact_survivor(&f, wq[lane < qn ? lane : 0], lane < qn);
 }

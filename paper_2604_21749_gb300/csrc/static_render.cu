@@ -13,6 +13,7 @@
 #include <cstring>
 #include <mutex>
 
+#include "cull_constants.h"
 #include "curast.h"
 #include "internal.h"
 
@@ -21,7 +22,12 @@ namespace {
 
 constexpr int kStaticMaxInstances = CURAST_STATIC_MAX_INSTANCES;
 constexpr uint64_t kStaticQ1 = 1ull << 16;    // queue-1 entries (16 B each); overflow is rasterized in place
-constexpr uint64_t kStaticQ2 = 1ull << 14;    // queue-2 tile parts (56 B each); overflow likewise
+constexpr uint64_t kStaticQ2 = 1ull << 14;    // queue-2 tile parts (64 B each); overflow likewise
+constexpr int kBoundBlocks = 304;             // partial bounds of the positions
+constexpr uint64_t kItem = 1024;              // triangles of a stage-1 work item
+// A frame of fewer (triangle, instance)s than this takes the exact path for all of them: finding the mesh's
+// bounds would take longer than it saves.
+constexpr uint64_t kCullFrom = 1ull << 17;
 
 constexpr size_t al(size_t x) { return (x + 255) / 256 * 256; }
 constexpr size_t kOffHdr = 0;
@@ -29,9 +35,10 @@ constexpr size_t kOffView = al(kOffHdr + sizeof(FrameHdr));
 constexpr size_t kOffMesh = al(kOffView + sizeof(ViewDev));
 constexpr size_t kOffSeg = al(kOffMesh + sizeof(MeshDev));
 constexpr size_t kOffRound = al(kOffSeg + sizeof(SegDev));
-constexpr size_t kOffCtr = al(kOffRound + sizeof(RoundDev));
+constexpr size_t kOffCtr = al(kOffRound + kMaxRounds * sizeof(RoundDev));
 constexpr size_t kOffErr = al(kOffCtr + sizeof(Counters));
-constexpr size_t kOffPairs = al(kOffErr + sizeof(unsigned));
+constexpr size_t kOffPart = al(kOffErr + sizeof(unsigned));                  // 6 floats a block
+constexpr size_t kOffPairs = al(kOffPart + kBoundBlocks * 6 * sizeof(float));
 constexpr size_t kOffQ1 = al(kOffPairs + kStaticMaxInstances * sizeof(PairDev));
 constexpr size_t kOffQ2 = al(kOffQ1 + kStaticQ1 * sizeof(Q1Entry));
 constexpr size_t kScratchBytes = al(kOffQ2 + kStaticQ2 * sizeof(Q2Entry));   // about 2 MB
@@ -40,47 +47,137 @@ constexpr size_t kScratchBytes = al(kOffQ2 + kStaticQ2 * sizeof(Q2Entry));   // 
 // copy of it until the process exits.
 static __device__ __align__(256) unsigned char g_static_scratch[kScratchBytes];
 
+// The survivor bitmap of a stage-1 round lies in queue 2's memory, which stage
+// 2 fills only after the last round: 8.4 M (triangle, instance)s a round.
+constexpr uint64_t kBitmapWords = kStaticQ2 * sizeof(Q2Entry) / 4;
+
 // Everything a frame needs, passed by value to the one-block set-up kernel.
 struct StaticFrame {
     FrameHdr hdr;
     ViewDev view;
     MeshDev mesh;
     SegDev seg;
-    RoundDev round;
+    uint64_t round_items;    // work items of a round
     int n;
+    int cull;                // 1: the mesh's bounds are being found
     float mv[kStaticMaxInstances][12];
     uint64_t base[kStaticMaxInstances];
 };
 
+// Clears the buffer and, for the cull, leaves each block's bounds of its share
+// of the positions in the scratch.  (A NaN is kept: it makes the bounds
+// unusable.)
+__global__ void __launch_bounds__(256) k_static_begin(uint64_t *vis, uint64_t n, const float *pos, uint64_t V) {
+    const uint64_t stride = (uint64_t)gridDim.x * 256, first = (uint64_t)blockIdx.x * 256 + threadIdx.x;
+    if ((reinterpret_cast<uintptr_t>(vis) & 15) == 0) {
+        ulonglong2 *v2 = reinterpret_cast<ulonglong2 *>(vis);
+        for (uint64_t k = first; k < n / 2; k += stride) v2[k] = make_ulonglong2(kEmpty, kEmpty);
+        if (first == 0 && (n & 1)) vis[n - 1] = kEmpty;
+    } else {
+        for (uint64_t k = first; k < n; k += stride) vis[k] = kEmpty;
+    }
+    if (!pos) return;
+    float lo[3] = {INFINITY, INFINITY, INFINITY}, hi[3] = {-INFINITY, -INFINITY, -INFINITY};
+    bool nan = false;
+    for (uint64_t i = first; i < V; i += stride)
+        for (int k = 0; k < 3; ++k) {
+            const float v = pos[3 * i + k];
+            lo[k] = fminf(lo[k], v);
+            hi[k] = fmaxf(hi[k], v);
+            nan |= v != v;
+        }
+    __shared__ float part[8][6];
+    nan = __syncthreads_or(nan);
+    for (int k = 0; k < 3; ++k)
+        for (int o = 16; o > 0; o >>= 1) {
+            lo[k] = fminf(lo[k], __shfl_xor_sync(0xffffffffu, lo[k], o));
+            hi[k] = fmaxf(hi[k], __shfl_xor_sync(0xffffffffu, hi[k], o));
+        }
+    if ((threadIdx.x & 31) == 0)
+        for (int k = 0; k < 3; ++k) part[threadIdx.x >> 5][k] = lo[k], part[threadIdx.x >> 5][3 + k] = hi[k];
+    __syncthreads();
+    if (threadIdx.x < 6) {
+        float v = part[0][threadIdx.x];
+        for (int w = 1; w < 8; ++w) v = threadIdx.x < 3 ? fminf(v, part[w][threadIdx.x]) : fmaxf(v, part[w][threadIdx.x]);
+        reinterpret_cast<float *>(g_static_scratch + kOffPart)[6 * blockIdx.x + threadIdx.x] = nan ? NAN : v;
+    }
+}
+
+// Rounds first .. first + kMaxRounds - 1 of the frame, and their work counters.
+// Thread t >= 0 of kMaxRounds.
+__device__ void static_rounds(unsigned char *g, int t, uint64_t first, uint64_t items, uint64_t round_items,
+                              uint64_t item_words) {
+    if (t >= 0 && t < kMaxRounds) {
+        RoundDev r;
+        r.b0 = min((first + t) * round_items, items);
+        r.b1 = min(r.b0 + round_items, items);
+        r.w0 = r.b0 * item_words;
+        r.w1 = r.b1 * item_words;
+        reinterpret_cast<RoundDev *>(g + kOffRound)[t] = r;
+        Counters &c = *reinterpret_cast<Counters *>(g + kOffCtr);
+        c.work[t] = 0;
+        c.xwork[t] = 0;
+    }
+}
+
+__global__ void __launch_bounds__(kMaxRounds) k_static_rounds(uint64_t first, uint64_t items, uint64_t round_items,
+                                                              uint64_t item_words) {
+    static_rounds(g_static_scratch, (int)threadIdx.x, first, items, round_items, item_words);
+}
+
 // Writes the frame tables into the scratch and zeroes its counters (they
 // keep the previous call's values otherwise).
-__global__ void k_static_setup(StaticFrame s) {
+__global__ void __launch_bounds__(256) k_static_setup(const __grid_constant__ StaticFrame s) {
     unsigned char *g = g_static_scratch;
-    const int t = threadIdx.x;
-    if (t < s.n) {
-        PairDev p;
-        for (int q = 0; q < 12; ++q) p.mv[q] = s.mv[t][q];
-        for (int q = 0; q < 12; ++q) p.fn[q] = 0.0f;
-        for (int q = 0; q < 4; ++q) p.fk[q] = 0.0f;
-        for (int q = 0; q < 3; ++q) p.fs[q] = 0.0f;
-        p.nlo = -INFINITY;    // nor a near-plane cull
-        p.wsafe = INFINITY;   // no conservative cull: every triangle takes the exact path
-        p.win = 0.0f;
-        p.base = s.base[t];
-        p.view = 0;
-        p.mesh = 0;
-        reinterpret_cast<PairDev *>(g + kOffPairs)[t] = p;
+    const int t = (int)threadIdx.x, lane = t & 31;
+    unsigned long long *c = reinterpret_cast<unsigned long long *>(g + kOffCtr);
+    for (size_t i = t; i < sizeof(Counters) / sizeof(unsigned long long); i += blockDim.x) c[i] = 0ull;
+    __syncthreads();
+    static_rounds(g, t - 192, 0, s.hdr.n_batches, s.round_items, (uint64_t)s.seg.npairs * 32);
+    // the mesh's bounds, one a warp: NaN or infinite ones turn the cull off
+    __shared__ float bound[6];
+    __shared__ int usable[6];
+    if (s.cull && t < 192) {
+        const int k = t >> 5;
+        const float *part = reinterpret_cast<const float *>(g + kOffPart);
+        float v = k < 3 ? INFINITY : -INFINITY;
+        bool nan = false;
+#pragma unroll 10
+        for (int b = lane; b < kBoundBlocks; b += 32) {
+            const float q = part[6 * b + k];
+            nan |= q != q;
+            v = k < 3 ? fminf(v, q) : fmaxf(v, q);
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            const float q = __shfl_xor_sync(0xffffffffu, v, o);
+            v = k < 3 ? fminf(v, q) : fmaxf(v, q);
+        }
+        nan = __any_sync(0xffffffffu, nan);
+        if (lane == 0) bound[k] = v, usable[k] = !nan && isfinite(v);
     }
-    if (t == 0) {
+    __syncthreads();
+    if (t < 32) {
+        bool bounded = s.cull != 0;
+        double lo[3] = {0.0, 0.0, 0.0}, hi[3] = {0.0, 0.0, 0.0};
+        for (int k = 0; k < 3 && bounded; ++k) lo[k] = bound[k], hi[k] = bound[3 + k];
+        for (int k = 0; k < 6; ++k) bounded = bounded && usable[k];
+        if (t < s.n) {
+            PairDev p;
+            for (int q = 0; q < 12; ++q) p.mv[q] = s.mv[t][q];
+            cull_constants(p, bounded, lo, hi, s.view);
+            p.base = s.base[t];
+            p.view = 0;
+            p.mesh = 0;
+            reinterpret_cast<PairDev *>(g + kOffPairs)[t] = p;
+        }
+    }
+    if (t == 64) {
         *reinterpret_cast<FrameHdr *>(g + kOffHdr) = s.hdr;
         *reinterpret_cast<ViewDev *>(g + kOffView) = s.view;
         *reinterpret_cast<MeshDev *>(g + kOffMesh) = s.mesh;
         *reinterpret_cast<SegDev *>(g + kOffSeg) = s.seg;
-        *reinterpret_cast<RoundDev *>(g + kOffRound) = s.round;
         *reinterpret_cast<unsigned *>(g + kOffErr) = 0u;
     }
-    unsigned long long *c = reinterpret_cast<unsigned long long *>(g + kOffCtr);
-    for (size_t i = t; i < sizeof(Counters) / sizeof(unsigned long long); i += blockDim.x) c[i] = 0ull;
 }
 
 // Per-device set-up: the scratch's device address and the launch shape.
@@ -167,13 +264,14 @@ extern "C" curast_status curast_render_static(const float *pos, uint64_t V, cons
             }
         fr.base[i] = (uint64_t)i * T;
     }
-    const uint64_t per_item = 256ull * 4;
-    fr.hdr.n_batches = T ? (T + per_item - 1) / per_item : 0;
+    const uint64_t items = (T + kItem - 1) / kItem, item_words = (uint64_t)n_instances * (kItem / 32);
+    fr.round_items = kBitmapWords / item_words;
+    const uint64_t rounds = (items + fr.round_items - 1) / fr.round_items;
+    fr.cull = T * (uint64_t)n_instances >= kCullFrom && V > 0;
+    fr.hdr.n_batches = items;
     fr.hdr.n_segs = T ? 1u : 0u;
     fr.hdr.n_views = 1;
-    fr.hdr.n_rounds = 1;
-    fr.round.b0 = 0;                      // one round over every item; no bitmap (fused stage 1)
-    fr.round.b1 = fr.hdr.n_batches;
+    fr.hdr.n_rounds = (uint32_t)(rounds < kMaxRounds ? rounds : kMaxRounds);
     fr.view.fx = proj[0];
     fr.view.fy = proj[5];
     fr.view.nearv = nearv;
@@ -204,7 +302,7 @@ extern "C" curast_status curast_render_static(const float *pos, uint64_t V, cons
     f.q1 = reinterpret_cast<Q1Entry *>(g + kOffQ1);
     f.q2 = reinterpret_cast<Q2Entry *>(g + kOffQ2);
     f.rounds = reinterpret_cast<const RoundDev *>(g + kOffRound);
-    f.bits = nullptr;   // no survivor bitmap: the fused cull kernel runs the exact path itself
+    f.bits = reinterpret_cast<uint32_t *>(g + kOffQ2);   // (stage 2 fills queue 2 after the last round)
     f.ctr = reinterpret_cast<Counters *>(g + kOffCtr);
     f.err = reinterpret_cast<unsigned *>(g + kOffErr);
     f.q1_cap = kStaticQ1;
@@ -214,7 +312,7 @@ extern "C" curast_status curast_render_static(const float *pos, uint64_t V, cons
     f.tile_log2 = 6;
     f.tpt = 4;
     fastdiv_consts(8u * f.tpt, f.g_m, f.g_s);
-    f.group_min = 0;
+    f.group_min = 2;
     f.s3_ray = 0;
     f.check = 1;
     f.stats = 0;
@@ -225,12 +323,21 @@ extern "C" curast_status curast_render_static(const float *pos, uint64_t V, cons
 
     const bool inst = n_instances > 1;
     const int sms = ds->shape.num_sms;
-    k_static_setup<<<1, 32, 0, s>>>(fr);
+    k_static_begin<<<kBoundBlocks, 256, 0, s>>>(vis, (uint64_t)W * (uint64_t)H, fr.cull ? pos : nullptr, V);
     if ((e = cudaGetLastError()) != cudaSuccess) return CURAST_ERR_CUDA;
-    if ((e = launch_clear(vis, (uint64_t)W * (uint64_t)H, s)) != cudaSuccess) return CURAST_ERR_CUDA;
-    if ((e = launch_stage1(f, inst, 1, 0, sms * ds->shape.stage1_blocks_per_sm[inst ? 1 : 0][1], true, s)) !=
-        cudaSuccess)
-        return CURAST_ERR_CUDA;
+    k_static_setup<<<1, 256, 0, s>>>(fr);
+    if ((e = cudaGetLastError()) != cudaSuccess) return CURAST_ERR_CUDA;
+    for (uint64_t r = 0; r < rounds; ++r) {
+        if (r > 0 && r % kMaxRounds == 0) {
+            k_static_rounds<<<1, kMaxRounds, 0, s>>>(r, items, fr.round_items, item_words);
+            if ((e = cudaGetLastError()) != cudaSuccess) return CURAST_ERR_CUDA;
+        }
+        const uint32_t k = (uint32_t)(r % kMaxRounds);
+        if ((e = launch_stage1(f, inst, 0, k, sms * ds->shape.stage1_blocks_per_sm[inst ? 1 : 0][0], fr.cull != 0, s)) !=
+            cudaSuccess)
+            return CURAST_ERR_CUDA;
+        if ((e = launch_stage1_exact(f, k, sms * ds->shape.stage1x_blocks_per_sm, s)) != cudaSuccess) return CURAST_ERR_CUDA;
+    }
     if ((e = launch_stage2(f, sms * ds->shape.stage2_blocks_per_sm, s)) != cudaSuccess) return CURAST_ERR_CUDA;
     if ((e = launch_stage3(f, sms * ds->shape.stage3_blocks_per_sm, s)) != cudaSuccess) return CURAST_ERR_CUDA;
     return CURAST_OK;

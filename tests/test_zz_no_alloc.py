@@ -111,3 +111,39 @@ def test_static_render_stages_2_3_and_queue_overflow():
         got = api.render_static(pos, idx, models, cam.view, cam.proj, cam.W, cam.H)
         torch.cuda.synchronize()
         assert torch.equal(got, want)
+
+
+@pytest.mark.parametrize("n,copies", [(1, 1), (255, 1), (256, 1), (160, 3), (700, 32), (90, 32)])
+def test_static_render_bounds_and_rounds(n, copies):
+    """Below and above the size from which the call finds the mesh's bounds, and
+    more work than one stage-1 round's bitmap holds (31 M (triangle, instance)s
+    against 8.4 M): the context render's words.  NaN and infinite positions turn
+    the cull off: the words are then those of the context's exact path."""
+    import __graft_entry__ as g
+    g.build()
+    from paper_2604_21749_gb300 import api
+    hf = S.heightfield_mesh(n, seed=3)
+    models = []
+    for k in range(copies):
+        m = np.eye(4, dtype=np.float32)
+        m[:3, 3] = (k % 6, 0.02 * k, k // 6)
+        models.append(m)
+    W, H = 501, 333
+    side = 6.0 if copies > 1 else 1.0
+    cam = S.Camera(S.look_at((side / 2, 0.7 * side, -0.3 * side), (side / 2, 0.0, side / 2)),
+                   S.perspective(60.0, W / H, 1e-2, 100.0), W, H)
+    for bad in (None, float("nan"), float("inf")):
+        pos, idx = hf.pos.clone().cuda(), hf.idx.cuda()
+        if bad is not None:
+            pos[pos.shape[0] // 2, 1] = bad
+        r = api.Renderer(0)
+        r.set_config(stage1_exact_all=int(bad is not None))
+        r.upload_mesh(pos, idx)
+        for m in models:
+            r.add_instance(0, m)
+        want = r.render(cam.view, cam.proj, W, H)
+        r.sync()
+        got = api.render_static(pos, idx, models, cam.view, cam.proj, W, H)
+        torch.cuda.synchronize()
+        assert bad is not None or (want != -1).any()
+        assert torch.equal(got, want), f"{int((got != want).sum())} pixels differ, bad vertex {bad}"
