@@ -14,11 +14,13 @@
 // nearly every step for a lane or two.
 #pragma once
 
+
 namespace s1 {
 constexpr int kExactWarps = 20;                      // one block an SM, 96 registers a thread
 constexpr int kExactK = 3;                           // survivors a lane gathers together
 constexpr int kBatch = 32 * kExactK;
 constexpr uint32_t kUnits = 13;                      // units dealt out of one block of the bitmap
+constexpr uint32_t kUnitSurvivors = 128;             // survivors of a unit, about
 constexpr int kDenseBits = 12;                       // words with as many survivors are unpacked by the whole warp
 constexpr uint32_t kSegPx = 2048;                    // pixels whose triangle starts are marked at once
 
@@ -282,19 +284,20 @@ __device__ __forceinline__ void small_raster(const FrameDev &f, s1::SmallBatch<K
 size_t exact_smem_bytes() { return sizeof(s1::ExactWarp) * s1::kExactWarps; }
 
 // The exact kernel, round r, one block of 20 warps an SM.  Warps take the
-// bitmap in units: survivors come in clusters where the view looks closely,
-// and a fixed deal of 32-word chunks to warps left some SMs with twice the
-// average (the full-HD view of a 4.2 M-triangle mesh: 179 us, 106 us now).
-// The SM's share of the first 7/8 of the units is taken from a counter in
-// shared memory, the rest from one in global memory, which evens the SMs out:
-// one global address takes an atomic add every 1.8 ns, too slow for every unit
-// (4-word units of that mesh: 59 of 117 us; 32-word units of the billion-
-// triangle frame: 1.75 ms against 0.91).  A unit is four words (128 triangles
-// of one pair, a 16-byte load) for each of 2^ll lanes, in runs of eight words
-// kUnits runs apart, so that a cluster spreads over several units; 2^ll is the
-// largest of 1 .. 32 that gives every warp twelve units.  Frames too small for
-// any of that deal single words, so that all warps work.  The words of the
-// next unit are in flight while a batch runs.
+// bitmap in units of 1 .. 128 words, a word, two or four for each lane:
+// survivors come in clusters where the view looks closely, and a fixed deal of
+// 32-word chunks to warps left some SMs with twice the average (the full-HD
+// view of a 4.2 M-triangle mesh: 179 us, 105 us now).  A unit holds some 128
+// survivors: with 64 the fetches cost more than the balance gains (75 M
+// triangles compressed: 671 us against 621), with 512 single units last too
+// long (the full-HD view 147 us, a clustered 100 M-triangle view 537 against
+// 397); sparse frames reach 128 words first.  Units of more than eight words
+// are runs of eight kUnits runs apart, so that a cluster spreads over several.
+// The SM's share of the units is taken from a counter in shared memory, the
+// last of them from one in global memory, which evens the SMs out: one global
+// address takes an atomic add every 1.8 ns, too slow for every unit (32-word
+// units of the billion-triangle frame: 1.75 ms against 0.90).  The words of
+// the next unit are in flight while a batch runs.
 template <bool RAY>
 __global__ void __launch_bounds__(32 * s1::kExactWarps, 1)
     k_stage1_exact(const __grid_constant__ FrameDev f, uint32_t r) {
@@ -303,7 +306,8 @@ __global__ void __launch_bounds__(32 * s1::kExactWarps, 1)
     __shared__ uint32_t s_taken;                    // units the SM has taken of its share
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     ExactWarp &S = reinterpret_cast<ExactWarp *>(exact_smem)[warp];
-    if (threadIdx.x == 0) s_taken = 0;
+    __shared__ uint32_t s_sample;                   // survivors among the words sampled
+    if (threadIdx.x == 0) s_taken = s_sample = 0;
     __syncthreads();
     const RoundDev rd = f.rounds[r];
     const uint64_t nwords = rd.w1 - rd.w0;
@@ -311,16 +315,29 @@ __global__ void __launch_bounds__(32 * s1::kExactWarps, 1)
     const uint32_t G = kConsumerWarps * f.tpt;
     const uint64_t per_item = (uint64_t)kConsumers * f.tpt;
     const uint32_t nw = gridDim.x * kExactWarps;
-    const bool quad = nwords >= 16ull * nw;         // 16-byte loads (a round's words are a multiple of 8)
-    int ll = quad ? 5 : 0;
-    while (ll > 0 && nwords >> (ll + 2) < 12ull * nw) --ll;
-    // units of single loads follow one another; larger ones take two lanes a run, kUnits units a block
-    const uint32_t block = ll ? kUnits << (ll + 2) : quad ? 4u : 1u;   // words
-    const uint32_t per_block = ll ? kUnits : 1u;
-    const uint32_t nunits = (uint32_t)((nwords + block - 1) / block) * per_block;   // (at most 2^34 words)
-    const uint64_t lane0 = lane >= 1 << ll ? nwords : ll ? (uint64_t)(lane >> 1) * 8 * kUnits + 4 * (lane & 1) : 0;
-    // the SM's share of the first 7/8 of the units, then whatever is left of the rest
-    const uint32_t shared_out = nunits - nunits / 8;
+    // 2^lw words a unit: some kUnitSurvivors of them, but no fewer units than warps.  How many survivors
+    // there are every block estimates from the same four words in every stretch of nwords / 640 (the cull
+    // would pay 3% for counting them); frames with few words need no estimate.
+    uint64_t units = nw;
+    if (nwords >= 8ull * nw) {
+        const uint64_t q = nwords / 4 * threadIdx.x / blockDim.x;
+        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(f.bits) + q);
+        const uint32_t n = __reduce_add_sync(0xffffffffu, __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w));
+        if (lane == 0 && n) atomicAdd(&s_sample, n);
+        __syncthreads();
+        units = max(units, s_sample * (nwords / (4 * blockDim.x)) / kUnitSurvivors);
+    }
+    const uint64_t per_unit = nwords / units;
+    int lw = 0;
+    while (lw < 7 && per_unit >> (lw + 1) != 0) ++lw;
+    const int wide = max(lw - 5, 0);                // 2^wide words a lane
+    const uint32_t per_block = lw > 3 ? kUnits : 1u;
+    const uint32_t block = per_block << lw;         // words
+    const uint32_t nunits = (uint32_t)((nwords + block - 1) / block) * per_block;   // (a unit is 128 words if many)
+    const uint32_t at = (uint32_t)lane << wide;     // the lane's place in its unit
+    const uint64_t lane0 = at >> lw != 0 ? nwords : (uint64_t)(at >> 3) * 8 * kUnits + (at & 7u);
+    // the SM's share of all units but the last, at most 1/8 of them, then whatever is left of those
+    const uint32_t shared_out = nunits - min(nunits / 8, 2 * nw);
     auto grab = [&]() -> uint32_t {
         const uint32_t u = blockIdx.x + atomicAdd(&s_taken, 1u) * gridDim.x;
         return u < shared_out ? u : shared_out + atomicAdd(&f.ctr->xwork[r], 1u);
@@ -333,12 +350,18 @@ __global__ void __launch_bounds__(32 * s1::kExactWarps, 1)
         const uint32_t unit = __shfl_sync(0xffffffffu, next, 0);
         more = unit < nunits;
         if (lane == 0 && more) next = grab();
-        const uint32_t b = ll ? unit / kUnits : unit;
-        word = lane0 + (uint64_t)b * block + (ll ? 8 * (unit - b * kUnits) : 0u);
+        const uint32_t b = lw > 3 ? unit / kUnits : unit;
+        word = lane0 + (uint64_t)b * block + (lw > 3 ? 8 * (unit - b * kUnits) : 0u);
         uint4 w = make_uint4(0u, 0u, 0u, 0u);
-        if (more && word < nwords) {
-            if (quad) w = __ldcs(reinterpret_cast<const uint4 *>(f.bits + word));
-            else w.x = __ldcs(f.bits + word);
+        if (more && word < nwords) {                // (a round's words are a multiple of 8)
+            if (wide == 0) {
+                w.x = __ldcs(f.bits + word);
+            } else if (wide == 1) {
+                const uint2 v = __ldcs(reinterpret_cast<const uint2 *>(f.bits + word));
+                w.x = v.x; w.y = v.y;
+            } else {
+                w = __ldcs(reinterpret_cast<const uint4 *>(f.bits + word));
+            }
         }
         return w;
     };
