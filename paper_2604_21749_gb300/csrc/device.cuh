@@ -31,6 +31,13 @@ struct ViewDev {             // one view of a frame
 
 struct alignas(16) PairDev { // one (instance, view) pair that survived host culling
     float mv[12];            // rows 0..2 of view * model, FP32 (the exact transform)
+    // its view's numbers the exact path needs (pair_view), in 16-byte words with the transform
+    float fx, fy, nearv, wmin;
+    float sx, sy;            // 256 W/2, 256 H/2: the snap's scale
+    int32_t W, H;
+    uint64_t base;           // global id of the instance's triangle 0
+    uint32_t view;
+    uint32_t mesh;
     // conservative tiny-triangle cull: rows giving X'*w, Y'*w and w with FMA,
     // where X' = X - 1/2 and Y' = Y - 1/2 put the pixel centres on integers;
     // the estimate and the exact snapped position lie at most
@@ -46,10 +53,19 @@ struct alignas(16) PairDev { // one (instance, view) pair that survived host cul
     // near-plane cull: a vertex whose estimated w (the w row) lies below nlo
     // has an exact w below the near plane; -inf disables the test
     float nlo;
-    uint64_t base;           // global id of the instance's triangle 0
-    uint32_t view;
-    uint32_t mesh;
 };
+
+// wmin: 2^-120 or the near plane, whichever is larger (1/w stays finite above).
+__host__ __device__ inline void pair_view(PairDev &p, const ViewDev &v) {
+    p.fx = v.fx;
+    p.fy = v.fy;
+    p.nearv = v.nearv;
+    p.wmin = v.nearv > 0x1p-120f ? v.nearv : 0x1p-120f;
+    p.sx = 256.0f * v.hw;
+    p.sy = 256.0f * v.hh;
+    p.W = v.W;
+    p.H = v.H;
+}
 
 // Constants of the division of 32-bit numbers by a fixed d >= 2 with a
 // multiply-high (Granlund and Montgomery, unsigned division by invariant

@@ -367,6 +367,7 @@ curast_status build_frame(curast_ctx *c, const curast_view *views, int nv, long 
                 p.base = c->base[i];
                 p.view = (uint32_t)v;
                 p.mesh = (uint32_t)m;
+                pair_view(p, c->hv[v]);
                 cull_constants(p, mr.bounded, mr.lo, mr.hi, c->hv[v]);
                 if (c->cfg.stage1_exact_all) p.wsafe = INFINITY, p.nlo = -INFINITY;   // no conservative cull
                 c->near_needed = c->near_needed || may_reach_near(p, mr, cams[v]);

@@ -28,22 +28,21 @@ constexpr uint32_t kSegPx = 2048;                    // pixels whose triangle st
 // loads of neighbouring records touch every bank once.
 struct __align__(16) SmallTri {
     int e0, e1, A;             // edge functions 0 and 1 at the centre of pixel (x0, y0); their sum with edge 2
-    uint32_t d0;               // edge 0 (vertex 1 to 2): dx & 0xFFFF | dy << 16, in subpixels
-    uint32_t d1;               // edge 1 (vertex 2 to 0)
+    int c0, c1;                // edges 0 (vertex 1 to 2) and 1 (2 to 0): dx + 65536 dy, in subpixels.  The sign
+                               // is that of dy, or of dx where dy is 0: negative for a top-left edge.
     float iz[3];               // 1/depth of the vertices
     uint32_t id;               // global id, low word
-    uint32_t idh;              // its 4 high bits | bit 4 + k: edge k is not top-left | view << 8
+    uint32_t idh;              // its 4 high bits | view << 8
     uint32_t at;               // x0 | y0 << 16 of the pixel range
     uint32_t shape;            // its width w | ceil(2^20 / w) << 11
 };
-
 static_assert(sizeof(SmallTri) == 3 * sizeof(uint4), "a record is three 16-byte words");
 
 // Up to 32 K small triangles of one warp, K a lane, and the pixel loop's marks.
 template <int K>
 struct SmallBatch {
     uint4 t[32 * K][3];        // the SmallTri of each slot
-    uint32_t npx[32 * K];      // pixels of its range (0: nothing to rasterize)
+    uint32_t npx[32 * K];    // pixels of its range (0: nothing to rasterize)
     uint32_t list[32 * K];     // triangles with pixels: first pixel of the batch | slot << 20
     uint32_t starts[kSegPx / 32];   // bit i: pixel i of the segment is a triangle's first
 };
@@ -59,26 +58,22 @@ __device__ __forceinline__ uint32_t fastdiv(uint32_t n, uint32_t m, uint32_t sh)
 }
 
 // The record of a front-facing triangle with both extents below 2^14
-// subpixels and at most 1024 pixels, w of them a row, from (x0, y0) on.
-__device__ __forceinline__ void put_small(uint4 (&t)[3], const int (&X)[3], const int (&Y)[3], const float (&iz)[3],
-                                          uint64_t id, uint32_t view, int x0, int y0, uint32_t w) {
+// subpixels, doubled area A and a range of at most 1024 pixels, w a row and h
+// a column, from (x0, y0) on; returns its pixels.
+__device__ __forceinline__ uint32_t put_small(uint4 (&t)[3], const int (&X)[3], const int (&Y)[3], const float (&iz)[3],
+                                              int A, uint64_t id, uint32_t view, int x0, int y0, uint32_t w, uint32_t h) {
     // m = ceil(2^20 / w): the approximate quotient is off by less than 1/w, so its floor is the true one or,
     // where w divides 2^20, perhaps one less
     uint32_t m = (uint32_t)(1048576.0f * rcp_approx((float)w));
     m += m * w < (1u << 20) ? 1u : 0u;
     // edge k runs from vertex k+1 to vertex k+2; (px, py) is the first pixel's centre
     const int px = 256 * x0 + 128, py = 256 * y0 + 128;
-    const int dx0 = X[2] - X[1], dy0 = Y[2] - Y[1], dx1 = X[0] - X[2], dy1 = Y[0] - Y[2], dx2 = X[1] - X[0], dy2 = Y[1] - Y[0];
+    const int dx0 = X[2] - X[1], dy0 = Y[2] - Y[1], dx1 = X[0] - X[2], dy1 = Y[0] - Y[2];
     const int e0 = dx0 * (py - Y[1]) - dy0 * (px - X[1]), e1 = dx1 * (py - Y[2]) - dy1 * (px - X[2]);
-    const uint32_t b0 = (dy0 < 0 || (dy0 == 0 && dx0 < 0)) ? 0u : 16u;
-    const uint32_t b1 = (dy1 < 0 || (dy1 == 0 && dx1 < 0)) ? 0u : 32u;
-    const uint32_t b2 = (dy2 < 0 || (dy2 == 0 && dx2 < 0)) ? 0u : 64u;
-    t[0] = make_uint4((uint32_t)e0, (uint32_t)e1, (uint32_t)(dx1 * dy2 - dx2 * dy1),
-                      ((uint32_t)dx0 & 0xFFFFu) | (uint32_t)dy0 << 16);
-    t[1] = make_uint4(((uint32_t)dx1 & 0xFFFFu) | (uint32_t)dy1 << 16, __float_as_uint(iz[0]), __float_as_uint(iz[1]),
-                      __float_as_uint(iz[2]));
-    t[2] = make_uint4((uint32_t)id, (uint32_t)(id >> 32) | b0 | b1 | b2 | view << 8, (uint32_t)x0 | (uint32_t)y0 << 16,
-                      w | m << 11);
+    t[0] = make_uint4((uint32_t)e0, (uint32_t)e1, (uint32_t)A, (uint32_t)(dx0 + 65536 * dy0));
+    t[1] = make_uint4((uint32_t)(dx1 + 65536 * dy1), __float_as_uint(iz[0]), __float_as_uint(iz[1]), __float_as_uint(iz[2]));
+    t[2] = make_uint4((uint32_t)id, (uint32_t)(id >> 32) | view << 8, (uint32_t)x0 | (uint32_t)y0 << 16, w | m << 11);
+    return w * h;
 }
 
 // Set-up of the survivor in `slot`: its class, and for a small triangle its
@@ -90,12 +85,13 @@ __device__ __forceinline__ void put_small(uint4 (&t)[3], const int (&X)[3], cons
 //     floats rounds to zero only when it is zero; NaN fails both forms; an
 //     infinite 128 w takes the outcodes);
 //   - snap's clamp: inside the guard band |X| < 129 * 8192 * 256 < 2^29, once
-//     1/w is finite; vertices with w < 2^-120 send the triangle to stage 2;
+//     1/w is finite; vertices with w < 2^-120 (wmin) send the triangle to
+//     stage 2;
 //   - its two multiplications by H/2 and 256 as one by 128 H (a scaling by a
 //     power of two is exact).
 template <bool RAY>
 __device__ __forceinline__ void exact_setup(const FrameDev &f, s1::ExactWarp &S, int slot, bool live) {
-    uint32_t npx = 0, px = 0;                        // px: pixels of a triangle for stage 2
+    uint32_t npx = 0, px = 0;                      // px: pixels of a triangle for stage 2
     bool queue = false;
     uint64_t id = 0;
     uint2 e = make_uint2(0u, 0u);
@@ -104,63 +100,55 @@ __device__ __forceinline__ void exact_setup(const FrameDev &f, s1::ExactWarp &S,
     if (live) {
         e = S.e[slot];
         const PairDev &pr = f.pairs[e.y];
-        const ViewDev &vw = f.views[pr.view];
+        const float4 *pw = reinterpret_cast<const float4 *>(&pr);
+        const float4 r0 = pw[0], r1 = pw[1], r2 = pw[2], cam = pw[3];
         const float4 pa = reinterpret_cast<const float4 *>(S.t[slot])[0], pb = reinterpret_cast<const float4 *>(S.t[slot])[1];
         const float p[9] = {pa.x, pa.y, pa.z, pa.w, pb.x, pb.y, pb.z, pb.w, __uint_as_float(S.t[slot][2].x)};
         // (scalar: the assembler contracts packed mul.rn.f32x2 / add.rn.f32x2 pairs into FMAs)
-        float mv[12];
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            const float4 row = reinterpret_cast<const float4 *>(pr.mv)[q];
-            mv[4 * q] = row.x; mv[4 * q + 1] = row.y; mv[4 * q + 2] = row.z; mv[4 * q + 3] = row.w;
-        }
+        const float mv[12] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w, r2.x, r2.y, r2.z, r2.w};
         CV c[3];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) c[k] = to_clip(mv, p[3 * k], p[3 * k + 1], p[3 * k + 2], vw.fx, vw.fy);
+        for (int k = 0; k < 3; ++k) c[k] = to_clip(mv, p[3 * k], p[3 * k + 1], p[3 * k + 2], cam.x, cam.y);
         id = pr.base + e.x;
         mesh = f.meshes + pr.mesh;
-        const float wmin = fmaxf(vw.nearv, 7.5231638e-37f);      // 2^-120
         bool inside = true;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             const float gw = __fmul_rn(kGuard, c[k].w);
-            inside &= (c[k].w >= wmin) & (gw < INFINITY) & (fabsf(c[k].x) <= gw) & (fabsf(c[k].y) <= gw);
+            inside &= (c[k].w >= cam.w) & (gw < INFINITY) & (fabsf(c[k].x) <= gw) & (fabsf(c[k].y) <= gw);
         }
         if (!inside) {
             // beyond one clip plane, or to be clipped by stage 2
-            queue = (outcode(c[0], vw.nearv) & outcode(c[1], vw.nearv) & outcode(c[2], vw.nearv)) == 0;
+            queue = (outcode(c[0], cam.z) & outcode(c[1], cam.z) & outcode(c[2], cam.z)) == 0;
             if (!queue) st = kStatClip;
         } else {
+            const float4 scr = pw[4];                // sx, sy, W, H
             int X[3], Y[3];
             float iz[3];
-            const float sx = __fmul_rn(vw.hw, 256.0f), sy = __fmul_rn(vw.hh, 256.0f);
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 iz[k] = __frcp_rn(c[k].w);
-                X[k] = __float2int_rn(__fmul_rn(__fadd_rn(__fmul_rn(c[k].x, iz[k]), 1.0f), sx));
-                Y[k] = __float2int_rn(__fmul_rn(__fadd_rn(__fmul_rn(c[k].y, iz[k]), 1.0f), sy));
+                X[k] = __float2int_rn(__fmul_rn(__fadd_rn(__fmul_rn(c[k].x, iz[k]), 1.0f), scr.x));
+                Y[k] = __float2int_rn(__fmul_rn(__fadd_rn(__fmul_rn(c[k].y, iz[k]), 1.0f), scr.y));
             }
             const int minX = min(X[0], min(X[1], X[2])), maxX = max(X[0], max(X[1], X[2]));
             const int minY = min(Y[0], min(Y[1], Y[2])), maxY = max(Y[0], max(Y[1], Y[2]));
             const bool big = max(maxX - minX, maxY - minY) >= (1 << 14);
             const int ux = X[1] - X[0], uy = Y[1] - Y[0], wx = X[2] - X[0], wy = Y[2] - Y[0];
-            const bool front = big ? (int64_t)ux * wy - (int64_t)wx * uy > 0 : ux * wy - wx * uy > 0;
+            const int A = ux * wy - wx * uy;         // (of no use where big)
+            const bool front = big ? (int64_t)ux * wy - (int64_t)wx * uy > 0 : A > 0;
             int x0, x1, y0, y1;
-            centre_range(minX, maxX, vw.W, x0, x1);
-            centre_range(minY, maxY, vw.H, y0, y1);
+            centre_range(minX, maxX, __float_as_int(scr.z), x0, x1);
+            centre_range(minY, maxY, __float_as_int(scr.w), y0, y1);
             if (!front) {
                 st = kStatBack;
             } else if (x0 > x1 || y0 > y1) {
                 st = kStatTiny;
             } else {
-                const uint32_t w = (uint32_t)(x1 - x0 + 1), n = w * (uint32_t)(y1 - y0 + 1);
-                queue = big || n > f.s1_max;
-                if (queue) {
-                    px = n;
-                } else {
-                    npx = n;
-                    put_small(S.t[slot], X, Y, iz, id, pr.view, x0, y0, w);
-                }
+                const uint32_t w = (uint32_t)(x1 - x0 + 1), h = (uint32_t)(y1 - y0 + 1);
+                queue = big || w * h > f.s1_max;
+                if (queue) px = w * h;
+                else npx = put_small(S.t[slot], X, Y, iz, A, id, pr.view, x0, y0, w, h);
             }
         }
     }
@@ -173,7 +161,7 @@ __device__ __forceinline__ void exact_setup(const FrameDev &f, s1::ExactWarp &S,
     }
 }
 
-// The pixels p0 .. p1 - 1 of a batch, 32 a step.  own / at0: the scan of
+// The pixels p0 .. p1 - 1 of a batch, 32 a step.  npx / at0: as in
 // small_raster; first: triangles that start before p0, less one.
 template <int K>
 __device__ __forceinline__ void small_span(const FrameDev &f, s1::SmallBatch<K> &S, const uint32_t (&npx)[K], uint32_t at0,
@@ -203,11 +191,13 @@ __device__ __forceinline__ void small_span(const FrameDev &f, s1::SmallBatch<K> 
             const uint4 ta = t[0], tb = t[1], tc = t[2];
             const uint32_t dy = (k * (tc.w >> 11)) >> 20, dx = k - dy * (tc.w & 2047u);
             // one column changes E_k by -256 dy_k and one row by 256 dx_k
-            const int e0 = (int)ta.x + (int)dy * ((int)(ta.w << 16) >> 8) - (int)dx * (((int)ta.w >> 16) << 8);
-            const int e1 = (int)ta.y + (int)dy * ((int)(tb.x << 16) >> 8) - (int)dx * (((int)tb.x >> 16) << 8);
+            const int X0 = (int)(ta.w << 16) >> 8, X1 = (int)(tb.x << 16) >> 8;
+            const int e0 = (int)ta.x + (int)dy * X0 - (int)dx * (((int)ta.w - (X0 >> 8)) >> 8);
+            const int e1 = (int)ta.y + (int)dy * X1 - (int)dx * (((int)tb.x - (X1 >> 8)) >> 8);
             const int e2 = (int)ta.z - e0 - e1;
-            const int b0 = (tc.y >> 4) & 1, b1 = (tc.y >> 5) & 1, b2 = (tc.y >> 6) & 1;
-            if (((e0 - b0) | (e1 - b1) | (e2 - b2)) < 0) continue;
+            // less 1 where the edge is not top-left: the signs decide; edge 2 is minus the sum of the others
+            if (((e0 - 1 - ((int)ta.w >> 31)) | (e1 - 1 - ((int)tb.x >> 31)) |
+                 (e2 - 1 - (-((int)ta.w + (int)tb.x) >> 31))) < 0) continue;
             const float s = __fadd_rn(__fadd_rn(__fmul_rn(__int2float_rn(e0), __uint_as_float(tb.y)),
                                                 __fmul_rn(__int2float_rn(e1), __uint_as_float(tb.z))),
                                       __fmul_rn(__int2float_rn(e2), __uint_as_float(tb.w)));
@@ -221,21 +211,23 @@ __device__ __forceinline__ void small_span(const FrameDev &f, s1::SmallBatch<K> 
 }
 
 // Rasterizes the small triangles of a batch: slot s holds npx[s] pixels.  The
-// ranges are laid end to end in the order (lane, u); the
-// triangle of pixel i is the last one to start at or before i, found by
-// counting the marked starts up to it.  The range is walked row by row: pixel
-// k of a range of width w is (k mod w, k / w), the division as a multiplication
-// by m = ceil(2^20 / w), exact for k, w <= 1024 (k (m w - 2^20) < 2^20).  The
-// edge functions are int32: both extents are below 2^14 subpixels, so
-// |E| < 2^30 at every visited sample, and E2 = A - E0 - E1 exactly.
+// ranges are laid end to end in the order (lane, u); the triangle of pixel i
+// is the last one to start at or before i, found by counting the marked starts
+// up to it.  A range is walked row by row: pixel k of a range of width w is
+// (k mod w, k / w), the division as a multiplication by m = ceil(2^20 / w),
+// exact for k, w <= 1024 (k (m w - 2^20) < 2^20).  The edge functions are
+// int32: both extents are below 2^14 subpixels, so |E| < 2^30 at every visited
+// sample, and E2 = A - E0 - E1 exactly.  (A lane a 2 x 2 quad, its covered
+// pixels one by one, needs fewer steps but was no faster: 923 us against 905
+// on the billion-triangle frame, 620 against 621 on compressed terrain.)
 // give(want, slot): where the batch holds more than 2 kSegPx pixels, hands
-// over the triangles that start past pixel kSegPx, the lanes' `want`ed ones in
-// lane order, and returns false to those it has no room for (the last ones);
-// nullptr keeps them all.
+// over the triangles that start past pixel kSegPx, the lanes' `want`ed ones
+// in lane order, and returns false to those it has no room for (the last
+// ones); nullptr keeps them all.
 template <int K, class Give>
 __device__ __forceinline__ void small_raster(const FrameDev &f, s1::SmallBatch<K> &S, int lane, Give give) {
     using namespace s1;
-    uint32_t npx[K], own = 0;                        // own: pixels | triangles << 20
+    uint32_t npx[K], own = 0;                      // own: pixels | triangles << 20
 #pragma unroll
     for (int u = 0; u < K; ++u) npx[u] = S.npx[lane + 32 * u];
 #pragma unroll
@@ -287,8 +279,8 @@ size_t exact_smem_bytes() { return sizeof(s1::ExactWarp) * s1::kExactWarps; }
 // bitmap in units of 1 .. 128 words, a word, two or four for each lane:
 // survivors come in clusters where the view looks closely, and a fixed deal of
 // 32-word chunks to warps left some SMs with twice the average (the full-HD
-// view of a 4.2 M-triangle mesh: 179 us, 105 us now).  A unit holds some 128
-// survivors: with 64 the fetches cost more than the balance gains (75 M
+// view of a 4.2 M-triangle mesh: 179 us, 105 us now).  A unit in a cluster
+// holds some 128 survivors: with 64 the fetches cost more than the balance gains (75 M
 // triangles compressed: 671 us against 621), with 512 single units last too
 // long (the full-HD view 147 us, a clustered 100 M-triangle view 537 against
 // 397); sparse frames reach 128 words first.  Units of more than eight words
@@ -306,7 +298,7 @@ __global__ void __launch_bounds__(32 * s1::kExactWarps, 1)
     __shared__ uint32_t s_taken;                    // units the SM has taken of its share
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     ExactWarp &S = reinterpret_cast<ExactWarp *>(exact_smem)[warp];
-    __shared__ uint32_t s_sample;                   // survivors among the words sampled
+    __shared__ uint32_t s_sample;                   // survivors at the places sampled | places with any << 20
     if (threadIdx.x == 0) s_taken = s_sample = 0;
     __syncthreads();
     const RoundDev rd = f.rounds[r];
@@ -315,19 +307,24 @@ __global__ void __launch_bounds__(32 * s1::kExactWarps, 1)
     const uint32_t G = kConsumerWarps * f.tpt;
     const uint64_t per_item = (uint64_t)kConsumers * f.tpt;
     const uint32_t nw = gridDim.x * kExactWarps;
-    // 2^lw words a unit: some kUnitSurvivors of them, but no fewer units than warps.  How many survivors
-    // there are every block estimates from the same four words in every stretch of nwords / 640 (the cull
-    // would pay 3% for counting them); frames with few words need no estimate.
-    uint64_t units = nw;
+    // 2^lw words a unit.  Every block estimates the survivors and their density where there are any from the
+    // same 640 places (the cull would pay 3% for counting them): a unit of kUnitSurvivors at that density,
+    // fewer where an SM would get less than 16 such units, but 16 words where there are twelve of that for
+    // every warp, and not so small that the fetches over empty stretches pile up.  Frames with few words need
+    // no estimate.
+    uint64_t per_unit = nwords / nw;
     if (nwords >= 8ull * nw) {
         const uint64_t q = nwords / 4 * threadIdx.x / blockDim.x;
         const uint4 v = __ldg(reinterpret_cast<const uint4 *>(f.bits) + q);
-        const uint32_t n = __reduce_add_sync(0xffffffffu, __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w));
-        if (lane == 0 && n) atomicAdd(&s_sample, n);
+        const uint32_t n = __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
+        const uint32_t sum = __reduce_add_sync(0xffffffffu, n) | (uint32_t)__popc(__ballot_sync(0xffffffffu, n != 0)) << 20;
+        if (lane == 0 && sum) atomicAdd(&s_sample, sum);
         __syncthreads();
-        units = max(units, s_sample * (nwords / (4 * blockDim.x)) / kUnitSurvivors);
+        const uint32_t bits = max(s_sample & 0xFFFFFu, 1u), places = s_sample >> 20;
+        const uint64_t survivors = bits * (nwords / (4 * blockDim.x));
+        const uint64_t hold = min((uint64_t)kUnitSurvivors, survivors / (16 * gridDim.x));
+        per_unit = max(max(hold * 4 * places / bits, min((uint64_t)16, nwords / (12 * (uint64_t)nw))), nwords / (128 * (uint64_t)nw));
     }
-    const uint64_t per_unit = nwords / units;
     int lw = 0;
     while (lw < 7 && per_unit >> (lw + 1) != 0) ++lw;
     const int wide = max(lw - 5, 0);                // 2^wide words a lane
@@ -408,16 +405,27 @@ __global__ void __launch_bounds__(32 * s1::kExactWarps, 1)
             const int cnt = __popc(m);
             const unsigned dense = __ballot_sync(0xffffffffu, cnt >= kDenseBits);
             if (dense) {
-                // a dense word: its bits a lane each, as many as fit
-                const int l = __ffs(dense) - 1;
-                const uint32_t bits = __shfl_sync(0xffffffffu, m, l), wt = __shfl_sync(0xffffffffu, t0, l),
-                               wp = __shfl_sync(0xffffffffu, pair, l);
-                const bool set = (bits >> lane) & 1u;
-                const int to = n + __popc(bits & lt_mask);
-                if (set && to < kBatch) S.e[to] = make_uint2(wt + lane, wp);
-                const unsigned rest = __ballot_sync(0xffffffffu, set && to >= kBatch);
-                if (lane == l) m = rest;
-                n = min(n + __popc(bits), kBatch);
+                // dense words: a word's bits a lane each, words that surely fit first, then as many bits as fit
+                unsigned left = dense;
+                for (; left != 0 && n + 32 <= kBatch; left &= left - 1) {
+                    const int l = __ffs(left) - 1;
+                    const uint32_t bits = __shfl_sync(0xffffffffu, m, l), wt = __shfl_sync(0xffffffffu, t0, l),
+                                   wp = __shfl_sync(0xffffffffu, pair, l);
+                    if ((bits >> lane) & 1u) S.e[n + __popc(bits & lt_mask)] = make_uint2(wt + lane, wp);
+                    n += __popc(bits);
+                }
+                if (((dense ^ left) >> lane) & 1u) m = 0;
+                if (left != 0 && n < kBatch) {
+                    const int l = __ffs(left) - 1;
+                    const uint32_t bits = __shfl_sync(0xffffffffu, m, l), wt = __shfl_sync(0xffffffffu, t0, l),
+                                   wp = __shfl_sync(0xffffffffu, pair, l);
+                    const bool set = (bits >> lane) & 1u;
+                    const int to = n + __popc(bits & lt_mask);
+                    if (set && to < kBatch) S.e[to] = make_uint2(wt + lane, wp);
+                    const unsigned rest = __ballot_sync(0xffffffffu, set && to >= kBatch);
+                    if (lane == l) m = rest;
+                    n = min(n + __popc(bits), kBatch);
+                }
                 continue;
             }
             // sparse words: every lane appends its first bits, as many as fit

@@ -178,9 +178,11 @@ __global__ void __launch_bounds__(32 * s2::kWarps) k_stage2(const __grid_constan
                 const int ey = max(Y[0], max(Y[1], Y[2])) - min(Y[0], min(Y[1], Y[2]));
                 if (cnt > 1024 || max(ex, ey) >= (1 << 14) || (!e.small && cnt > (int64_t)f.s2_max)) {
                     whole = true;
-                } else if (cnt > 0 && (X[1] - X[0]) * (Y[2] - Y[0]) - (X[2] - X[0]) * (Y[1] - Y[0]) > 0) {
-                    npx = (uint32_t)cnt;
-                    put_small(S.t[lane], X, Y, iz, e.id, view, x0, y0, (uint32_t)(x1 - x0 + 1));
+                } else if (cnt > 0) {
+                    const int A = (X[1] - X[0]) * (Y[2] - Y[0]) - (X[2] - X[0]) * (Y[1] - Y[0]);
+                    if (A > 0)
+                        npx = put_small(S.t[lane], X, Y, iz, A, e.id, view, x0, y0, (uint32_t)(x1 - x0 + 1),
+                                          (uint32_t)(y1 - y0 + 1));
                 }
             } else {
                 clip = per == 1 || clipped_visible(c, &vw);

@@ -168,6 +168,7 @@ __global__ void __launch_bounds__(256) k_static_setup(const __grid_constant__ St
             p.base = s.base[t];
             p.view = 0;
             p.mesh = 0;
+            pair_view(p, s.view);
             reinterpret_cast<PairDev *>(g + kOffPairs)[t] = p;
         }
     }
