@@ -200,6 +200,7 @@ struct FrameDev {
     uint32_t *bits;          // survivor bitmap of the current round
     Counters *ctr;
     unsigned *err;           // sticky error bits, cleared by curast_sync
+    unsigned long long *stamps;   // start times (ns) of the frame's kernels, kStamp*; nullptr: not taken
     uint64_t q1_cap, q2_cap;
     uint32_t s1_max;         // stage-1 bbox pixel limit
     uint32_t s2_max;         // stage-2 bbox pixel limit
@@ -218,7 +219,33 @@ struct FrameDev {
     uint32_t *tile_fill;     // n_tiles: scatter cursors
     uint2 *units;            // (tile, first part in part_sorted): up to 8 parts of one tile
     uint32_t *part_sorted;   // q2_cap: queue-2 indices in tile order
+    uint32_t pdl;            // (host) 1: the stage kernels are launched ahead of their predecessor's end
 };
+
+// Times of the frame's kernels: the starts of the clear, the first cull, the
+// last exact kernel, stages 2 and 3, and the end of stage 3.
+enum Stamp { kStampClear = 0, kStampCull, kStampExact, kStampStage2, kStampStage3, kStampEnd, kStampCount };
+
+__device__ __forceinline__ unsigned long long now_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+// Every stage kernel starts with this: it may have been launched while the
+// kernel before it in the stream still runs, waits here until that one is done
+// and its writes are visible, and lets the next one be launched in turn (which
+// waits for this one here).  stamp: the time it takes, or kStampCount.
+__device__ __forceinline__ void begin_stage(const FrameDev &f, int stamp) {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
+    if (f.stamps && stamp != kStampCount && blockIdx.x == 0 && threadIdx.x == 0) f.stamps[stamp] = now_ns();
+}
+
+// The end of a block of the last kernel.
+__device__ __forceinline__ void end_frame(const FrameDev &f) {
+    if (f.stamps && threadIdx.x == 0) atomicMax(f.stamps + kStampEnd, now_ns());
+}
 
 constexpr unsigned kErrIndex = 1u;     // a vertex index >= V was skipped
 constexpr unsigned kErrTimeout = 2u;   // a bounded wait on a bulk copy gave up

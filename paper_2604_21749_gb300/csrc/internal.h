@@ -19,6 +19,23 @@ struct LaunchShape {
 cudaError_t query_launch_shape(LaunchShape *out, int device);
 
 cudaError_t launch_clear(uint64_t *vis, uint64_t n, cudaStream_t s);
+
+// The start of a frame (k_begin): n16 16-byte words of tables copied from
+// pinned host memory, counters and tile counts zeroed, buffers cleared.
+constexpr int kBeginViews = 8;
+struct BeginArgs {
+    const uint4 *src;
+    uint4 *dst;
+    uint64_t n16;
+    Counters *ctr;
+    uint32_t *tile_cnt;
+    uint32_t n_tiles;
+    int n_vis;
+    unsigned long long *stamps;
+    uint64_t *vis[kBeginViews];
+    uint64_t n[kBeginViews];
+};
+cudaError_t launch_begin(const BeginArgs &a, cudaStream_t s);
 // Stage 1 of round r: the cull kernel, then the exact kernel over the round's
 // bitmap.  near = false launches the cull without its near-plane test (valid
 // when no pair's mesh bounds reach the near plane).

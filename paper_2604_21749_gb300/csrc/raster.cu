@@ -9,18 +9,34 @@ namespace curast {
 // ------------------------------------------------------------------ clear --
 // Section 4.1: the framebuffer starts each frame at the empty word (all
 // ones, larger than any fragment).  16-byte stores, grid-stride.
-__global__ void __launch_bounds__(256) k_clear(uint64_t *vis, uint64_t n) {
-    const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-    uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const bool aligned = (reinterpret_cast<uintptr_t>(vis) & 15) == 0;
-    if (aligned) {
+__device__ __forceinline__ void fill_empty(uint64_t *vis, uint64_t n, uint64_t i, uint64_t stride) {
+    if ((reinterpret_cast<uintptr_t>(vis) & 15) == 0) {
         ulonglong2 *v2 = reinterpret_cast<ulonglong2 *>(vis);
-        const uint64_t n2 = n / 2;
-        for (uint64_t k = i; k < n2; k += stride) v2[k] = make_ulonglong2(kEmpty, kEmpty);
+        for (uint64_t k = i; k < n / 2; k += stride) v2[k] = make_ulonglong2(kEmpty, kEmpty);
         if (i == 0 && (n & 1)) vis[n - 1] = kEmpty;
     } else {
         for (uint64_t k = i; k < n; k += stride) vis[k] = kEmpty;
     }
+}
+
+__global__ void __launch_bounds__(256) k_clear(uint64_t *vis, uint64_t n) {
+    fill_empty(vis, n, (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, (uint64_t)gridDim.x * blockDim.x);
+}
+
+// The start of a frame in one launch: the tables from pinned host memory
+// (read in place), zeroed counters, cleared buffers.  Three copies, a memset,
+// a clear and the events between the stages took more of a small frame than
+// its kernels (131 k triangles on 640x480: 83 us a frame, the kernels 37 us);
+// with this, and each stage launched ahead of its predecessor's end, 46 us.
+__global__ void __launch_bounds__(256) k_begin(const __grid_constant__ BeginArgs a) {
+    const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (uint64_t)gridDim.x * blockDim.x;
+    asm volatile("griddepcontrol.launch_dependents;");
+    if (a.stamps && i == 0)
+        for (unsigned long long k = 0, t = now_ns(); k < kStampCount; ++k) a.stamps[k] = t;
+    for (uint64_t k = i; k < a.n16; k += stride) a.dst[k] = a.src[k];
+    for (uint64_t k = i; k < sizeof(Counters) / 8; k += stride) reinterpret_cast<unsigned long long *>(a.ctr)[k] = 0ull;
+    for (uint64_t k = i; k < a.n_tiles; k += stride) a.tile_cnt[k] = 0u;
+    for (int v = 0; v < a.n_vis; ++v) fill_empty(a.vis[v], a.n[v], i, stride);
 }
 
 // ----------------------------------------------------- whole-triangle path --
@@ -205,6 +221,7 @@ __global__ void __launch_bounds__(256) k_stage3(const __grid_constant__ FrameDev
     __shared__ SubTri part[s3::kGrab];               // x0 .. y1: the range inside the tile, x0 > x1: none
     __shared__ uint32_t s_view[s3::kGrab], s_ray[s3::kGrab];   // s_ray: pair + 1 of a ray-cast part
     __shared__ unsigned long long s_i;
+    begin_stage(f, kStampStage3);
     const unsigned long long total = *((volatile unsigned long long *)&f.ctr->q2_count);
     const unsigned long long n = total < f.q2_cap ? total : f.q2_cap;
     const int ts = 1 << f.tile_log2;
@@ -285,6 +302,7 @@ __global__ void __launch_bounds__(256) k_stage3(const __grid_constant__ FrameDev
         }
         __syncthreads();
     }
+    end_frame(f);
 }
 
 // ------------------------------------------------------- binned stage 3 --
@@ -306,7 +324,8 @@ size_t stage3_tile_smem(uint32_t tile_log2) { return (size_t)8 << (2 * tile_log2
 // (tile, first part) of every tile, ceil(count / kUnitParts) each (their
 // number in ctr->s3_tiles).
 constexpr int kScanThreads = 1024;
-__global__ void __launch_bounds__(kScanThreads) k_bin_scan(FrameDev f) {
+__global__ void __launch_bounds__(kScanThreads) k_bin_scan(const __grid_constant__ FrameDev f) {
+    begin_stage(f, kStampStage3);
     __shared__ uint32_t wsum[kScanThreads / 32], wnu[kScanThreads / 32];
     const uint32_t n = f.n_tiles;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
@@ -354,7 +373,8 @@ __global__ void __launch_bounds__(kScanThreads) k_bin_scan(FrameDev f) {
 }
 
 // Queue-2 part indices into tile order.
-__global__ void __launch_bounds__(256) k_bin_scatter(FrameDev f) {
+__global__ void __launch_bounds__(256) k_bin_scatter(const __grid_constant__ FrameDev f) {
+    begin_stage(f, kStampCount);
     const unsigned long long total = *((volatile unsigned long long *)&f.ctr->q2_count);
     const unsigned long long n = total < f.q2_cap ? total : f.q2_cap;
     for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < n;
@@ -380,7 +400,8 @@ struct PartRec {
 // part's range -- one column, every (256 / ts)-th row -- with the edge
 // functions stepped from row to row; then it writes each of its covered
 // pixels once to the visibility buffer and resets the word.
-__global__ void __launch_bounds__(256) k_stage3_tiles(FrameDev f) {
+__global__ void __launch_bounds__(256) k_stage3_tiles(const __grid_constant__ FrameDev f) {
+    begin_stage(f, kStampCount);
     extern __shared__ __align__(16) unsigned long long tw[];     // the tile's words
     __shared__ PartRec pr[kUnitParts];
     __shared__ unsigned long long s_i;
@@ -483,6 +504,7 @@ __global__ void __launch_bounds__(256) k_stage3_tiles(FrameDev f) {
         }
         __syncthreads();
     }
+    end_frame(f);
 }
 
 // -------------------------------------------------------------- compare --
@@ -590,45 +612,67 @@ cudaError_t launch_clear(uint64_t *vis, uint64_t n, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+cudaError_t launch_begin(const BeginArgs &a, cudaStream_t s) {
+    uint64_t work = a.n16;
+    for (int v = 0; v < a.n_vis; ++v) work = a.n[v] / 2 > work ? a.n[v] / 2 : work;
+    uint64_t blocks = (work + 255) / 256;
+    blocks = blocks < 8 ? 8 : blocks > 4096 ? 4096 : blocks;
+    k_begin<<<(unsigned)blocks, 256, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+// A stage kernel, launched ahead of its predecessor's end where the frame
+// allows it (begin_stage waits).
+template <class... P, class... A>
+static cudaError_t launch_stage(bool pdl, void (*k)(P...), int blocks, int threads, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 cudaError_t launch_stage1(const FrameDev &f, bool instanced, int variant, uint32_t r, int blocks, bool near,
                           cudaStream_t s) {
     const size_t s0 = stage1_smem_bytes<false>(), si = stage1_smem_bytes<true>();
+    const bool p = f.pdl != 0;
     if (instanced) {
-        if (variant == 1 && near) k_stage1<true, true, true><<<blocks, s1::kThreads, si, s>>>(f, r);
-        else if (variant == 1) k_stage1<true, true, false><<<blocks, s1::kThreads, si, s>>>(f, r);
-        else if (near) k_stage1<true, false, true><<<blocks, s1::kThreads, si, s>>>(f, r);
-        else k_stage1<true, false, false><<<blocks, s1::kThreads, si, s>>>(f, r);
-    } else {
-        if (variant == 2) k_stage1_win<<<blocks, s1::kThreads, stage1_win_smem_bytes(), s>>>(f, r);
-        else if (variant == 1 && near) k_stage1<false, true, true><<<blocks, s1::kThreads, s0, s>>>(f, r);
-        else if (variant == 1) k_stage1<false, true, false><<<blocks, s1::kThreads, s0, s>>>(f, r);
-        else if (near) k_stage1<false, false, true><<<blocks, s1::kThreads, s0, s>>>(f, r);
-        else k_stage1<false, false, false><<<blocks, s1::kThreads, s0, s>>>(f, r);
+        if (variant == 1 && near) return launch_stage(p, k_stage1<true, true, true>, blocks, s1::kThreads, si, s, f, r);
+        if (variant == 1) return launch_stage(p, k_stage1<true, true, false>, blocks, s1::kThreads, si, s, f, r);
+        if (near) return launch_stage(p, k_stage1<true, false, true>, blocks, s1::kThreads, si, s, f, r);
+        return launch_stage(p, k_stage1<true, false, false>, blocks, s1::kThreads, si, s, f, r);
     }
-    return cudaGetLastError();
+    if (variant == 2) return launch_stage(p, k_stage1_win, blocks, s1::kThreads, stage1_win_smem_bytes(), s, f, r);
+    if (variant == 1 && near) return launch_stage(p, k_stage1<false, true, true>, blocks, s1::kThreads, s0, s, f, r);
+    if (variant == 1) return launch_stage(p, k_stage1<false, true, false>, blocks, s1::kThreads, s0, s, f, r);
+    if (near) return launch_stage(p, k_stage1<false, false, true>, blocks, s1::kThreads, s0, s, f, r);
+    return launch_stage(p, k_stage1<false, false, false>, blocks, s1::kThreads, s0, s, f, r);
 }
 
 cudaError_t launch_stage1_exact(const FrameDev &f, uint32_t r, int blocks, cudaStream_t s) {
-    if (f.s3_ray) k_stage1_exact<true><<<blocks, 32 * s1::kExactWarps, exact_smem_bytes(), s>>>(f, r);
-    else k_stage1_exact<false><<<blocks, 32 * s1::kExactWarps, exact_smem_bytes(), s>>>(f, r);
-    return cudaGetLastError();
+    if (f.s3_ray) return launch_stage(f.pdl != 0, k_stage1_exact<true>, blocks, 32 * s1::kExactWarps, exact_smem_bytes(), s, f, r);
+    return launch_stage(f.pdl != 0, k_stage1_exact<false>, blocks, 32 * s1::kExactWarps, exact_smem_bytes(), s, f, r);
 }
 
 cudaError_t launch_stage2(const FrameDev &f, int blocks, cudaStream_t s) {
-    k_stage2<<<blocks, 32 * s2::kWarps, 0, s>>>(f);
-    return cudaGetLastError();
+    return launch_stage(f.pdl != 0, k_stage2, blocks, 32 * s2::kWarps, 0, s, f);
 }
 
 cudaError_t launch_stage3(const FrameDev &f, int blocks, cudaStream_t s) {
-    k_stage3<<<blocks, 256, 0, s>>>(f);
-    return cudaGetLastError();
+    return launch_stage(f.pdl != 0, k_stage3, blocks, 256, 0, s, f);
 }
 
 cudaError_t launch_stage3_binned(const FrameDev &f, int scatter_blocks, int tile_blocks, cudaStream_t s) {
-    k_bin_scan<<<1, kScanThreads, 0, s>>>(f);
-    k_bin_scatter<<<scatter_blocks, 256, 0, s>>>(f);
-    k_stage3_tiles<<<tile_blocks, 256, stage3_tile_smem(f.tile_log2), s>>>(f);
-    return cudaGetLastError();
+    cudaError_t e = launch_stage(f.pdl != 0, k_bin_scan, 1, kScanThreads, 0, s, f);
+    if (e == cudaSuccess) e = launch_stage(f.pdl != 0, k_bin_scatter, scatter_blocks, 256, 0, s, f);
+    if (e == cudaSuccess) e = launch_stage(f.pdl != 0, k_stage3_tiles, tile_blocks, 256, stage3_tile_smem(f.tile_log2), s, f);
+    return e;
 }
 
 cudaError_t launch_aabb(const float *pos, uint64_t V, float *scratch, float *out6, cudaStream_t s) {

@@ -207,11 +207,16 @@ struct curast_ctx {
     PinBuf<float> h_inst_mv;
     cudaEvent_t ev_inst_mv = nullptr;
 
-    // frame tables: [hdr | views | segs | pairs], one device and one pinned copy
+    // frame tables: [hdr | views | segs | pairs], one device copy and a ring of pinned ones, so that the host
+    // can prepare frames while earlier ones run (ev_tab: the frame that read the slot is done, or its copy).
+    // A frame captured by the caller keeps its slot: replays read it again.
     DevBuf<unsigned char> d_tab;
-    PinBuf<unsigned char> h_tab;
+    static constexpr int kSlots = 4;
+    PinBuf<unsigned char> h_tab[kSlots];
+    cudaEvent_t ev_tab[kSlots] = {nullptr, nullptr, nullptr, nullptr};
+    bool kept[kSlots] = {false, false, false, false};
+    int slot = 0;
     size_t cap_views = 0, cap_segs = 0, cap_pairs = 0;
-    cudaEvent_t ev_tab = nullptr;
     std::vector<ViewDev> hv;
     std::vector<PairDev> hp;
     std::vector<SegDev> hs;
@@ -233,8 +238,8 @@ struct curast_ctx {
     float *d_aabb = nullptr;              // 256*6 scratch + 6 result
     unsigned long long *d_diff = nullptr;
 
-    cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-    bool ev_recorded = false;
+    unsigned long long *d_stamps = nullptr;   // kStampCount times of the last frame that took them
+    int stamped = -1;                     // its table slot, or -1: none yet
 
     cudaGraphExec_t gexec = nullptr;
     std::vector<uint64_t> gkey;
@@ -480,37 +485,40 @@ size_t off_segs(const curast_ctx *c) { return align_up(kHdrBytes + c->cap_views 
 size_t off_pairs(const curast_ctx *c) { return align_up(off_segs(c) + c->cap_segs * sizeof(SegDev), 256); }
 size_t tab_bytes(const curast_ctx *c) { return off_pairs(c) + c->cap_pairs * sizeof(PairDev); }
 
-curast_status upload_frame(curast_ctx *c, cudaStream_t s) {
+// Fills the next pinned copy of the frame's tables; the frame's first kernel
+// reads it in place.
+curast_status stage_frame(curast_ctx *c, bool capturing) {
     if (c->hv.size() > c->cap_views || c->hs.size() > c->cap_segs || c->hp.size() > c->cap_pairs) {
-        CU(cudaEventSynchronize(c->ev_tab));
+        for (bool k : c->kept)
+            if (k) return CURAST_ERR_CUDA;   // a captured frame writes the tables' present copy
+        for (cudaEvent_t e : c->ev_tab) CU(cudaEventSynchronize(e));
         c->cap_views = std::max<size_t>(c->hv.size(), std::max<size_t>(2 * c->cap_views, 8));
         c->cap_segs = std::max<size_t>(c->hs.size(), std::max<size_t>(2 * c->cap_segs, 256));
         c->cap_pairs = std::max<size_t>(c->hp.size(), std::max<size_t>(2 * c->cap_pairs, 256));
         c->d_tab.release();
-        c->h_tab.release();
         CU(c->d_tab.reserve(tab_bytes(c)));
-        CU(c->h_tab.reserve(tab_bytes(c)));
+        for (auto &h : c->h_tab) CU(h.reserve(tab_bytes(c)));
         invalidate_graph(c);
     }
-    // the pinned staging copy may still feed the previous frame's upload
-    CU(cudaEventSynchronize(c->ev_tab));
-    unsigned char *h = c->h_tab.p;
+    int slot = (c->slot + 1) % curast_ctx::kSlots, left = 0;
+    while (c->kept[slot]) slot = (slot + 1) % curast_ctx::kSlots;   // one is always left
+    for (bool k : c->kept) left += !k;
+    if (capturing && left == 1) return CURAST_ERR_CUDA;
+    c->slot = slot;
+    c->kept[slot] = capturing;
+    // the slot may still feed the frame of four calls ago
+    CU(cudaEventSynchronize(c->ev_tab[c->slot]));
+    unsigned char *h = c->h_tab[c->slot].p;
     std::memcpy(h, &c->hdr, sizeof(FrameHdr));
     std::memcpy(h + kRoundsOff, c->rounds.data(), c->rounds.size() * sizeof(RoundDev));
     std::memcpy(h + off_views(c), c->hv.data(), c->hv.size() * sizeof(ViewDev));
     std::memcpy(h + off_segs(c), c->hs.data(), c->hs.size() * sizeof(SegDev));
     std::memcpy(h + off_pairs(c), c->hp.data(), c->hp.size() * sizeof(PairDev));
-    const size_t n1 = off_views(c) + c->hv.size() * sizeof(ViewDev);
-    CU(cudaMemcpyAsync(c->d_tab.p, h, n1, cudaMemcpyHostToDevice, s));
-    if (!c->hs.empty())
-        CU(cudaMemcpyAsync(c->d_tab.p + off_segs(c), h + off_segs(c), c->hs.size() * sizeof(SegDev),
-                           cudaMemcpyHostToDevice, s));
-    if (!c->hp.empty())
-        CU(cudaMemcpyAsync(c->d_tab.p + off_pairs(c), h + off_pairs(c), c->hp.size() * sizeof(PairDev),
-                           cudaMemcpyHostToDevice, s));
-    CU(cudaEventRecord(c->ev_tab, s));
     return CURAST_OK;
 }
+
+// Bytes of the tables in use (whole 16-byte words).
+size_t used_bytes(const curast_ctx *c) { return align_up(off_pairs(c) + c->hp.size() * sizeof(PairDev), 16); }
 
 FrameDev make_frame_dev(const curast_ctx *c) {
     FrameDev f;
@@ -525,6 +533,8 @@ FrameDev make_frame_dev(const curast_ctx *c) {
     f.bits = c->d_bits.p;
     f.ctr = c->d_ctr;
     f.err = c->d_err;
+    f.stamps = nullptr;
+    f.pdl = 0;
     f.q1_cap = c->cfg.queue1_capacity;
     f.q2_cap = c->cfg.queue2_capacity;
     f.s1_max = c->cfg.stage1_max_pixels;
@@ -550,35 +560,57 @@ FrameDev make_frame_dev(const curast_ctx *c) {
     return f;
 }
 
-// clear (optional) -> reset counters -> stage 1 (cull, exact) -> stage 2 -> stage 3
-curast_status enqueue_stages(curast_ctx *c, bool clear, bool timing, cudaStream_t s) {
-    const FrameDev f = make_frame_dev(c);
+// How a frame's launches are issued: on the caller's stream, on the caller's
+// stream while that is captured (no times, each kernel after its predecessor's
+// end), or into the context's own graph (as captured; the tables are copied
+// before each replay).
+enum class Frame { direct, captured, replayed };
+
+// tables, clear (optional), counters -> stage 1 (cull, exact) -> stage 2 -> stage 3.
+curast_status enqueue_stages(curast_ctx *c, bool clear, Frame how, cudaStream_t s) {
+    FrameDev f = make_frame_dev(c);
     const int sms = c->shape.num_sms;
-    if (timing) CU(cudaEventRecord(c->ev[0], s));
+    BeginArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.ctr = c->d_ctr;
+    if (f.s3_bin) {
+        a.tile_cnt = f.tile_cnt;
+        a.n_tiles = c->n_tiles;
+    }
+    if (how == Frame::direct) {
+        f.pdl = 1;
+        f.stamps = a.stamps = c->d_stamps;
+    }
+    if (how != Frame::replayed) {
+        a.src = reinterpret_cast<const uint4 *>(c->h_tab[c->slot].p);
+        a.dst = reinterpret_cast<uint4 *>(c->d_tab.p);
+        a.n16 = used_bytes(c) / 16;
+    }
     if (clear)
-        for (const ViewDev &v : c->hv) CU(launch_clear(v.vis, (uint64_t)v.W * (uint64_t)v.H, s));
-    CU(cudaMemsetAsync(c->d_ctr, 0, sizeof(Counters), s));
-    if (f.s3_bin && c->n_tiles) CU(cudaMemsetAsync(f.tile_cnt, 0, (size_t)c->n_tiles * sizeof(uint32_t), s));
-    if (timing) CU(cudaEventRecord(c->ev[1], s));
-    // stage 1 round by round: the cull fills the survivor bitmap, the exact
-    // kernel empties it (ev[2] falls after the last round's cull)
+        for (size_t v = 0; v < c->hv.size(); ++v) {
+            const uint64_t n = (uint64_t)c->hv[v].W * (uint64_t)c->hv[v].H;
+            if (v < (size_t)kBeginViews) {
+                a.vis[v] = c->hv[v].vis;
+                a.n[v] = n;
+                a.n_vis = (int)v + 1;
+            } else {
+                CU(launch_clear(c->hv[v].vis, n, s));
+            }
+        }
+    CU(launch_begin(a, s));
+    // stage 1 round by round: the cull fills the survivor bitmap, the exact kernel empties it
     const uint32_t nr = (uint32_t)c->rounds.size();
     for (uint32_t r = 0; r < nr; ++r) {
         const int variant = c->round_comp[r] ? 1 : (!c->instanced && c->cfg.stage1_vertex_reuse ? 2 : 0);
         CU(launch_stage1(f, c->instanced, variant, r, sms * c->shape.stage1_blocks_per_sm[c->instanced ? 1 : 0][variant],
                          c->near_needed, s));
-        if (timing && r + 1 == nr) CU(cudaEventRecord(c->ev[2], s));
         CU(launch_stage1_exact(f, r, sms * c->shape.stage1x_blocks_per_sm, s));
     }
-    if (timing) CU(cudaEventRecord(c->ev[3], s));
     CU(launch_stage2(f, sms * c->shape.stage2_blocks_per_sm, s));
-    if (timing) CU(cudaEventRecord(c->ev[4], s));
     if (f.s3_bin)
         CU(launch_stage3_binned(f, sms * 4, sms * c->shape.stage3t_blocks_per_sm[c->cfg.tile_log2 - 4], s));
     else
         CU(launch_stage3(f, sms * c->shape.stage3_blocks_per_sm, s));
-    if (timing) CU(cudaEventRecord(c->ev[5], s));
-    c->ev_recorded = c->ev_recorded || timing;
     return CURAST_OK;
 }
 
@@ -589,9 +621,20 @@ curast_status render_views(curast_ctx *c, const curast_view *views, int nv, long
     if (st != CURAST_OK) return st;
     st = build_frame(c, views, nv, only_mesh);
     if (st != CURAST_OK) return st;
-    st = upload_frame(c, s);
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CU(cudaStreamIsCapturing(s, &cap));
+    const bool capturing = cap != cudaStreamCaptureStatusNone;
+    st = stage_frame(c, capturing);
     if (st != CURAST_OK) return st;
-    if (!graph) return enqueue_stages(c, clear, true, s);
+    if (!graph) {
+        st = enqueue_stages(c, clear, capturing ? Frame::captured : Frame::direct, s);
+        if (capturing) return st;
+        const curast_status rec = cuda_status(cudaEventRecord(c->ev_tab[c->slot], s));
+        if (st == CURAST_OK) c->stamped = c->slot;
+        return st != CURAST_OK ? st : rec;
+    }
+    CU(cudaMemcpyAsync(c->d_tab.p, c->h_tab[c->slot].p, used_bytes(c), cudaMemcpyHostToDevice, s));
+    if (!capturing) CU(cudaEventRecord(c->ev_tab[c->slot], s));
     std::vector<uint64_t> key = {(uint64_t)nv, (uint64_t)c->instanced, (uint64_t)clear,
                                  (uint64_t)(uintptr_t)c->d_tab.p, (uint64_t)(uintptr_t)c->d_meshes.p,
                                  (uint64_t)(uintptr_t)c->d_bits.p, (uint64_t)c->rounds.size(),
@@ -610,7 +653,7 @@ curast_status render_views(curast_ctx *c, const curast_view *views, int nv, long
         cudaGraph_t gr = nullptr;
         cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            st = enqueue_stages(c, clear, false, cs);
+            st = enqueue_stages(c, clear, Frame::replayed, cs);
             e = cudaStreamEndCapture(cs, &gr);
         }
         if (e == cudaSuccess && st == CURAST_OK) e = cudaGraphInstantiate(&c->gexec, gr, 0);
@@ -824,8 +867,9 @@ curast_status curast_create(curast_ctx **out, int device) {
     if (st == CURAST_OK) st = cuda_status(cudaMemset(c->d_ctr, 0, sizeof(Counters)));
     if (st == CURAST_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&c->d_aabb), (256 * 6 + 6) * sizeof(float)));
     if (st == CURAST_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&c->d_diff), sizeof(unsigned long long)));
-    for (int k = 0; k < 6 && st == CURAST_OK; ++k) st = cuda_status(cudaEventCreate(&c->ev[k]));
-    if (st == CURAST_OK) st = cuda_status(cudaEventCreateWithFlags(&c->ev_tab, cudaEventDisableTiming));
+    if (st == CURAST_OK) st = cuda_status(cudaMalloc(reinterpret_cast<void **>(&c->d_stamps), kStampCount * sizeof(unsigned long long)));
+    for (cudaEvent_t &ev : c->ev_tab)
+        if (st == CURAST_OK) st = cuda_status(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
     if (st == CURAST_OK) st = cuda_status(cudaEventCreateWithFlags(&c->ev_inst_mv, cudaEventDisableTiming));
     if (st == CURAST_OK) st = alloc_queues(c);
     if (st == CURAST_OK) st = cuda_status(c->d_inst.reserve(1));
@@ -848,7 +892,7 @@ void curast_destroy(curast_ctx *c) {
     c->d_inst_mv.release();
     c->h_inst_mv.release();
     c->d_tab.release();
-    c->h_tab.release();
+    for (auto &h : c->h_tab) h.release();
     c->d_q1.release();
     c->d_q2.release();
     c->d_sorted.release();
@@ -859,9 +903,9 @@ void curast_destroy(curast_ctx *c) {
     if (c->d_err) cudaFree(c->d_err);
     if (c->d_aabb) cudaFree(c->d_aabb);
     if (c->d_diff) cudaFree(c->d_diff);
-    for (cudaEvent_t &e : c->ev)
+    if (c->d_stamps) cudaFree(c->d_stamps);
+    for (cudaEvent_t e : c->ev_tab)
         if (e) cudaEventDestroy(e);
-    if (c->ev_tab) cudaEventDestroy(c->ev_tab);
     if (c->ev_inst_mv) cudaEventDestroy(c->ev_inst_mv);
     if (c->aux) cudaStreamDestroy(c->aux);
     delete c;
@@ -1172,10 +1216,13 @@ curast_status curast_last_frame(const curast_ctx *c, curast_frame_info *out) {
 
 curast_status curast_stage_times(curast_ctx *c, float out[5]) {
     if (!c || !out) return CURAST_ERR_INVALID_ARG;
-    if (!c->ev_recorded) return CURAST_ERR_INVALID_ARG;
+    if (c->stamped < 0) return CURAST_ERR_INVALID_ARG;
     DeviceGuard g(c->device);
-    CU(cudaEventSynchronize(c->ev[5]));
-    for (int k = 0; k < 5; ++k) CU(cudaEventElapsedTime(&out[k], c->ev[k], c->ev[k + 1]));
+    CU(cudaEventSynchronize(c->ev_tab[c->stamped]));
+    unsigned long long t[kStampCount];
+    CU(cudaMemcpyAsync(t, c->d_stamps, sizeof(t), cudaMemcpyDeviceToHost, c->aux));
+    CU(cudaStreamSynchronize(c->aux));
+    for (int k = 0; k < 5; ++k) out[k] = t[k + 1] > t[k] ? (float)((double)(t[k + 1] - t[k]) * 1e-6) : 0.0f;
     return CURAST_OK;
 }
 

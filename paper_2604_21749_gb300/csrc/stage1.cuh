@@ -896,6 +896,7 @@ __global__ void __launch_bounds__(s1::kThreads, s1::kCullBlocks)
     using namespace s1;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     Smem<INST> &S = *reinterpret_cast<Smem<INST> *>(smem_raw);
+    begin_stage(f, r == 0 ? kStampCull : kStampCount);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const RoundDev rd = f.rounds[r];
     const int n_segs = (int)f.hdr->n_segs;

@@ -301,6 +301,8 @@ __global__ void __launch_bounds__(32 * s1::kExactWarps, 1)
     __shared__ uint32_t s_sample;                   // survivors at the places sampled | places with any << 20
     if (threadIdx.x == 0) s_taken = s_sample = 0;
     __syncthreads();
+    begin_stage(f, kStampCount);
+    if (f.stamps && blockIdx.x == 0 && threadIdx.x == 0 && r + 1 == f.hdr->n_rounds) f.stamps[kStampExact] = now_ns();
     const RoundDev rd = f.rounds[r];
     const uint64_t nwords = rd.w1 - rd.w0;
     const int n_segs = (int)f.hdr->n_segs;

@@ -328,6 +328,7 @@ __global__ void __launch_bounds__(s1::kThreads, s1w::kBlocks) k_stage1_win(const
     using namespace s1w;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     Smem &S = *reinterpret_cast<Smem *>(smem_raw);
+    begin_stage(f, r == 0 ? kStampCull : kStampCount);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const RoundDev rd = f.rounds[r];
     const int n_segs = (int)f.hdr->n_segs;

@@ -143,6 +143,7 @@ __global__ void __launch_bounds__(32 * s2::kWarps) k_stage2(const __grid_constan
     __shared__ s1::SmallBatch<1> sw[kWarps];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     s1::SmallBatch<1> &S = sw[warp];
+    begin_stage(f, kStampStage2);
     const unsigned long long total = *((volatile unsigned long long *)&f.ctr->q1_count);
     const unsigned long long n = total < f.q1_cap ? total : f.q1_cap;
     const unsigned long long nw = (unsigned long long)gridDim.x * kWarps;

@@ -317,6 +317,10 @@ extern "C" curast_status curast_render_static(const float *pos, uint64_t V, cons
     f.s3_ray = 0;
     f.check = 1;
     f.stats = 0;
+    f.stamps = nullptr;
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capturing) != cudaSuccess) return CURAST_ERR_CUDA;
+    f.pdl = capturing == cudaStreamCaptureStatusNone;
     f.s3_bin = 0;     // stage 3 writes straight to the buffer (no tile bins in the scratch)
     f.n_tiles = 0;
     f.tile_cnt = f.tile_start = f.tile_fill = f.part_sorted = nullptr;
