@@ -66,6 +66,17 @@ struct InstDev {                // an instance of the screen passes
     uint32_t mesh, pad;
 };
 
+// The instances of a scene of at most kFew, as parameters of a screen pass
+// (its own copy of the tables): no upload before the kernel, and no chain of
+// loads in it from a pixel's id to the buffers of its mesh.
+constexpr int kFew = 8;
+struct FewInst {
+    uint64_t base[kFew + 1];    // of instances past the last one: the total
+    uint32_t mesh_id[kFew];
+    float mv[kFew][12];
+    MeshDev mesh[kFew];
+};
+
 struct ShadeArgs {
     const uint64_t *vis;
     int W, H;
@@ -89,14 +100,15 @@ struct ShadeArgs {
     const float *grad_out;
     float *grad_attr;
     float *grad_pos;
+    FewInst few;                // n_inst <= kFew (inst_mv and inst are not read then)
 };
 
-cudaError_t launch_resolve(ShadeArgs a, cudaStream_t s);
+cudaError_t launch_resolve(ShadeArgs &a, cudaStream_t s);
 // a.W, a.H: the super-sampled buffer (ss W x ss H); W, H: the output
 cudaError_t launch_resolve_ss(const ShadeArgs &a, int W, int H, cudaStream_t s);
 // resolve with textures and the 4-ray mip-level choice (Section 4.4)
-cudaError_t launch_resolve_textured(ShadeArgs a, cudaStream_t s);
-cudaError_t launch_interpolate(ShadeArgs a, cudaStream_t s);
+cudaError_t launch_resolve_textured(ShadeArgs &a, cudaStream_t s);
+cudaError_t launch_interpolate(ShadeArgs &a, cudaStream_t s);
 cudaError_t launch_interpolate_backward(const ShadeArgs &a, cudaStream_t s);
 
 }  // namespace curast

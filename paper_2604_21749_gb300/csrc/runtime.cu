@@ -280,33 +280,35 @@ void invalidate_graph(curast_ctx *c) {
     c->gkey.clear();
 }
 
+MeshDev mesh_dev(const MeshRec &r) {
+    MeshDev m{};
+    m.pos = r.pos;
+    m.idx = r.idx;
+    m.rgba = r.rgba;
+    m.V = r.V;
+    m.T = r.T;
+    m.uv = r.uv;
+    m.tex = r.tex;
+    m.tex_log2 = r.tex_log2;
+    if (r.comp) {
+        m.cidx = r.cidx;
+        m.qpos = r.qpos;
+        m.gflag = r.gflag;
+        m.bits = r.bits;
+        m.mask = r.bits >= 32 ? ~0u : (1u << r.bits) - 1u;
+        m.imin = r.imin;
+        for (int a = 0; a < 3; ++a) {
+            m.lo[a] = r.clo[a];
+            m.step[a] = r.cstep[a];
+        }
+    }
+    return m;
+}
+
 curast_status sync_scene(curast_ctx *c, cudaStream_t s) {
     if (c->meshes_dirty) {
         std::vector<MeshDev> md(c->meshes.size());
-        for (size_t i = 0; i < md.size(); ++i) {
-            const MeshRec &r = c->meshes[i];
-            md[i] = MeshDev{};
-            md[i].pos = r.pos;
-            md[i].idx = r.idx;
-            md[i].rgba = r.rgba;
-            md[i].V = r.V;
-            md[i].T = r.T;
-            md[i].uv = r.uv;
-            md[i].tex = r.tex;
-            md[i].tex_log2 = r.tex_log2;
-            if (r.comp) {
-                md[i].cidx = r.cidx;
-                md[i].qpos = r.qpos;
-                md[i].gflag = r.gflag;
-                md[i].bits = r.bits;
-                md[i].mask = r.bits >= 32 ? ~0u : (1u << r.bits) - 1u;
-                md[i].imin = r.imin;
-                for (int a = 0; a < 3; ++a) {
-                    md[i].lo[a] = r.clo[a];
-                    md[i].step[a] = r.cstep[a];
-                }
-            }
-        }
+        for (size_t i = 0; i < md.size(); ++i) md[i] = mesh_dev(c->meshes[i]);
         const bool grow = md.size() > c->d_meshes.cap;
         CU(c->d_meshes.reserve(std::max<size_t>(md.size(), 1)));
         if (grow) invalidate_graph(c);
@@ -687,9 +689,21 @@ curast_status shade_setup(curast_ctx *c, const float *view, const float *proj, i
     if (st != CURAST_OK) return st;
     st = sync_scene(c, s);
     if (st != CURAST_OK) return st;
-    st = upload_inst_mv(c, view, s);
-    if (st != CURAST_OK) return st;
+    const size_t n = c->insts.size();
+    if (n > (size_t)kFew) {
+        st = upload_inst_mv(c, view, s);
+        if (st != CURAST_OK) return st;
+    }
     std::memset(a, 0, sizeof(*a));
+    if (n <= (size_t)kFew) {
+        for (size_t i = 0; i < n; ++i) {
+            a->few.base[i] = c->base[i];
+            a->few.mesh_id[i] = c->insts[i].mesh;
+            a->few.mesh[i] = mesh_dev(c->meshes[c->insts[i].mesh]);
+            model_view(view, c->insts[i].model, a->few.mv[i]);
+        }
+        for (size_t i = n; i <= (size_t)kFew; ++i) a->few.base[i] = c->base[n];
+    }
     a->vis = vis;
     a->W = W;
     a->H = H;
@@ -698,7 +712,7 @@ curast_status shade_setup(curast_ctx *c, const float *view, const float *proj, i
     a->inst_mv = c->d_inst_mv.p;
     a->inst = c->d_inst.p;
     a->meshes = c->d_meshes.p;
-    a->n_inst = (int)c->insts.size();
+    a->n_inst = (int)n;
     return CURAST_OK;
 }
 

@@ -25,17 +25,27 @@ __device__ __forceinline__ float interp3(float b0, float b1, float b2, float c0,
 struct Under {
     uint64_t lo = 1, hi = 0;
     int inst = -1;
-    const MeshDev *mesh = nullptr;
+    const MeshDev *mesh = nullptr;          // (not FEW)
 };
 
 // Section 4.4: the mesh instance owning a global id is found by binary
 // search of the exclusive prefix sum (last instance with base <= id), unless
 // it is the one under the previous pixel.  False for an empty pixel and for an
-// id past the last instance's triangles.
+// id past the last instance's triangles.  FEW: the tables are parameters.
+template <bool FEW>
 __device__ __forceinline__ bool find_instance(const ShadeArgs &a, uint64_t key, Under &u) {
     if (key == kEmpty) return false;
     const uint64_t id = key & kIdMask;
     if (id < u.lo || id >= u.hi) {
+        if (FEW) {
+            if (a.n_inst == 0 || id < a.few.base[0]) return false;
+            int i = 0;
+            while (i + 1 < a.n_inst && a.few.base[i + 1] <= id) ++i;
+            u.inst = i;
+            u.lo = a.few.base[i];
+            u.hi = a.few.base[i + 1];
+            return id < u.hi;
+        }
         int lo = 0, hi = a.n_inst;   // first index with base > id
         while (lo < hi) {
             const int mid = (lo + hi) >> 1;
@@ -50,9 +60,19 @@ __device__ __forceinline__ bool find_instance(const ShadeArgs &a, uint64_t key, 
     return id < u.hi;
 }
 
+template <bool FEW>
+__device__ __forceinline__ const MeshDev &mesh_of(const ShadeArgs &a, const Under &u) {
+    return FEW ? a.few.mesh[u.inst] : *u.mesh;
+}
+
+template <bool FEW>
+__device__ __forceinline__ void model_view_of(const ShadeArgs &a, int inst, float (&mv)[12]) {
+#pragma unroll
+    for (int q = 0; q < 12; ++q) mv[q] = FEW ? a.few.mv[inst][q] : __ldg(a.inst_mv + 12 * (size_t)inst + q);
+}
+
 // Vertex indices of the pixel's triangle; false when one is out of range.
-__device__ __forceinline__ bool pixel_indices(const Under &u, uint64_t key, uint32_t (&vi)[3]) {
-    const MeshDev &m = *u.mesh;
+__device__ __forceinline__ bool pixel_indices(const MeshDev &m, const Under &u, uint64_t key, uint32_t (&vi)[3]) {
     const uint64_t k = 3 * ((key & kIdMask) - u.lo);
     const uint32_t *idx = m.idx;
     if (!m.cidx) {
@@ -67,8 +87,8 @@ __device__ __forceinline__ bool pixel_indices(const Under &u, uint64_t key, uint
 }
 
 // Object-space positions of the three vertices (pos: the caller's, or null).
-__device__ __forceinline__ void pixel_positions(const Under &u, const float *pos, const uint32_t (&vi)[3], float (&p)[9]) {
-    const float *src = pos ? pos : u.mesh->pos;
+__device__ __forceinline__ void pixel_positions(const MeshDev &m, const float *pos, const uint32_t (&vi)[3], float (&p)[9]) {
+    const float *src = pos ? pos : m.pos;
     if (src) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -77,7 +97,7 @@ __device__ __forceinline__ void pixel_positions(const Under &u, const float *pos
         }
     } else {
 #pragma unroll
-        for (int c = 0; c < 3; ++c) mesh_vertex(*u.mesh, vi[c], p[3 * c], p[3 * c + 1], p[3 * c + 2]);
+        for (int c = 0; c < 3; ++c) mesh_vertex(m, vi[c], p[3 * c], p[3 * c + 1], p[3 * c + 2]);
     }
 }
 
@@ -151,20 +171,22 @@ __device__ __forceinline__ void ray_tables(float *rx, float *ry, int x0, int nx,
 // Colours of the samples (x, y0 + k), k < n <= 2, of a W-wide buffer:
 // barycentrics of the pixel-centre ray; 0 where the sample is empty or the
 // mesh has no colours.
+template <bool FEW>
 __device__ __forceinline__ void resolve_pair(const ShadeArgs &a, const uint64_t (&key)[2], float rx, const float *ry,
                                              Under &u, float (&c)[2][4]) {
     uint32_t vi[2][3], q[2][3];
     float p[2][9];
-    const float *mv[2];
+    int inst[2];
     bool ok[2];
 #pragma unroll
     for (int k = 0; k < 2; ++k) {
-        ok[k] = find_instance(a, key[k], u) && u.mesh->rgba;
-        if (ok[k]) ok[k] = pixel_indices(u, key[k], vi[k]);
+        ok[k] = find_instance<FEW>(a, key[k], u) && mesh_of<FEW>(a, u).rgba;
+        if (ok[k]) ok[k] = pixel_indices(mesh_of<FEW>(a, u), u, key[k], vi[k]);
         if (ok[k]) {
-            mv[k] = a.inst_mv + 12 * (size_t)u.inst;
-            pixel_positions(u, nullptr, vi[k], p[k]);
-            const uint32_t *rgba = reinterpret_cast<const uint32_t *>(u.mesh->rgba);
+            const MeshDev &m = mesh_of<FEW>(a, u);
+            inst[k] = u.inst;
+            pixel_positions(m, nullptr, vi[k], p[k]);
+            const uint32_t *rgba = reinterpret_cast<const uint32_t *>(m.rgba);
 #pragma unroll
             for (int v = 0; v < 3; ++v) q[k][v] = __ldg(rgba + vi[k][v]);
         }
@@ -173,13 +195,15 @@ __device__ __forceinline__ void resolve_pair(const ShadeArgs &a, const uint64_t 
     for (int k = 0; k < 2; ++k) {
         c[k][0] = c[k][1] = c[k][2] = c[k][3] = 0.0f;
         if (ok[k]) {
-            float b0, b1, b2;
-            ray_bary(plane_of(mv[k], p[k]), rx, ry[k], b0, b1, b2);
+            float mv[12], b0, b1, b2;
+            model_view_of<FEW>(a, inst[k], mv);
+            ray_bary(plane_of(mv, p[k]), rx, ry[k], b0, b1, b2);
             blend_rgba(b0, b1, b2, q[k], c[k]);
         }
     }
 }
 
+template <bool FEW>
 __global__ void __launch_bounds__(256, 4) k_resolve(const __grid_constant__ ShadeArgs a) {
     using namespace sh;
     __shared__ float rx[32], ry[kTile + 1];
@@ -199,7 +223,7 @@ __global__ void __launch_bounds__(256, 4) k_resolve(const __grid_constant__ Shad
         if (k >= n) break;
         const uint64_t two[2] = {key[k], key[k + 1]};
         float c[2][4];
-        resolve_pair(a, two, rx[lane], ry + ly + k, u, c);
+        resolve_pair<FEW>(a, two, rx[lane], ry + ly + k, u, c);
         store_rgba(a, pix0 + (size_t)k * a.W, c[0]);
         if (k + 1 < n) store_rgba(a, pix0 + (size_t)(k + 1) * a.W, c[1]);
     }
@@ -211,6 +235,7 @@ __global__ void __launch_bounds__(256, 4) k_resolve(const __grid_constant__ Shad
 // colours summed row by row, y outer and x inner, then divided by ss^2.  A
 // block resolves a square of samples as k_resolve does, (32 / ss) outputs a
 // side, keeps their colours in shared memory, and sums each output's there.
+template <bool FEW>
 __global__ void __launch_bounds__(256, 4) k_resolve_ss(const __grid_constant__ ShadeArgs a, int W, int H) {
     using namespace sh;
     __shared__ float rx[32], ry[kTile + 1];
@@ -230,7 +255,7 @@ __global__ void __launch_bounds__(256, 4) k_resolve_ss(const __grid_constant__ S
         if (k >= n) break;
         const uint64_t two[2] = {key[k], key[k + 1]};
         float c[2][4];
-        resolve_pair(a, two, rx[lane], ry + ly + k, u, c);
+        resolve_pair<FEW>(a, two, rx[lane], ry + ly + k, u, c);
         col[ly + k][lane] = make_float4(c[0][0], c[0][1], c[0][2], c[0][3]);
         col[ly + k + 1][lane] = make_float4(c[1][0], c[1][1], c[1][2], c[1][3]);
     }
@@ -266,6 +291,7 @@ __global__ void __launch_bounds__(256, 4) k_resolve_ss(const __grid_constant__ S
 // nearest texel of that level at the pixel's own uv (column floor(u s), row
 // floor(v s), s the level's side, clamped to it), c = byte / 255.  Pixels of
 // meshes without a texture take the vertex colours of k_resolve.
+template <bool FEW>
 __global__ void __launch_bounds__(256) k_resolve_tex(const __grid_constant__ ShadeArgs a) {
     using namespace sh;
     __shared__ float rx[33], ry[kTile + 1];
@@ -286,11 +312,17 @@ __global__ void __launch_bounds__(256) k_resolve_tex(const __grid_constant__ Sha
         float c[4] = {0.0f, 0.0f, 0.0f, 0.0f};
         int lev = 255;
         uint32_t vi[3];
-        if (find_instance(a, key[k], u) && (u.mesh->uv || u.mesh->rgba) && pixel_indices(u, key[k], vi)) {
-            float p[9];
-            pixel_positions(u, nullptr, vi, p);
-            const float2 *uv = reinterpret_cast<const float2 *>(u.mesh->uv);
-            const float *mv = a.inst_mv + 12 * (size_t)u.inst;
+        bool shown = find_instance<FEW>(a, key[k], u);
+        if (shown) {
+            const MeshDev &m = mesh_of<FEW>(a, u);
+            shown = (m.uv || m.rgba) && pixel_indices(m, u, key[k], vi);
+        }
+        if (shown) {
+            const MeshDev &m = mesh_of<FEW>(a, u);
+            float p[9], mv[12];
+            pixel_positions(m, nullptr, vi, p);
+            const float2 *uv = reinterpret_cast<const float2 *>(m.uv);
+            model_view_of<FEW>(a, u.inst, mv);
             if (uv) {
                 const float2 t0 = __ldg(uv + vi[0]), t1 = __ldg(uv + vi[1]), t2 = __ldg(uv + vi[2]);
                 const Plane P = plane_of(mv, p);
@@ -306,7 +338,7 @@ __global__ void __launch_bounds__(256) k_resolve_tex(const __grid_constant__ Sha
                                            fminf(fminf(us[0], us[1]), fminf(us[2], us[3])));
                 const float dv = __fsub_rn(fmaxf(fmaxf(vs[0], vs[1]), fmaxf(vs[2], vs[3])),
                                            fminf(fminf(vs[0], vs[1]), fminf(vs[2], vs[3])));
-                const int L = u.mesh->tex_log2;
+                const int L = m.tex_log2;
                 const float F = __fmul_rn(fmaxf(du, dv), __int2float_rn(1 << L));
                 lev = 0;
                 if (F >= 1.0f) lev = isfinite(F) ? (int)((__float_as_uint(F) >> 23) & 0xFFu) - 127 : L;
@@ -322,11 +354,11 @@ __global__ void __launch_bounds__(256) k_resolve_tex(const __grid_constant__ Sha
                 if (!(cv >= 0.0f)) cv = 0.0f;
                 if (cv > __fsub_rn(fs, 1.0f)) cv = __fsub_rn(fs, 1.0f);
                 const uint64_t texel = off + (uint64_t)(uint32_t)cv * (uint64_t)side + (uint64_t)(uint32_t)cu;
-                const uint32_t q = __ldg(reinterpret_cast<const uint32_t *>(u.mesh->tex) + texel);
+                const uint32_t q = __ldg(reinterpret_cast<const uint32_t *>(m.tex) + texel);
 #pragma unroll
                 for (int ch = 0; ch < 4; ++ch) c[ch] = byte_unit(q, ch);
             } else {
-                const uint32_t *rgba = reinterpret_cast<const uint32_t *>(u.mesh->rgba);
+                const uint32_t *rgba = reinterpret_cast<const uint32_t *>(m.rgba);
                 const uint32_t q[3] = {__ldg(rgba + vi[0]), __ldg(rgba + vi[1]), __ldg(rgba + vi[2])};
                 float b0, b1, b2;
                 ray_bary(plane_of(mv, p), rx[lane], ry[ly + k], b0, b1, b2);
@@ -342,14 +374,17 @@ __global__ void __launch_bounds__(256) k_resolve_tex(const __grid_constant__ Sha
 // ------------------------------------------------------- interpolate fwd --
 // The pixel's triangle when it belongs to an instance of the interpolated
 // mesh: its vertex indices and positions.
+template <bool FEW>
 __device__ __forceinline__ bool interp_pixel(const ShadeArgs &a, uint64_t key, Under &u, uint32_t (&vi)[3], float (&p)[9]) {
-    if (!find_instance(a, key, u) || u.mesh != a.meshes + a.mesh || !pixel_indices(u, key, vi)) return false;
-    pixel_positions(u, a.pos, vi, p);
+    if (!find_instance<FEW>(a, key, u)) return false;
+    if (FEW ? a.few.mesh_id[u.inst] != a.mesh : u.mesh != a.meshes + a.mesh) return false;
+    if (!pixel_indices(mesh_of<FEW>(a, u), u, key, vi)) return false;
+    pixel_positions(mesh_of<FEW>(a, u), a.pos, vi, p);
     return true;
 }
 
 // CN: the number of channels where it is a usual one, 0: a.C of them.
-template <int CN>
+template <int CN, bool FEW>
 __global__ void __launch_bounds__(256) k_interp_fwd(const __grid_constant__ ShadeArgs a) {
     using namespace sh;
     __shared__ float rx[32], ry[kTile + 1];
@@ -370,18 +405,20 @@ __global__ void __launch_bounds__(256) k_interp_fwd(const __grid_constant__ Shad
         float *o = a.out + (size_t)C * (pix0 + (size_t)k * a.W);
         uint32_t vi[3];
         float p[9];
-        if (interp_pixel(a, key[k], u, vi, p)) {
+        if (interp_pixel<FEW>(a, key[k], u, vi, p)) {
+            float mv[12];
+            model_view_of<FEW>(a, u.inst, mv);
             const float *c0 = a.attr + (size_t)C * vi[0], *c1 = a.attr + (size_t)C * vi[1], *c2 = a.attr + (size_t)C * vi[2];
             float b0, b1, b2;
             if (CN) {                                // (the attributes' loads go out with the positions')
                 float t[3][CN ? CN : 1];
 #pragma unroll
                 for (int ch = 0; ch < CN; ++ch) t[0][ch] = __ldg(c0 + ch), t[1][ch] = __ldg(c1 + ch), t[2][ch] = __ldg(c2 + ch);
-                ray_bary(plane_of(a.inst_mv + 12 * (size_t)u.inst, p), rx[lane], ry[ly + k], b0, b1, b2);
+                ray_bary(plane_of(mv, p), rx[lane], ry[ly + k], b0, b1, b2);
 #pragma unroll
                 for (int ch = 0; ch < CN; ++ch) o[ch] = interp3(b0, b1, b2, t[0][ch], t[1][ch], t[2][ch]);
             } else {
-                ray_bary(plane_of(a.inst_mv + 12 * (size_t)u.inst, p), rx[lane], ry[ly + k], b0, b1, b2);
+                ray_bary(plane_of(mv, p), rx[lane], ry[ly + k], b0, b1, b2);
                 for (int ch = 0; ch < C; ++ch) o[ch] = interp3(b0, b1, b2, __ldg(c0 + ch), __ldg(c1 + ch), __ldg(c2 + ch));
             }
         } else {
@@ -469,6 +506,7 @@ constexpr int kBwdWarps = 8;
 
 struct BwdGroup { uint32_t members, v[3]; };
 
+template <bool FEW>
 __global__ void __launch_bounds__(32 * kBwdWarps) k_interp_bwd(const __grid_constant__ ShadeArgs a) {
     extern __shared__ float bwd_vals[];              // [warp][lane][n | 1]
     __shared__ BwdGroup groups[kBwdWarps][32];
@@ -495,12 +533,11 @@ __global__ void __launch_bounds__(32 * kBwdWarps) k_interp_bwd(const __grid_cons
     const size_t pix = (size_t)y * a.W + x;
     if (x < a.W && y < a.H) {
         key = a.vis[pix];
-        hit = interp_pixel(a, key, u, vi, p);
+        hit = interp_pixel<FEW>(a, key, u, vi, p);
     }
     if (hit) {
         float mv[12];
-#pragma unroll
-        for (int q = 0; q < 12; ++q) mv[q] = __ldg(a.inst_mv + 12 * (size_t)u.inst + q);
+        model_view_of<FEW>(a, u.inst, mv);
         // v0 as double-floats, row by row
         DF v0[3];
 #pragma unroll
@@ -601,40 +638,53 @@ static dim3 pixel_grid(int W, int H, int rows) { return dim3((unsigned)((W + 31)
 
 cudaError_t launch_resolve_ss(const ShadeArgs &a, int W, int H, cudaStream_t s) {
     const int side = 32 / a.ss;
-    k_resolve_ss<<<dim3((unsigned)((W + side - 1) / side), (unsigned)((H + side - 1) / side)), 256, 0, s>>>(a, W, H);
+    const dim3 grid((unsigned)((W + side - 1) / side), (unsigned)((H + side - 1) / side));
+    if (a.n_inst <= kFew) k_resolve_ss<true><<<grid, 256, 0, s>>>(a, W, H);
+    else k_resolve_ss<false><<<grid, 256, 0, s>>>(a, W, H);
     return cudaGetLastError();
 }
 
-cudaError_t launch_resolve(ShadeArgs a, cudaStream_t s) {
-    a.rows = rows_of(a.W, a.H);
-    k_resolve<<<pixel_grid(a.W, a.H, a.rows), 256, 0, s>>>(a);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_resolve_textured(ShadeArgs a, cudaStream_t s) {
-    a.rows = rows_of(a.W, a.H);
-    k_resolve_tex<<<pixel_grid(a.W, a.H, a.rows), 256, 0, s>>>(a);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_interpolate(ShadeArgs a, cudaStream_t s) {
+cudaError_t launch_resolve(ShadeArgs &a, cudaStream_t s) {
     a.rows = rows_of(a.W, a.H);
     const dim3 grid = pixel_grid(a.W, a.H, a.rows);
-    if (a.C == 1) k_interp_fwd<1><<<grid, 256, 0, s>>>(a);
-    else if (a.C == 3) k_interp_fwd<3><<<grid, 256, 0, s>>>(a);
-    else if (a.C == 4) k_interp_fwd<4><<<grid, 256, 0, s>>>(a);
-    else k_interp_fwd<0><<<grid, 256, 0, s>>>(a);
+    if (a.n_inst <= kFew) k_resolve<true><<<grid, 256, 0, s>>>(a);
+    else k_resolve<false><<<grid, 256, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_resolve_textured(ShadeArgs &a, cudaStream_t s) {
+    a.rows = rows_of(a.W, a.H);
+    const dim3 grid = pixel_grid(a.W, a.H, a.rows);
+    if (a.n_inst <= kFew) k_resolve_tex<true><<<grid, 256, 0, s>>>(a);
+    else k_resolve_tex<false><<<grid, 256, 0, s>>>(a);
+    return cudaGetLastError();
+}
+
+template <bool FEW>
+static void interp_fwd(const ShadeArgs &a, dim3 grid, cudaStream_t s) {
+    if (a.C == 1) k_interp_fwd<1, FEW><<<grid, 256, 0, s>>>(a);
+    else if (a.C == 3) k_interp_fwd<3, FEW><<<grid, 256, 0, s>>>(a);
+    else if (a.C == 4) k_interp_fwd<4, FEW><<<grid, 256, 0, s>>>(a);
+    else k_interp_fwd<0, FEW><<<grid, 256, 0, s>>>(a);
+}
+
+cudaError_t launch_interpolate(ShadeArgs &a, cudaStream_t s) {
+    a.rows = rows_of(a.W, a.H);
+    const dim3 grid = pixel_grid(a.W, a.H, a.rows);
+    if (a.n_inst <= kFew) interp_fwd<true>(a, grid, s);
+    else interp_fwd<false>(a, grid, s);
     return cudaGetLastError();
 }
 
 cudaError_t launch_interpolate_backward(const ShadeArgs &a, cudaStream_t s) {
     const int n = (a.grad_pos ? 9 : 0) + (a.grad_attr ? 3 * a.C : 0);
     const size_t smem = (size_t)32 * kBwdWarps * (n | 1) * sizeof(float);
+    void (*k)(ShadeArgs) = a.n_inst <= kFew ? k_interp_bwd<true> : k_interp_bwd<false>;
     if (smem > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_interp_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
-    k_interp_bwd<<<pixel_grid(a.W, a.H, 1), 32 * kBwdWarps, smem, s>>>(a);
+    k<<<pixel_grid(a.W, a.H, 1), 32 * kBwdWarps, smem, s>>>(a);
     return cudaGetLastError();
 }
 

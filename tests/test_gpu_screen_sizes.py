@@ -111,3 +111,38 @@ def test_interpolation(api, n, size, C, want):
         if got is not None:
             assert np.linalg.norm(got.cpu().numpy() - ref) <= 1e-4 * max(np.linalg.norm(ref), 1e-30)
     del keep
+
+
+@pytest.mark.parametrize("n", [1, 7, 8])
+def test_instances_as_parameters(api, n):
+    """Up to eight instances travel as kernel parameters; the same ones
+    followed by others that are out of sight go up as tables: same images."""
+    W, H = 333, 210
+    hf, sp = S.heightfield_mesh(40, seed=4), S.sphere_mesh(16, seed=5)
+    inst = []
+    for k in range(17):
+        m = np.eye(4, dtype=np.float32)
+        m[:3, 3] = (0.7 * (k % 3) - 0.7, 0.05 * k, 0.6 * (k // 3)) if k < n else (0.0, 0.0, -500.0 - 9 * k)
+        inst.append(Instance(k % 2, m))
+    cam = Camera(S.look_at((0.5, 1.6, -1.4), (0.4, 0.0, 0.6)), S.perspective(70.0, W / H, 0.01, 100.0), W, H)
+    uv, tx = S.grid_uv(40).cuda(), S.texture_mip_chain(6, seed=1).cuda()
+    attr = torch.rand((hf.pos.shape[0], 3), generator=torch.Generator().manual_seed(1)).cuda()
+    got = []
+    for count in (n, 17):
+        r = api.Renderer(0)
+        keep = upload(r, Scene([hf, sp], inst[:count], [cam]), compressed=(1,))
+        vis = r.render(cam.view, cam.proj, W, H)
+        out = [vis, *r.resolve(cam.view, cam.proj, vis)]
+        out.append(r.interpolate(0, cam.view, cam.proj, vis, attr))
+        out += r.resolve_ss(cam.view, cam.proj, vis, 3) if W % 3 == 0 and H % 3 == 0 else []
+        r.set_mesh_texture(0, uv, tx, 6)
+        out += r.resolve_textured(cam.view, cam.proj, vis)
+        ga, gp = r.interpolate_backward(0, cam.view, cam.proj, vis, attr, torch.ones((H, W, 3), device="cuda"))
+        got.append((out, ga))
+        r.sync()
+        del keep
+    assert (got[0][0][0] != -1).any() and got[0][0][3].abs().sum() > 0
+    for a, b in zip(got[0][0], got[1][0]):
+        assert torch.equal(a, b)
+    # sums of at most W H terms, nearly all of one sign, in any order
+    torch.testing.assert_close(got[0][1], got[1][1], rtol=2 * W * H * 2.0 ** -24, atol=1e-4)
