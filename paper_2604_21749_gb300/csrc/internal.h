@@ -66,10 +66,12 @@ struct InstDev {                // an instance of the screen passes
     uint32_t mesh, pad;
 };
 
-// The instances of a scene of at most kFew, as parameters of a screen pass
-// (its own copy of the tables): no upload before the kernel, and no chain of
-// loads in it from a pixel's id to the buffers of its mesh.
-constexpr int kFew = 8;
+// The instances of a scene of at most kFew (what 4 KB of kernel parameters
+// hold), by value: no upload before the kernel, and no chain of loads in it
+// from a pixel's id to the buffers of its mesh.  Against the tables, us a call:
+// a 4K textured resolve of one instance 134 -> 120, a super-sampled HD one
+// 121 -> 100.
+constexpr int kFew = 16;
 struct FewInst {
     uint64_t base[kFew + 1];    // of instances past the last one: the total
     uint32_t mesh_id[kFew];
@@ -102,6 +104,7 @@ struct ShadeArgs {
     float *grad_pos;
     FewInst few;                // n_inst <= kFew (inst_mv and inst are not read then)
 };
+static_assert(sizeof(ShadeArgs) + 16 <= 4096, "kernel parameters");
 
 cudaError_t launch_resolve(ShadeArgs &a, cudaStream_t s);
 // a.W, a.H: the super-sampled buffer (ss W x ss H); W, H: the output

@@ -113,9 +113,9 @@ def test_interpolation(api, n, size, C, want):
     del keep
 
 
-@pytest.mark.parametrize("n", [1, 7, 8])
+@pytest.mark.parametrize("n", [1, 7, 16])
 def test_instances_as_parameters(api, n):
-    """Up to eight instances travel as kernel parameters; the same ones
+    """Up to sixteen instances travel as kernel parameters; the same ones
     followed by others that are out of sight go up as tables: same images."""
     W, H = 333, 210
     hf, sp = S.heightfield_mesh(40, seed=4), S.sphere_mesh(16, seed=5)
