@@ -152,18 +152,26 @@ def _check(st: int, what: str):
         raise CurastError(st, what)
 
 
+_Mat = C.c_float * 16
+
+
+# What each call pays before its kernels: matrices copied as bytes, pointers as
+# plain integers (the argument types are declared), the stream handle without
+# a stream object: 0.7 and 0.3 us for a matrix and the stream, 3.3 and 3.2 from
+# Python floats and a stream object; a small resolve 16 us for 31.
 def _mat(m) -> C.Array:
     a = np.ascontiguousarray(np.asarray(m.cpu() if hasattr(m, "cpu") else m, dtype=np.float32)).reshape(16)
-    return (C.c_float * 16)(*[float(x) for x in a])
+    return _Mat.from_buffer_copy(a)
 
 
 def _ptr(t: Optional[torch.Tensor]):
-    return None if t is None else C.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
 
 
 def _stream(stream=None):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _need(t: torch.Tensor, dtype, what: str, device):
@@ -283,8 +291,8 @@ class Renderer:
     def _views(views) -> C.Array:
         arr = (View * len(views))()
         for k, (view, proj, W, H, vis) in enumerate(views):
-            arr[k].view[:] = list(_mat(view))
-            arr[k].proj[:] = list(_mat(proj))
+            arr[k].view = _mat(view)
+            arr[k].proj = _mat(proj)
             arr[k].W, arr[k].H = int(W), int(H)
             arr[k].vis = vis.data_ptr()
         return arr
@@ -445,7 +453,7 @@ def render_static(pos: torch.Tensor, idx: torch.Tensor, models, view, proj, W: i
     else:
         arr = np.ascontiguousarray(np.stack([np.asarray(m, np.float32).reshape(16) for m in models]), np.float32)
         n = arr.shape[0]
-        mats = (C.c_float * (16 * n))(*[float(x) for x in arr.reshape(-1)])
+        mats = (C.c_float * (16 * n)).from_buffer_copy(arr)
     with torch.cuda.device(dev):
         st = stream if stream is not None else torch.cuda.current_stream(dev)
         if st.device != dev:
