@@ -220,18 +220,15 @@ __device__ __forceinline__ bool range_touched(const SubTri &s, int x0, int x1, i
 __global__ void __launch_bounds__(256) k_stage3(const __grid_constant__ FrameDev f) {
     __shared__ SubTri part[s3::kGrab];               // x0 .. y1: the range inside the tile, x0 > x1: none
     __shared__ uint32_t s_view[s3::kGrab], s_ray[s3::kGrab];   // s_ray: pair + 1 of a ray-cast part
-    __shared__ unsigned long long s_i;
+    __shared__ unsigned long long s_next;
     begin_stage(f, kStampStage3);
     const unsigned long long total = *((volatile unsigned long long *)&f.ctr->q2_count);
     const unsigned long long n = total < f.q2_cap ? total : f.q2_cap;
     const int ts = 1 << f.tile_log2;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t per = (uint32_t)max(1ull, min((unsigned long long)s3::kGrab, n / (2ull * gridDim.x)));
-    for (;;) {
-        if (tid == 0) s_i = atomicAdd(&f.ctr->q2_next, (unsigned long long)per);
-        __syncthreads();
-        const unsigned long long i0 = s_i;
-        if (i0 >= n) break;
+    // the first grab is the block's own by its number: no atomic for it, and none for a block without parts
+    for (unsigned long long i0 = (unsigned long long)blockIdx.x * per; i0 < n; i0 = s_next) {
         const int g = (int)min((unsigned long long)per, n - i0);
         if (tid < g) {
             const Q2Entry e = f.q2[i0 + tid];
@@ -300,6 +297,7 @@ __global__ void __launch_bounds__(256) k_stage3(const __grid_constant__ FrameDev
                 }
             }
         }
+        if (tid == 32) s_next = (unsigned long long)gridDim.x * per + atomicAdd(&f.ctr->q2_next, (unsigned long long)per);
         __syncthreads();
     }
     end_frame(f);

@@ -7,23 +7,31 @@
 // 1024 pixels go through the small triangles' pixel loop together; the warp
 // works through the rest one by one, rasterizing sub-triangles of at most
 // s2_max pixels itself and splitting larger ones along tile boundaries into
-// stage-3 parts.
+// stage-3 parts.  A queue shorter than the warps gives each triangle several
+// of them, which share its pixels or tiles.
 #pragma once
 
 namespace s2 {
 constexpr int kWarps = 4;
 constexpr unsigned long long kGrabPx = 2048;
+constexpr unsigned kMaxShare = 16;
+
+// The share of a triangle that a warp has: the k-th of n.
+struct Share { uint32_t k, n; };
 }
 
-// The tiles of [x0, x1] x [y0, y1] as stage-3 parts, with one reservation of
-// queue 2.  RAY: the whole triangle is ray cast, s holds its id alone.  Parts
+// The warp's share of the tiles of [x0, x1] x [y0, y1] as stage-3 parts, with
+// one reservation of queue 2.  RAY: the whole triangle is ray cast, s holds its id alone.  Parts
 // past the queue's capacity are rasterized in place.  Returns their number.
 template <bool RAY>
 __device__ __forceinline__ uint32_t append_parts(const FrameDev &f, const SubTri &s, uint32_t pidx, uint32_t view,
-                                                 const ViewDev &vw, int x0, int x1, int y0, int y1, int lane) {
+                                                 const ViewDev &vw, int x0, int x1, int y0, int y1, int lane,
+                                                 s2::Share sh) {
     const int tl = (int)f.tile_log2, ts = 1 << tl;
     const int tx0 = x0 >> tl, ty0 = y0 >> tl, ntx = (x1 >> tl) - tx0 + 1;
-    const int nt = ntx * ((y1 >> tl) - ty0 + 1);
+    const int all = ntx * ((y1 >> tl) - ty0 + 1);
+    const int each = (all + (int)sh.n - 1) / (int)sh.n, first = each * (int)sh.k, nt = min(each, all - first);
+    if (nt <= 0) return 0;
     unsigned long long base = 0;
     if (lane == 0) base = atomicAdd(&f.ctr->q2_count, (unsigned long long)nt);
     base = __shfl_sync(0xffffffffu, base, 0);
@@ -39,7 +47,7 @@ __device__ __forceinline__ uint32_t append_parts(const FrameDev &f, const SubTri
         w1 = make_uint4((uint32_t)s.Y[1], (uint32_t)s.Y[2], __float_as_uint(s.iz[0]), __float_as_uint(s.iz[1]));
         w2 = make_uint4(__float_as_uint(s.iz[2]), view, (uint32_t)s.id, (uint32_t)(s.id >> 32));
     }
-    int tx = lane % ntx, ty = ty0 + lane / ntx;      // stepped by 32 tiles: sy rows and sx columns
+    int tx = (first + lane) % ntx, ty = ty0 + (first + lane) / ntx;   // stepped by 32 tiles: sy rows and sx columns
     const int sx = 32 % ntx, sy = 32 / ntx;
     for (int k = lane; k < nt; k += 32) {
         const uint32_t ex = (uint32_t)(tx0 + tx), ey = (uint32_t)ty;
@@ -68,19 +76,19 @@ __device__ __forceinline__ uint32_t append_parts(const FrameDev &f, const SubTri
 
 // One sub-triangle by the whole warp.
 __device__ __forceinline__ void stage2_subtri(const FrameDev &f, SubTri &s, uint32_t view, const ViewDev &vw, int lane,
-                                              unsigned long long &n_s2, unsigned long long &n_parts) {
+                                              s2::Share sh, unsigned long long &n_s2, unsigned long long &n_parts) {
     if (!setup_subtri(s, vw.W, vw.H)) return;
     const int64_t cnt = (int64_t)(s.x1 - s.x0 + 1) * (int64_t)(s.y1 - s.y0 + 1);
     if (cnt <= (int64_t)f.s2_max) {
-        raster_range(s, s.x0, s.x1, s.y0, s.y1, lane, 32, vw.vis, vw.W);
-        ++n_s2;
+        raster_range(s, s.x0, s.x1, s.y0, s.y1, lane + 32 * (int)sh.k, 32 * (int)sh.n, vw.vis, vw.W);
+        n_s2 += sh.k == 0;
     } else {
-        n_parts += append_parts<false>(f, s, 0u, view, vw, s.x0, s.x1, s.y0, s.y1, lane);
+        n_parts += append_parts<false>(f, s, 0u, view, vw, s.x0, s.x1, s.y0, s.y1, lane, sh);
     }
 }
 
 // One queued triangle that reaches beyond a plane, by the whole warp.
-__device__ __noinline__ void stage2_clipped(const FrameDev *fp, const Q1Entry *ep, unsigned long long *n_s2,
+__device__ __noinline__ void stage2_clipped(const FrameDev *fp, const Q1Entry *ep, s2::Share sh, unsigned long long *n_s2,
                                             unsigned long long *n_parts) {
     const FrameDev &f = *fp;
     const int lane = threadIdx.x & 31;
@@ -104,16 +112,25 @@ __device__ __noinline__ void stage2_clipped(const FrameDev *fp, const Q1Entry *e
         const int64_t cnt = poly_range(X, Y, np, vw.W, vw.H, x0, x1, y0, y1);
         if (cnt == 0) return;
         if (cnt > (int64_t)f.s2_max) {
-            *n_parts += append_parts<true>(f, s, e.pair, pr.view, vw, x0, x1, y0, y1, lane);
+            *n_parts += append_parts<true>(f, s, e.pair, pr.view, vw, x0, x1, y0, y1, lane, sh);
             return;
         }
     }
     unsigned long long a = 0, b = 0;
-    for (int j = 1; j + 1 < np; ++j) {
+    // sub-triangles dealt out to the shares, or all of them to each
+    const uint32_t m = (uint32_t)np - 2, each = sh.n / m;
+    int j = 1, end = np - 1;
+    if (each > 0) {
+        if (sh.k / each >= m) return;
+        j += (int)(sh.k / each);
+        end = j + 1;
+        sh = {sh.k % each, each};
+    }
+    for (; j < end; ++j) {
         s.X[0] = X[0]; s.X[1] = X[j]; s.X[2] = X[j + 1];
         s.Y[0] = Y[0]; s.Y[1] = Y[j]; s.Y[2] = Y[j + 1];
         s.iz[0] = iz[0]; s.iz[1] = iz[j]; s.iz[2] = iz[j + 1];
-        stage2_subtri(f, s, pr.view, vw, lane, a, b);
+        stage2_subtri(f, s, pr.view, vw, lane, sh, a, b);
     }
     *n_s2 += a;
     *n_parts += b;
@@ -137,7 +154,12 @@ __device__ __noinline__ bool clipped_visible(const CV *c, const ViewDev *vw) {
 // would work long after the others; a short queue is dealt out singly, so that
 // all warps share it.  (A 100 M-triangle view whose queue is half clipped
 // triangles without a pixel and half small ones handed over: 67 us singly,
-// 35 us in sevens.)
+// 35 us in sevens.)  A warp's first grab is its own by its number, so that the
+// ones without any leave at once: one atomic of each of 2432 warps on one
+// counter is 4 us.  A queue of fewer triangles than half the warps gives each
+// to several, up to kMaxShare: the triangles in it are then as a rule the large
+// ones, and a single warp would write thousands of parts (twelve triangles
+// that fill 3840 x 2160: 23 us, 14 shared).
 __global__ void __launch_bounds__(32 * s2::kWarps) k_stage2(const __grid_constant__ FrameDev f) {
     using namespace s2;
     __shared__ s1::SmallBatch<1> sw[kWarps];
@@ -150,11 +172,12 @@ __global__ void __launch_bounds__(32 * s2::kWarps) k_stage2(const __grid_constan
     const unsigned long long fair = max(n / (2 * nw), n < nw ? 1ull : 4ull);
     const unsigned long long light = kGrabPx * total / (*((volatile unsigned long long *)&f.ctr->q1_px) + 1);
     const uint32_t per = (uint32_t)max(1ull, min(32ull, min(fair, light)));
+    const uint32_t share = 2 * n <= nw ? (uint32_t)min((unsigned long long)kMaxShare, nw / (n + 1)) : 1u;   // per is 1 then
     unsigned long long n_s2 = 0, n_parts = 0;
+    unsigned long long unit = (unsigned long long)warp * gridDim.x + blockIdx.x;   // neighbours on different SMs
     for (;;) {
-        unsigned long long i0 = 0;
-        if (lane == 0) i0 = atomicAdd(&f.ctr->q1_next, (unsigned long long)per);
-        i0 = __shfl_sync(0xffffffffu, i0, 0);
+        const unsigned long long i0 = share > 1 ? (uint32_t)unit / share : unit * per;
+        const Share sh = {share > 1 ? (uint32_t)unit % share : 0u, share};
         if (i0 >= n) break;
         const uint32_t g = (uint32_t)min((unsigned long long)per, n - i0);
         uint32_t npx = 0, view = 0;
@@ -189,6 +212,7 @@ __global__ void __launch_bounds__(32 * s2::kWarps) k_stage2(const __grid_constan
                 clip = per == 1 || clipped_visible(c, &vw);
             }
         }
+        if (sh.k != 0) npx = 0;                       // whole in the first share
         S.npx[lane] = npx;
         __syncwarp();
         small_raster<1>(f, S, lane, nullptr);
@@ -207,13 +231,16 @@ __global__ void __launch_bounds__(32 * s2::kWarps) k_stage2(const __grid_constan
             const ViewDev &vw = f.views[v];
             int x0, x1, y0, y1;
             if (f.s3_ray && poly_range(s.X, s.Y, 3, vw.W, vw.H, x0, x1, y0, y1) > (int64_t)f.s2_max)
-                n_parts += append_parts<true>(f, s, pair, v, vw, x0, x1, y0, y1, lane);
+                n_parts += append_parts<true>(f, s, pair, v, vw, x0, x1, y0, y1, lane, sh);
             else
-                stage2_subtri(f, s, v, vw, lane, n_s2, n_parts);
+                stage2_subtri(f, s, v, vw, lane, sh, n_s2, n_parts);
         }
         for (unsigned m = __ballot_sync(0xffffffffu, clip); m; m &= m - 1)
-            stage2_clipped(&f, f.q1 + i0 + (__ffs(m) - 1), &n_s2, &n_parts);
+            stage2_clipped(&f, f.q1 + i0 + (__ffs(m) - 1), sh, &n_s2, &n_parts);
         __syncwarp();
+        if (share > 1) break;                         // units for all warps at most: n share <= nw
+        if (lane == 0) unit = nw + atomicAdd(&f.ctr->q1_next, 1ull);
+        unit = __shfl_sync(0xffffffffu, unit, 0);
     }
     if (f.stats && lane == 0) {
         stat_add(f, kStatS2, n_s2);

@@ -6,6 +6,7 @@ import pytest
 import torch
 
 import synthetic as S
+from oracle import oracle as orc
 from synthetic.scenes import Camera, Instance, Mesh, Scene
 
 from gpu_util import assert_vis_equal, oracle_vis, upload
@@ -119,4 +120,31 @@ def test_room_large(api, size):
     vis = r.render(cam.view, cam.proj, W, H)
     r.sync()
     assert_vis_equal(vis, oracle_vis(scene, cam), f"room {W} x {H}")
+    del keep
+
+
+@pytest.mark.parametrize("ray", [0, 1])
+@pytest.mark.parametrize("n", [1, 2, 33, 151, 152, 304, 607, 608, 609, 1215, 1217])
+def test_stage2_shares(api, n, ray):
+    """Short queues of triangles cut by the near plane and the guard band, each
+    shared by sixteen warps down to one; parts counted once."""
+    rng = np.random.default_rng(n)
+    pos = rng.uniform(-1, 1, (n, 3, 3)) * (2.0, 2.0, 1.0) + (0.0, 0.0, -0.6)
+    pos[::3] *= (40.0, 40.0, 1.0)
+    idx = np.arange(3 * n, dtype=np.int32).reshape(n, 3)
+    scene = Scene([Mesh(pos=torch.tensor(pos.reshape(-1, 3).astype(np.float32)), idx=torch.from_numpy(idx))],
+                  [Instance(0, np.eye(4, dtype=np.float32))],
+                  [Camera(np.eye(4, dtype=np.float32), S.perspective(90.0, 1.0, 1e-2, 10.0), 140, 100)])
+    cam = scene.cameras[0]
+    r = api.Renderer(0)
+    r.set_config(stage1_max_pixels=1, stage2_max_pixels=64, tile_log2=4, stage1_exact_all=1, stage3_raycast=ray,
+                 collect_stats=1)
+    keep = upload(r, scene, with_colour=False)
+    vis = r.render(cam.view, cam.proj, cam.W, cam.H)
+    parts = r.sync()["queued_stage3"]
+    ref = orc.render_paper(orc.OracleScene(scene), cam, 1, 64) if ray else oracle_vis(scene, cam)
+    assert_vis_equal(vis, ref, f"{n} clipped triangles")
+    again = r.render(cam.view, cam.proj, cam.W, cam.H)
+    assert r.sync()["queued_stage3"] == parts
+    assert torch.equal(vis, again)
     del keep
