@@ -87,24 +87,13 @@ __device__ __forceinline__ void stage2_subtri(const FrameDev &f, SubTri &s, uint
     }
 }
 
-// One queued triangle that reaches beyond a plane, by the whole warp.
-__device__ __noinline__ void stage2_clipped(const FrameDev *fp, const Q1Entry *ep, s2::Share sh, unsigned long long *n_s2,
-                                            unsigned long long *n_parts) {
-    const FrameDev &f = *fp;
-    const int lane = threadIdx.x & 31;
-    const Q1Entry e = *ep;
-    const PairDev &pr = f.pairs[e.pair];
-    const ViewDev vw = f.views[pr.view];
-    CV c[3];
-    load_clip(f, f.meshes[pr.mesh], e.pair, e.id - pr.base, vw, c);
-    CV poly[kMaxPoly];
-    const int np = clip_polygon(c, vw.nearv, poly);
-    if (np < 3) return;
-    int X[kMaxPoly], Y[kMaxPoly];
-    float iz[kMaxPoly];
-    for (int k = 0; k < np; ++k) snap(poly[k], vw.hw, vw.hh, X[k], Y[k], iz[k]);
+// A queued triangle as the polygon of its screen vertices (X, Y, iz)[0 .. np),
+// by the whole warp.
+__device__ __forceinline__ void stage2_poly(const FrameDev &f, const int *X, const int *Y, const float *iz, int np,
+                                            uint64_t id, uint32_t pair, uint32_t view, const ViewDev &vw, int lane,
+                                            s2::Share sh, unsigned long long &n_s2, unsigned long long &n_parts) {
     SubTri s;
-    s.id = e.id;
+    s.id = id;
     if (f.s3_ray) {
         // the paper's stage 3: a triangle whose visible bbox holds more
         // than s2_max pixel centres is ray cast over that range, in tiles
@@ -112,11 +101,10 @@ __device__ __noinline__ void stage2_clipped(const FrameDev *fp, const Q1Entry *e
         const int64_t cnt = poly_range(X, Y, np, vw.W, vw.H, x0, x1, y0, y1);
         if (cnt == 0) return;
         if (cnt > (int64_t)f.s2_max) {
-            *n_parts += append_parts<true>(f, s, e.pair, pr.view, vw, x0, x1, y0, y1, lane, sh);
+            n_parts += append_parts<true>(f, s, pair, view, vw, x0, x1, y0, y1, lane, sh);
             return;
         }
     }
-    unsigned long long a = 0, b = 0;
     // sub-triangles dealt out to the shares, or all of them to each
     const uint32_t m = (uint32_t)np - 2, each = sh.n / m;
     int j = 1, end = np - 1;
@@ -130,10 +118,8 @@ __device__ __noinline__ void stage2_clipped(const FrameDev *fp, const Q1Entry *e
         s.X[0] = X[0]; s.X[1] = X[j]; s.X[2] = X[j + 1];
         s.Y[0] = Y[0]; s.Y[1] = Y[j]; s.Y[2] = Y[j + 1];
         s.iz[0] = iz[0]; s.iz[1] = iz[j]; s.iz[2] = iz[j + 1];
-        stage2_subtri(f, s, pr.view, vw, lane, sh, a, b);
+        stage2_subtri(f, s, view, vw, lane, sh, n_s2, n_parts);
     }
-    *n_s2 += a;
-    *n_parts += b;
 }
 
 // Whether a triangle beyond some plane covers anything: false when its
@@ -159,7 +145,7 @@ __device__ __noinline__ bool clipped_visible(const CV *c, const ViewDev *vw) {
 // counter is 4 us.  A queue of fewer triangles than half the warps gives each
 // to several, up to kMaxShare: the triangles in it are then as a rule the large
 // ones, and a single warp would write thousands of parts (twelve triangles
-// that fill 3840 x 2160: 23 us, 14 shared).
+// that fill 3840 x 2160: 23 us, 11 shared).
 __global__ void __launch_bounds__(32 * s2::kWarps) k_stage2(const __grid_constant__ FrameDev f) {
     using namespace s2;
     __shared__ s1::SmallBatch<1> sw[kWarps];
@@ -169,10 +155,11 @@ __global__ void __launch_bounds__(32 * s2::kWarps) k_stage2(const __grid_constan
     const unsigned long long total = *((volatile unsigned long long *)&f.ctr->q1_count);
     const unsigned long long n = total < f.q1_cap ? total : f.q1_cap;
     const unsigned long long nw = (unsigned long long)gridDim.x * kWarps;
-    const unsigned long long fair = max(n / (2 * nw), n < nw ? 1ull : 4ull);
-    const unsigned long long light = kGrabPx * total / (*((volatile unsigned long long *)&f.ctr->q1_px) + 1);
-    const uint32_t per = (uint32_t)max(1ull, min(32ull, min(fair, light)));
-    const uint32_t share = 2 * n <= nw ? (uint32_t)min((unsigned long long)kMaxShare, nw / (n + 1)) : 1u;   // per is 1 then
+    const uint32_t fair = max((uint32_t)min(n, 64 * nw) / (uint32_t)(2 * nw), n < nw ? 1u : 4u);
+    const float light = __fdividef((float)kGrabPx * __ull2float_rn(total),
+                                   __ull2float_rn(*((volatile unsigned long long *)&f.ctr->q1_px)) + 1.0f);
+    const uint32_t per = max(1u, min(32u, min(fair, (uint32_t)light)));
+    const uint32_t share = 2 * n <= nw ? min(kMaxShare, (uint32_t)nw / ((uint32_t)n + 1)) : 1u;   // per is 1 then
     unsigned long long n_s2 = 0, n_parts = 0;
     unsigned long long unit = (unsigned long long)warp * gridDim.x + blockIdx.x;   // neighbours on different SMs
     for (;;) {
@@ -182,11 +169,8 @@ __global__ void __launch_bounds__(32 * s2::kWarps) k_stage2(const __grid_constan
         const uint32_t g = (uint32_t)min((unsigned long long)per, n - i0);
         uint32_t npx = 0, view = 0;
         bool whole = false, clip = false;             // for the warp: unclipped, clipped
-        int X[3] = {0, 0, 0}, Y[3] = {0, 0, 0};
-        float iz[3] = {0.0f, 0.0f, 0.0f};
-        Q1Entry e{0, 0, 0};
         if (lane < g) {
-            e = f.q1[i0 + lane];
+            const Q1Entry e = f.q1[i0 + lane];
             const PairDev &pr = f.pairs[e.pair];
             view = pr.view;
             const ViewDev &vw = f.views[view];
@@ -194,6 +178,8 @@ __global__ void __launch_bounds__(32 * s2::kWarps) k_stage2(const __grid_constan
             load_clip(f, f.meshes[pr.mesh], e.pair, e.id - pr.base, vw, c);
             if ((outcode(c[0], vw.nearv) | outcode(c[1], vw.nearv) | outcode(c[2], vw.nearv)) == 0) {
                 // inside every plane: Sutherland-Hodgman would return it unchanged
+                int X[3], Y[3];
+                float iz[3];
 #pragma unroll
                 for (int k = 0; k < 3; ++k) snap(c[k], vw.hw, vw.hh, X[k], Y[k], iz[k]);
                 int x0, x1, y0, y1;
@@ -202,6 +188,9 @@ __global__ void __launch_bounds__(32 * s2::kWarps) k_stage2(const __grid_constan
                 const int ey = max(Y[0], max(Y[1], Y[2])) - min(Y[0], min(Y[1], Y[2]));
                 if (cnt > 1024 || max(ex, ey) >= (1 << 14) || (!e.small && cnt > (int64_t)f.s2_max)) {
                     whole = true;
+                    S.t[lane][0] = make_uint4((uint32_t)X[0], (uint32_t)X[1], (uint32_t)X[2], (uint32_t)Y[0]);
+                    S.t[lane][1] = make_uint4((uint32_t)Y[1], (uint32_t)Y[2], __float_as_uint(iz[0]), __float_as_uint(iz[1]));
+                    S.t[lane][2] = make_uint4(__float_as_uint(iz[2]), 0u, 0u, 0u);
                 } else if (cnt > 0) {
                     const int A = (X[1] - X[0]) * (Y[2] - Y[0]) - (X[2] - X[0]) * (Y[1] - Y[0]);
                     if (A > 0)
@@ -210,6 +199,9 @@ __global__ void __launch_bounds__(32 * s2::kWarps) k_stage2(const __grid_constan
                 }
             } else {
                 clip = per == 1 || clipped_visible(c, &vw);
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+                    S.t[lane][k] = make_uint4(__float_as_uint(c[k].x), __float_as_uint(c[k].y), __float_as_uint(c[k].w), 0u);
             }
         }
         if (sh.k != 0) npx = 0;                       // whole in the first share
@@ -217,26 +209,30 @@ __global__ void __launch_bounds__(32 * s2::kWarps) k_stage2(const __grid_constan
         __syncwarp();
         small_raster<1>(f, S, lane, nullptr);
         n_s2 += __popc(__ballot_sync(0xffffffffu, npx != 0));
-        for (unsigned m = __ballot_sync(0xffffffffu, whole); m; m &= m - 1) {
+        const unsigned clipped = __ballot_sync(0xffffffffu, clip);
+        for (unsigned m = __ballot_sync(0xffffffffu, whole) | clipped; m; m &= m - 1) {
             const int l = __ffs(m) - 1;
-            SubTri s;
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                s.X[k] = __shfl_sync(0xffffffffu, X[k], l);
-                s.Y[k] = __shfl_sync(0xffffffffu, Y[k], l);
-                s.iz[k] = __shfl_sync(0xffffffffu, iz[k], l);
-            }
-            s.id = __shfl_sync(0xffffffffu, e.id, l);
-            const uint32_t v = __shfl_sync(0xffffffffu, view, l), pair = __shfl_sync(0xffffffffu, e.pair, l);
+            const Q1Entry e = f.q1[i0 + l];
+            const uint32_t v = f.pairs[e.pair].view;
             const ViewDev &vw = f.views[v];
-            int x0, x1, y0, y1;
-            if (f.s3_ray && poly_range(s.X, s.Y, 3, vw.W, vw.H, x0, x1, y0, y1) > (int64_t)f.s2_max)
-                n_parts += append_parts<true>(f, s, pair, v, vw, x0, x1, y0, y1, lane, sh);
-            else
-                stage2_subtri(f, s, v, vw, lane, sh, n_s2, n_parts);
+            const uint4 ta = S.t[l][0], tb = S.t[l][1], tc = S.t[l][2];
+            int X[kMaxPoly], Y[kMaxPoly], np = 3;
+            float iz[kMaxPoly];
+            if (clipped >> l & 1u) {
+                const CV c[3] = {{__uint_as_float(ta.x), __uint_as_float(ta.y), __uint_as_float(ta.z)},
+                                 {__uint_as_float(tb.x), __uint_as_float(tb.y), __uint_as_float(tb.z)},
+                                 {__uint_as_float(tc.x), __uint_as_float(tc.y), __uint_as_float(tc.z)}};
+                CV poly[kMaxPoly];
+                np = clip_polygon(c, vw.nearv, poly);
+                if (np < 3) continue;
+                for (int k = 0; k < np; ++k) snap(poly[k], vw.hw, vw.hh, X[k], Y[k], iz[k]);
+            } else {
+                X[0] = (int)ta.x; X[1] = (int)ta.y; X[2] = (int)ta.z;
+                Y[0] = (int)ta.w; Y[1] = (int)tb.x; Y[2] = (int)tb.y;
+                iz[0] = __uint_as_float(tb.z); iz[1] = __uint_as_float(tb.w); iz[2] = __uint_as_float(tc.x);
+            }
+            stage2_poly(f, X, Y, iz, np, e.id, e.pair, v, vw, lane, sh, n_s2, n_parts);
         }
-        for (unsigned m = __ballot_sync(0xffffffffu, clip); m; m &= m - 1)
-            stage2_clipped(&f, f.q1 + i0 + (__ffs(m) - 1), sh, &n_s2, &n_parts);
         __syncwarp();
         if (share > 1) break;                         // units for all warps at most: n share <= nw
         if (lane == 0) unit = nw + atomicAdd(&f.ctr->q1_next, 1ull);
