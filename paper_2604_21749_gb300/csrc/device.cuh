@@ -309,6 +309,9 @@ static __device__ __noinline__ int clip_polygon(const CV tri[3], float nearv, CV
     int n = 3;
     a[0] = tri[0]; a[1] = tri[1]; a[2] = tri[2];
     for (int p = 0; p < 5 && n > 0; ++p) {
+        bool inside = true;
+        for (int i = 0; i < n; ++i) inside &= plane_value(p, a[i], nearv) >= 0.0f;
+        if (inside) continue;                        // the pass would copy the polygon
         int m = 0;
         CV prev = a[n - 1];
         float fprev = plane_value(p, prev, nearv);
