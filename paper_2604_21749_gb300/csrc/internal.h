@@ -36,6 +36,23 @@ struct BeginArgs {
     uint64_t n[kBeginViews];
 };
 cudaError_t launch_begin(const BeginArgs &a, cudaStream_t s);
+// A stage kernel, launched ahead of its predecessor's end where the frame
+// allows it (begin_stage waits).
+template <class... P, class... A>
+inline cudaError_t launch_stage(bool pdl, void (*k)(P...), int blocks, int threads, size_t smem, cudaStream_t s, A... args) {
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 // Stage 1 of round r: the cull kernel, then the exact kernel over the round's
 // bitmap.  near = false launches the cull without its near-plane test (valid
 // when no pair's mesh bounds reach the near plane).

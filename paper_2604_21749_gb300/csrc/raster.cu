@@ -619,23 +619,6 @@ cudaError_t launch_begin(const BeginArgs &a, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-// A stage kernel, launched ahead of its predecessor's end where the frame
-// allows it (begin_stage waits).
-template <class... P, class... A>
-static cudaError_t launch_stage(bool pdl, void (*k)(P...), int blocks, int threads, size_t smem, cudaStream_t s, A... args) {
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = dim3((unsigned)blocks);
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cfg.attrs = at;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, k, args...);
-}
-
 cudaError_t launch_stage1(const FrameDev &f, bool instanced, int variant, uint32_t r, int blocks, bool near,
                           cudaStream_t s) {
     const size_t s0 = stage1_smem_bytes<false>(), si = stage1_smem_bytes<true>();

@@ -69,6 +69,7 @@ struct StaticFrame {
 // unusable.)
 __global__ void __launch_bounds__(256) k_static_begin(uint64_t *vis, uint64_t n, const float *pos, uint64_t V) {
     const uint64_t stride = (uint64_t)gridDim.x * 256, first = (uint64_t)blockIdx.x * 256 + threadIdx.x;
+    asm volatile("griddepcontrol.launch_dependents;");
     if ((reinterpret_cast<uintptr_t>(vis) & 15) == 0) {
         ulonglong2 *v2 = reinterpret_cast<ulonglong2 *>(vis);
         for (uint64_t k = first; k < n / 2; k += stride) v2[k] = make_ulonglong2(kEmpty, kEmpty);
@@ -130,6 +131,8 @@ __global__ void __launch_bounds__(kMaxRounds) k_static_rounds(uint64_t first, ui
 __global__ void __launch_bounds__(256) k_static_setup(const __grid_constant__ StaticFrame s) {
     unsigned char *g = g_static_scratch;
     const int t = (int)threadIdx.x, lane = t & 31;
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;");
     unsigned long long *c = reinterpret_cast<unsigned long long *>(g + kOffCtr);
     for (size_t i = t; i < sizeof(Counters) / sizeof(unsigned long long); i += blockDim.x) c[i] = 0ull;
     __syncthreads();
@@ -330,8 +333,7 @@ extern "C" curast_status curast_render_static(const float *pos, uint64_t V, cons
     const int sms = ds->shape.num_sms;
     k_static_begin<<<kBoundBlocks, 256, 0, s>>>(vis, (uint64_t)W * (uint64_t)H, fr.cull ? pos : nullptr, V);
     if ((e = cudaGetLastError()) != cudaSuccess) return CURAST_ERR_CUDA;
-    k_static_setup<<<1, 256, 0, s>>>(fr);
-    if ((e = cudaGetLastError()) != cudaSuccess) return CURAST_ERR_CUDA;
+    if ((e = launch_stage(f.pdl != 0, k_static_setup, 1, 256, 0, s, fr)) != cudaSuccess) return CURAST_ERR_CUDA;
     for (uint64_t r = 0; r < rounds; ++r) {
         if (r > 0 && r % kMaxRounds == 0) {
             k_static_rounds<<<1, kMaxRounds, 0, s>>>(r, items, fr.round_items, item_words);
