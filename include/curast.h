@@ -349,9 +349,10 @@ curast_status curast_last_frame(const curast_ctx *ctx, curast_frame_info *out);
  * device check failed since the previous curast_sync, else CURAST_OK. */
 curast_status curast_sync(curast_ctx *ctx, curast_stream stream, curast_stats *stats);
 
-/* Per-stage device times (ms) of the last render issued on this context:
- * out[0] clear, [1] stage-1 cull, [2] stage-1 exact path, [3] stage 2,
- * [4] stage 3; waits for them. */
+/* Per-stage device times (ms) of the last render issued on this context
+ * (graph replays and captured renders take none): out[0] clear, [1] stage-1
+ * cull, [2] stage-1 exact path, [3] stage 2, [4] stage 3; waits for them.
+ * They run from one stage's first block to the next one's. */
 curast_status curast_stage_times(curast_ctx *ctx, float out[5]);
 
 /* Picks stage thresholds, tile size, batch shape, pairs per work item and the

@@ -235,10 +235,12 @@ __device__ __forceinline__ unsigned long long now_ns() {
 // Every stage kernel starts with this: it may have been launched while the
 // kernel before it in the stream still runs, waits here until that one is done
 // and its writes are visible, and lets the next one be launched in turn (which
-// waits for this one here).  stamp: the time it takes, or kStampCount.
+// waits for this one here).  stamp: the time it takes, or kStampCount.  LAST:
+// the frame's last kernel, whose successor is the caller's and stays behind it.
+template <bool LAST = false>
 __device__ __forceinline__ void begin_stage(const FrameDev &f, int stamp) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;");
+    if (!LAST) asm volatile("griddepcontrol.launch_dependents;");
     if (f.stamps && stamp != kStampCount && blockIdx.x == 0 && threadIdx.x == 0) f.stamps[stamp] = now_ns();
 }
 
@@ -397,7 +399,7 @@ __device__ __forceinline__ bool setup_subtri(SubTri &s, int W, int H) {
 // with the same rounding (32 bits hold the float's 24, the half and a sticky
 // bit), and the power of two put back is exact.  All on 32-bit words: GB300
 // converts 64-bit integers at a sixteenth of that rate, which bounded stages
-// 2 and 3 (twelve huge triangles at 4K: stage 3 69 us, 43 us with this).
+// 2 and 3 (twelve huge triangles at 4K: stage 3 69 us, 46 with this).
 __device__ __forceinline__ float nonneg_to_float(int64_t v) {
     const uint32_t hi = (uint32_t)((uint64_t)v >> 32), lo = (uint32_t)v;
     const int s = __clz((int)hi);                    // 32 where hi is 0

@@ -26,7 +26,7 @@ __global__ void __launch_bounds__(256) k_clear(uint64_t *vis, uint64_t n) {
 // The start of a frame in one launch: the tables from pinned host memory
 // (read in place), zeroed counters, cleared buffers.  Three copies, a memset,
 // a clear and the events between the stages took more of a small frame than
-// its kernels (131 k triangles on 640x480: 83 us a frame, the kernels 37 us);
+// its kernels (131 k triangles on 512x512: 83 us a frame, the kernels 37 us);
 // with this, and each stage launched ahead of its predecessor's end, 46 us.
 __global__ void __launch_bounds__(256) k_begin(const __grid_constant__ BeginArgs a) {
     const uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = (uint64_t)gridDim.x * blockDim.x;
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(256) k_stage3(const __grid_constant__ FrameDev
     __shared__ SubTri part[s3::kGrab];               // x0 .. y1: the range inside the tile, x0 > x1: none
     __shared__ uint32_t s_view[s3::kGrab], s_ray[s3::kGrab];   // s_ray: pair + 1 of a ray-cast part
     __shared__ unsigned long long s_next;
-    begin_stage(f, kStampStage3);
+    begin_stage<true>(f, kStampStage3);
     const unsigned long long total = *((volatile unsigned long long *)&f.ctr->q2_count);
     const unsigned long long n = total < f.q2_cap ? total : f.q2_cap;
     const int ts = 1 << f.tile_log2;
@@ -399,7 +399,7 @@ struct PartRec {
 // functions stepped from row to row; then it writes each of its covered
 // pixels once to the visibility buffer and resets the word.
 __global__ void __launch_bounds__(256) k_stage3_tiles(const __grid_constant__ FrameDev f) {
-    begin_stage(f, kStampCount);
+    begin_stage<true>(f, kStampCount);
     extern __shared__ __align__(16) unsigned long long tw[];     // the tile's words
     __shared__ PartRec pr[kUnitParts];
     __shared__ unsigned long long s_i;

@@ -3,8 +3,8 @@
 // Warp-specialized pipeline: one producer warp grabs work items from the
 // global counter, stages each item's index triples in shared memory with a
 // TMA bulk copy and fills the item's per-(instance, view) constants; eight
-// consumer warps cull and rasterize.  Producer and consumers meet only at
-// full / empty mbarriers of a three-slot ring, so no block-wide barrier
+// consumer warps cull into the survivor bitmap.  Producer and consumers meet
+// only at full / empty mbarriers of a ring of slots, so no block-wide barrier
 // stalls the consumers.
 #pragma once
 
