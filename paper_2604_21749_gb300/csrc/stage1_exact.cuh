@@ -22,7 +22,7 @@ constexpr int kBatch = 32 * kExactK;
 constexpr uint32_t kUnits = 13;                      // units dealt out of one block of the bitmap
 constexpr uint32_t kUnitSurvivors = 128;             // survivors of a unit, about
 constexpr int kDenseBits = 12;                       // words with as many survivors are unpacked by the whole warp
-constexpr uint32_t kSegPx = 2048;                    // pixels whose triangle starts are marked at once
+constexpr uint32_t kSegPx = 1024;                    // pixels whose triangle starts are marked at once
 
 // A small triangle ready for the pixel loop, 48 bytes: eight lanes' 16-byte
 // loads of neighbouring records touch every bank once.
@@ -470,7 +470,8 @@ __global__ void __launch_bounds__(32 * s1::kExactWarps, 1)
         __syncwarp();
         // a batch of heavy triangles (a near surface, up to 128 pixels each) would keep its warp long after
         // the others: what starts past kSegPx pixels goes to stage 2, which deals triangles out finely (a
-        // close 4K view of a 100 M-triangle scan: exact kernel and stage 2 521 + 67 us, 453 + 41 us with it)
+        // close 4K view of a 100 M-triangle scan: exact kernel and stage 2 521 + 67 us, 453 + 41 us with it
+        // past 2048 pixels; past 1024 or 2048, 349 + 68 and 385 + 46; past 512, 322 + 116)
         small_raster<kExactK>(f, S, lane, [&](bool want, int slot) -> bool {
             unsigned long long base = 0;
             const unsigned all = __ballot_sync(0xffffffffu, want);
