@@ -20,6 +20,19 @@ constexpr unsigned kMaxShare = 16;
 struct Share { uint32_t k, n; };
 }
 
+// A part that queue 2 has no room for, by one lane.  (Out of line: the kernel
+// waits for its instructions where the queue is short.)
+template <bool RAY>
+__device__ __noinline__ void part_in_place(const FrameDev *f, const SubTri *s, uint32_t pidx, const ViewDev *vw, int x0, int x1,
+                                           int y0, int y1) {
+    if (RAY) {
+        RayTri R;
+        if (ray_tri_of(*f, pidx, s->id, R)) ray_range(R, x0, x1, y0, y1, 0, 1, *vw, s->id);
+    } else {
+        raster_range(*s, x0, x1, y0, y1, 0, 1, vw->vis, vw->W);
+    }
+}
+
 // The warp's share of the tiles of [x0, x1] x [y0, y1] as stage-3 parts, with
 // one reservation of queue 2.  RAY: the whole triangle is ray cast, s holds its id alone.  Parts
 // past the queue's capacity are rasterized in place.  Returns their number.
@@ -63,12 +76,8 @@ __device__ __forceinline__ uint32_t append_parts(const FrameDev &f, const SubTri
             atomicAdd(&f.ctr->overflow2, 1ull);
             const int rx0 = max(x0, (int)ex * ts), rx1 = min(x1, (int)ex * ts + ts - 1);
             const int ry0 = max(y0, (int)ey * ts), ry1 = min(y1, (int)ey * ts + ts - 1);
-            if (RAY) {
-                RayTri R;
-                if (ray_tri_of(f, pidx, s.id, R)) ray_range(R, rx0, rx1, ry0, ry1, 0, 1, vw, s.id);
-            } else {
-                raster_range(s, rx0, rx1, ry0, ry1, 0, 1, vw.vis, vw.W);
-            }
+            const SubTri t = s;
+            part_in_place<RAY>(&f, &t, pidx, &vw, rx0, rx1, ry0, ry1);
         }
     }
     return (uint32_t)nt;
@@ -145,7 +154,7 @@ __device__ __noinline__ bool clipped_visible(const CV *c, const ViewDev *vw) {
 // counter is 4 us.  A queue of fewer triangles than half the warps gives each
 // to several, up to kMaxShare: the triangles in it are then as a rule the large
 // ones, and a single warp would write thousands of parts (twelve triangles
-// that fill 3840 x 2160: 23 us, 11 shared).
+// that fill 3840 x 2160: 23 us, 8 now).
 __global__ void __launch_bounds__(32 * s2::kWarps) k_stage2(const __grid_constant__ FrameDev f) {
     using namespace s2;
     __shared__ s1::SmallBatch<1> sw[kWarps];
