@@ -58,7 +58,7 @@ inline cudaError_t launch_stage(bool pdl, void (*k)(P...), int blocks, int threa
 // when no pair's mesh bounds reach the near plane).
 cudaError_t launch_stage1(const FrameDev &f, bool instanced, int variant, uint32_t r, int blocks, bool near,
                           cudaStream_t s);
-cudaError_t launch_stage1_exact(const FrameDev &f, uint32_t r, int blocks, cudaStream_t s);
+cudaError_t launch_stage1_exact(const FrameDev &f, bool comp, uint32_t r, int blocks, cudaStream_t s);
 cudaError_t launch_stage2(const FrameDev &f, int blocks, cudaStream_t s);
 cudaError_t launch_stage3(const FrameDev &f, int blocks, cudaStream_t s);
 // Binned stage 3: scan of the per-tile part counts, scatter of the parts into

@@ -580,11 +580,12 @@ cudaError_t query_launch_shape(LaunchShape *o, int device) {
         if (e != cudaSuccess) return e;
         o->stage1_blocks_per_sm[1][2] = o->stage1_blocks_per_sm[0][2];
     }
-    e = cudaFuncSetAttribute(k_stage1_exact<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)exact_smem_bytes());
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(k_stage1_exact<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)exact_smem_bytes());
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o->stage1x_blocks_per_sm, k_stage1_exact<false>,
+    for (auto k : {k_stage1_exact<false, false>, k_stage1_exact<false, true>, k_stage1_exact<true, false>,
+                   k_stage1_exact<true, true>}) {
+        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)exact_smem_bytes());
+        if (e != cudaSuccess) return e;
+    }
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o->stage1x_blocks_per_sm, k_stage1_exact<false, false>,
                                                       32 * s1::kExactWarps, exact_smem_bytes());
     if (e != cudaSuccess) return e;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o->stage2_blocks_per_sm, k_stage2, 32 * s2::kWarps, 0);
@@ -636,9 +637,10 @@ cudaError_t launch_stage1(const FrameDev &f, bool instanced, int variant, uint32
     return launch_stage(p, k_stage1<false, false, false>, blocks, s1::kThreads, s0, s, f, r);
 }
 
-cudaError_t launch_stage1_exact(const FrameDev &f, uint32_t r, int blocks, cudaStream_t s) {
-    if (f.s3_ray) return launch_stage(f.pdl != 0, k_stage1_exact<true>, blocks, 32 * s1::kExactWarps, exact_smem_bytes(), s, f, r);
-    return launch_stage(f.pdl != 0, k_stage1_exact<false>, blocks, 32 * s1::kExactWarps, exact_smem_bytes(), s, f, r);
+cudaError_t launch_stage1_exact(const FrameDev &f, bool comp, uint32_t r, int blocks, cudaStream_t s) {
+    const auto k = f.s3_ray ? (comp ? k_stage1_exact<true, true> : k_stage1_exact<true, false>)
+                            : (comp ? k_stage1_exact<false, true> : k_stage1_exact<false, false>);
+    return launch_stage(f.pdl != 0, k, blocks, 32 * s1::kExactWarps, exact_smem_bytes(), s, f, r);
 }
 
 cudaError_t launch_stage2(const FrameDev &f, int blocks, cudaStream_t s) {

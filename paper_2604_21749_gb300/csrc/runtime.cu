@@ -606,7 +606,7 @@ curast_status enqueue_stages(curast_ctx *c, bool clear, Frame how, cudaStream_t 
         const int variant = c->round_comp[r] ? 1 : (!c->instanced && c->cfg.stage1_vertex_reuse ? 2 : 0);
         CU(launch_stage1(f, c->instanced, variant, r, sms * c->shape.stage1_blocks_per_sm[c->instanced ? 1 : 0][variant],
                          c->near_needed, s));
-        CU(launch_stage1_exact(f, r, sms * c->shape.stage1x_blocks_per_sm, s));
+        CU(launch_stage1_exact(f, c->round_comp[r] != 0, r, sms * c->shape.stage1x_blocks_per_sm, s));
     }
     CU(launch_stage2(f, sms * c->shape.stage2_blocks_per_sm, s));
     if (f.s3_bin)

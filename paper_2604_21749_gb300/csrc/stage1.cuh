@@ -270,10 +270,11 @@ __device__ __forceinline__ bool group_cull(const FastPair &fp, float3 c, float3 
 // order, clip outcodes, snap, culls, then stage-1 raster or queue 1.
 // e = (triangle within its mesh, pair).  f must live in parameter or global
 // memory (queue-1 overflow passes its address on).
+template <bool COMP>
 __device__ __forceinline__ void exact_gather(const FrameDev &f, uint2 e, bool live, Tri9 &p) {
     if (live) {
         const MeshDev &mesh = f.meshes[f.pairs[e.y].mesh];
-        if (!compressed(mesh)) {
+        if (!COMP) {
             const uint32_t *ix = mesh.idx + 3 * (uint64_t)e.x;
             const float *pos = mesh.pos;
             const uint32_t i0 = __ldg(ix), i1 = __ldg(ix + 1), i2 = __ldg(ix + 2);

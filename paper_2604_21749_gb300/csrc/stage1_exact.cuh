@@ -289,8 +289,9 @@ size_t exact_smem_bytes() { return sizeof(s1::ExactWarp) * s1::kExactWarps; }
 // last of them from one in global memory, which evens the SMs out: one global
 // address takes an atomic add every 1.8 ns, too slow for every unit (32-word
 // units of the billion-triangle frame: 1.75 ms against 0.90).  The words of
-// the next unit are in flight while a batch runs.
-template <bool RAY>
+// the next unit are in flight while a batch runs.  COMP: the round's meshes
+// are compressed (one kernel for both tested it per triangle, 1% of the frame).
+template <bool RAY, bool COMP>
 __global__ void __launch_bounds__(32 * s1::kExactWarps, 1)
     k_stage1_exact(const __grid_constant__ FrameDev f, uint32_t r) {
     using namespace s1;
@@ -454,7 +455,7 @@ __global__ void __launch_bounds__(32 * s1::kExactWarps, 1)
 #pragma unroll
             for (int u = 0; u < kExactK; ++u) {
                 const bool live = lane + 32 * u < n;
-                exact_gather(f, S.e[live ? lane + 32 * u : 0], live, p[u]);
+                exact_gather<COMP>(f, S.e[live ? lane + 32 * u : 0], live, p[u]);
             }
 #pragma unroll
             for (int u = 0; u < kExactK; ++u) {

@@ -343,7 +343,7 @@ extern "C" curast_status curast_render_static(const float *pos, uint64_t V, cons
         if ((e = launch_stage1(f, inst, 0, k, sms * ds->shape.stage1_blocks_per_sm[inst ? 1 : 0][0], fr.cull != 0, s)) !=
             cudaSuccess)
             return CURAST_ERR_CUDA;
-        if ((e = launch_stage1_exact(f, k, sms * ds->shape.stage1x_blocks_per_sm, s)) != cudaSuccess) return CURAST_ERR_CUDA;
+        if ((e = launch_stage1_exact(f, false, k, sms * ds->shape.stage1x_blocks_per_sm, s)) != cudaSuccess) return CURAST_ERR_CUDA;
     }
     if ((e = launch_stage2(f, sms * ds->shape.stage2_blocks_per_sm, s)) != cudaSuccess) return CURAST_ERR_CUDA;
     if ((e = launch_stage3(f, sms * ds->shape.stage3_blocks_per_sm, s)) != cudaSuccess) return CURAST_ERR_CUDA;
