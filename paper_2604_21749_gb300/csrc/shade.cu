@@ -506,20 +506,24 @@ constexpr int kBwdWarps = 8;
 
 struct BwdGroup { uint32_t members, v[3]; };
 
+struct BwdShared {                                   // of a block, beside the numbers
+    BwdGroup groups[kBwdWarps][32];
+    uint32_t dest[9 + 3 * kMaxC];                    // number: vertex | offset in the row << 2 | attribute << 31
+    DF rx[32], ry[8];
+};
+
 template <bool FEW>
 __global__ void __launch_bounds__(32 * kBwdWarps) k_interp_bwd(const __grid_constant__ ShadeArgs a) {
     extern __shared__ float bwd_vals[];              // [warp][lane][n | 1]
-    __shared__ BwdGroup groups[kBwdWarps][32];
-    __shared__ uint32_t dest[9 + 3 * kMaxC];         // number: vertex | offset in the row << 2 | attribute << 31
-    __shared__ DF rx[32], ry[8];
+    __shared__ BwdShared blk;
     const int C = a.C, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int np = a.grad_pos ? 9 : 0, n = np + (a.grad_attr ? 3 * C : 0);
     const int bx = blockIdx.x * 32, by = blockIdx.y * 8;
-    if (threadIdx.x < 32) rx[lane] = ray_coord(bx + lane, a.W, a.fx);
-    else if (threadIdx.x < 40) ry[threadIdx.x - 32] = ray_coord(by + threadIdx.x - 32, a.H, a.fy);
+    if (threadIdx.x < 32) blk.rx[lane] = ray_coord(bx + lane, a.W, a.fx);
+    else if (threadIdx.x < 40) blk.ry[threadIdx.x - 32] = ray_coord(by + threadIdx.x - 32, a.H, a.fy);
     else if (threadIdx.x >= 64 && threadIdx.x < 64 + n) {
         const int c = threadIdx.x - 64, q = c - np;
-        dest[c] = c < np ? (uint32_t)(c / 3) | (uint32_t)(c % 3) << 2 : (uint32_t)(q / C) | (uint32_t)(q % C) << 2 | 1u << 31;
+        blk.dest[c] = c < np ? (uint32_t)(c / 3) | (uint32_t)(c % 3) << 2 : (uint32_t)(q / C) | (uint32_t)(q % C) << 2 | 1u << 31;
     }
     __syncthreads();
     const int lx = (warp & 3) * 8 + (lane & 7), ly = (warp >> 2) * 4 + (lane >> 3);
@@ -548,7 +552,7 @@ __global__ void __launch_bounds__(32 * kBwdWarps) k_interp_bwd(const __grid_cons
             v0[r] = df_add(acc, {mv[4 * r + 3], 0.0f});
         }
         // the pixel-centre ray as double-floats
-        const DF dx = rx[lx], dy = ry[ly];
+        const DF dx = blk.rx[lx], dy = blk.ry[ly];
         const DF dz = {-1.0f, 0.0f};
         const float3 r = make_float3(dx.hi, dy.hi, -1.0f);
         // m = v0 x r
@@ -604,18 +608,18 @@ __global__ void __launch_bounds__(32 * kBwdWarps) k_interp_bwd(const __grid_cons
     const unsigned same = __match_any_sync(0xffffffffu, (unsigned long long)(hit ? key & kIdMask : kEmpty)) & hits;
     const bool leads = hit && (same & ((1u << lane) - 1u)) == 0;
     const unsigned leaders = __ballot_sync(0xffffffffu, leads);
-    if (leads) groups[warp][__popc(leaders & ((1u << lane) - 1u))] = BwdGroup{same, {vi[0], vi[1], vi[2]}};
+    if (leads) blk.groups[warp][__popc(leaders & ((1u << lane) - 1u))] = BwdGroup{same, {vi[0], vi[1], vi[2]}};
     __syncwarp();
     const float *all = bwd_vals + (size_t)32 * warp * (n | 1);
     const int total = __popc(leaders) * n;
     const int dg = 32 / n, dc = 32 - dg * n;         // a step of 32 numbers: dg groups and dc numbers
     int g = lane / n, c = lane - g * n;
     for (int i = lane; i < total; i += 32) {
-        const BwdGroup &gr = groups[warp][g];
+        const BwdGroup &gr = blk.groups[warp][g];
         uint32_t m = gr.members;
         float sum = all[(__ffs(m) - 1) * (n | 1) + c];
         for (m &= m - 1; m; m &= m - 1) sum = __fadd_rn(sum, all[(__ffs(m) - 1) * (n | 1) + c]);
-        const uint32_t d = dest[c], off = (d >> 2) & 31u;
+        const uint32_t d = blk.dest[c], off = (d >> 2) & 31u;
         const size_t v = gr.v[d & 3u];
         atomicAdd(d >> 31 ? a.grad_attr + (size_t)C * v + off : a.grad_pos + 3 * v + off, sum);
         g += dg;
@@ -681,7 +685,7 @@ cudaError_t launch_interpolate_backward(const ShadeArgs &a, cudaStream_t s) {
     const int n = (a.grad_pos ? 9 : 0) + (a.grad_attr ? 3 * a.C : 0);
     const size_t smem = (size_t)32 * kBwdWarps * (n | 1) * sizeof(float);
     void (*k)(ShadeArgs) = a.n_inst <= kFew ? k_interp_bwd<true> : k_interp_bwd<false>;
-    if (smem > 48 * 1024) {
+    if (smem + sizeof(BwdShared) > 48 * 1024) {      // (what a launch may have without asking counts both)
         const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
