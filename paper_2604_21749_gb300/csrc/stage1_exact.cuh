@@ -314,11 +314,12 @@ __global__ void __launch_bounds__(32 * s1::kExactWarps, 1)
     // same 640 places (the cull would pay 3% for counting them): a unit of kUnitSurvivors at that density,
     // fewer where an SM would get less than 16 such units, but 16 words where there are twelve of that for
     // every warp, and not so small that the fetches over empty stretches pile up.  Frames with few words need
-    // no estimate.
+    // no estimate.  All blocks have to arrive at the same split: the cull before this kernel wrote the words
+    // while it was already resident, so they are read from L2, never through the constant-data path.
     uint64_t per_unit = nwords / nw;
     if (nwords >= 8ull * nw) {
         const uint64_t q = nwords / 4 * threadIdx.x / blockDim.x;
-        const uint4 v = __ldg(reinterpret_cast<const uint4 *>(f.bits) + q);
+        const uint4 v = __ldcg(reinterpret_cast<const uint4 *>(f.bits) + q);
         const uint32_t n = __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w);
         const uint32_t sum = __reduce_add_sync(0xffffffffu, n) | (uint32_t)__popc(__ballot_sync(0xffffffffu, n != 0)) << 20;
         if (lane == 0 && sum) atomicAdd(&s_sample, sum);
