@@ -20,21 +20,23 @@ using namespace curast;
 
 namespace {
 
+// keep: where an outgrown buffer goes that a captured frame may still name (nullptr: it is freed).
 template <class T>
 struct DevBuf {
     T *p = nullptr;
     size_t cap = 0;
-    cudaError_t reserve(size_t n) {
+    cudaError_t reserve(size_t n, std::vector<void *> *keep = nullptr) {
         if (n <= cap) return cudaSuccess;
-        release();
+        release(keep);
         size_t c = std::max<size_t>(n, 16);
         cudaError_t e = cudaMalloc(reinterpret_cast<void **>(&p), c * sizeof(T));
         if (e != cudaSuccess) { p = nullptr; return e; }
         cap = c;
         return cudaSuccess;
     }
-    void release() {
-        if (p) cudaFree(p);
+    void release(std::vector<void *> *keep = nullptr) {
+        if (p && keep) keep->push_back(p);
+        else if (p) cudaFree(p);
         p = nullptr;
         cap = 0;
     }
@@ -209,12 +211,14 @@ struct curast_ctx {
 
     // frame tables: [hdr | views | segs | pairs], one device copy and a ring of pinned ones, so that the host
     // can prepare frames while earlier ones run (ev_tab: the frame that read the slot is done, or its copy).
-    // A frame captured by the caller keeps its slot: replays read it again.
+    // A frame captured by the caller keeps its slot, which replays read again, and with it every device buffer
+    // that is outgrown later.
     DevBuf<unsigned char> d_tab;
     static constexpr int kSlots = 4;
     PinBuf<unsigned char> h_tab[kSlots];
     cudaEvent_t ev_tab[kSlots] = {nullptr, nullptr, nullptr, nullptr};
     bool kept[kSlots] = {false, false, false, false};
+    std::vector<void *> outgrown;
     int slot = 0;
     size_t cap_views = 0, cap_segs = 0, cap_pairs = 0;
     std::vector<ViewDev> hv;
@@ -280,6 +284,20 @@ void invalidate_graph(curast_ctx *c) {
     c->gkey.clear();
 }
 
+bool is_kept(const curast_ctx *c, int slot) { return c->kept[slot]; }
+
+// Where buffers that a captured frame may name go when they are outgrown: null where there is no such frame.
+std::vector<void *> *keep(curast_ctx *c) {
+    for (int k = 0; k < curast_ctx::kSlots; ++k)
+        if (is_kept(c, k)) return &c->outgrown;
+    return nullptr;
+}
+
+void free_outgrown(curast_ctx *c) {
+    for (void *p : c->outgrown) cudaFree(p);
+    c->outgrown.clear();
+}
+
 MeshDev mesh_dev(const MeshRec &r) {
     MeshDev m{};
     m.pos = r.pos;
@@ -310,7 +328,7 @@ curast_status sync_scene(curast_ctx *c, cudaStream_t s) {
         std::vector<MeshDev> md(c->meshes.size());
         for (size_t i = 0; i < md.size(); ++i) md[i] = mesh_dev(c->meshes[i]);
         const bool grow = md.size() > c->d_meshes.cap;
-        CU(c->d_meshes.reserve(std::max<size_t>(md.size(), 1)));
+        CU(c->d_meshes.reserve(std::max<size_t>(md.size(), 1), keep(c)));
         if (grow) invalidate_graph(c);
         if (!md.empty()) CU(cudaMemcpyAsync(c->d_meshes.p, md.data(), md.size() * sizeof(MeshDev), cudaMemcpyHostToDevice, s));
         c->meshes_dirty = false;
@@ -453,7 +471,7 @@ curast_status build_frame(curast_ctx *c, const curast_view *views, int nv, long 
     if (c->rounds.size() > (size_t)kMaxRounds) return CURAST_ERR_INVALID_ARG;   // unreachable by the cap above
     uint64_t maxw = 1;
     for (const RoundDev &r : c->rounds) maxw = std::max(maxw, r.w1 - r.w0);
-    CU(c->d_bits.reserve(maxw));
+    CU(c->d_bits.reserve(maxw, keep(c)));
     // stage-3 tiles of every view, numbered view by view, row by row
     {
         const uint64_t ts = 1ull << c->cfg.tile_log2;
@@ -466,9 +484,9 @@ curast_status build_frame(curast_ctx *c, const curast_view *views, int nv, long 
         if (nt >= (1ull << 31)) return CURAST_ERR_INVALID_ARG;
         c->n_tiles = (uint32_t)nt;
         if (c->cfg.stage3_tile_buffer) {
-            CU(c->d_tiles.reserve(3 * nt + 1));
+            CU(c->d_tiles.reserve(3 * nt + 1, keep(c)));
             // a tile of c parts makes ceil(c / 8) units
-            CU(c->d_units.reserve(nt + c->cfg.queue2_capacity / 8 + 1));
+            CU(c->d_units.reserve(nt + c->cfg.queue2_capacity / 8 + 1, keep(c)));
         }
     }
     c->hdr.n_batches = nb;
@@ -488,28 +506,38 @@ size_t off_pairs(const curast_ctx *c) { return align_up(off_segs(c) + c->cap_seg
 size_t tab_bytes(const curast_ctx *c) { return off_pairs(c) + c->cap_pairs * sizeof(PairDev); }
 
 // Fills the next pinned copy of the frame's tables; the frame's first kernel
-// reads it in place.
+// reads it in place.  Three of the copies may belong to captured frames: one is
+// always left for the others.
 curast_status stage_frame(curast_ctx *c, bool capturing) {
     if (c->hv.size() > c->cap_views || c->hs.size() > c->cap_segs || c->hp.size() > c->cap_pairs) {
-        for (bool k : c->kept)
-            if (k) return CURAST_ERR_CUDA;   // a captured frame writes the tables' present copy
         for (cudaEvent_t e : c->ev_tab) CU(cudaEventSynchronize(e));
         c->cap_views = std::max<size_t>(c->hv.size(), std::max<size_t>(2 * c->cap_views, 8));
         c->cap_segs = std::max<size_t>(c->hs.size(), std::max<size_t>(2 * c->cap_segs, 256));
         c->cap_pairs = std::max<size_t>(c->hp.size(), std::max<size_t>(2 * c->cap_pairs, 256));
-        c->d_tab.release();
-        CU(c->d_tab.reserve(tab_bytes(c)));
-        for (auto &h : c->h_tab) CU(h.reserve(tab_bytes(c)));
+        c->d_tab.release(keep(c));
         invalidate_graph(c);
+        const cudaError_t e = c->d_tab.reserve(tab_bytes(c));
+        if (e != cudaSuccess) {
+            c->cap_views = c->cap_segs = c->cap_pairs = 0;   // (the next frame tries again)
+            return cuda_status(e);
+        }
     }
-    int slot = (c->slot + 1) % curast_ctx::kSlots, left = 0;
-    while (c->kept[slot]) slot = (slot + 1) % curast_ctx::kSlots;   // one is always left
-    for (bool k : c->kept) left += !k;
+    int left = 0;
+    for (int k = 0; k < curast_ctx::kSlots; ++k) {
+        if (is_kept(c, k)) continue;
+        ++left;
+        if (c->h_tab[k].cap < tab_bytes(c)) {
+            CU(cudaEventSynchronize(c->ev_tab[k]));
+            CU(c->h_tab[k].reserve(tab_bytes(c)));
+        }
+    }
     if (capturing && left == 1) return CURAST_ERR_CUDA;
+    int slot = (c->slot + 1) % curast_ctx::kSlots;
+    while (is_kept(c, slot)) slot = (slot + 1) % curast_ctx::kSlots;
+    // the slot may still feed the frame of four calls ago
+    CU(cudaEventSynchronize(c->ev_tab[slot]));
     c->slot = slot;
     c->kept[slot] = capturing;
-    // the slot may still feed the frame of four calls ago
-    CU(cudaEventSynchronize(c->ev_tab[c->slot]));
     unsigned char *h = c->h_tab[c->slot].p;
     std::memcpy(h, &c->hdr, sizeof(FrameHdr));
     std::memcpy(h + kRoundsOff, c->rounds.data(), c->rounds.size() * sizeof(RoundDev));
@@ -717,9 +745,9 @@ curast_status shade_setup(curast_ctx *c, const float *view, const float *proj, i
 }
 
 curast_status alloc_queues(curast_ctx *c) {
-    c->d_q1.release();
-    c->d_q2.release();
-    c->d_sorted.release();
+    c->d_q1.release(keep(c));
+    c->d_q2.release(keep(c));
+    c->d_sorted.release(keep(c));
     CU(c->d_q1.reserve(std::max<uint64_t>(c->cfg.queue1_capacity, 1)));
     CU(c->d_q2.reserve(std::max<uint64_t>(c->cfg.queue2_capacity, 1)));
     CU(c->d_sorted.reserve(std::max<uint64_t>(c->cfg.queue2_capacity, 1)));
@@ -901,6 +929,7 @@ void curast_destroy(curast_ctx *c) {
     cudaDeviceSynchronize();
     invalidate_graph(c);
     for (MeshRec &m : c->meshes) free_compressed(m);
+    free_outgrown(c);
     c->d_meshes.release();
     c->d_inst.release();
     c->d_inst_mv.release();
