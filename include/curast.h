@@ -59,6 +59,7 @@ typedef int32_t curast_status;
 #define CURAST_ERR_BAD_CAMERA           -8  /* proj is not symmetric perspective*/
 #define CURAST_ERR_NOT_BUILT            -9  /* no kernel image for this device  */
 #define CURAST_ERR_TOO_LARGE           -10  /* over a fixed capacity of curast_render_static */
+#define CURAST_ERR_CAPTURES            -11  /* three captured frames of the context are alive */
 
 typedef struct curast_ctx curast_ctx;
 
@@ -224,6 +225,19 @@ curast_status curast_add_instance(curast_ctx *ctx, uint32_t mesh_id, const float
 curast_status curast_clear_instances(curast_ctx *ctx);
 
 /* ------------------------------------------------------------ render --- */
+
+/* Stream capture.  curast_render, curast_render_mesh and curast_render_batch
+ * with use_graph = 0 may be captured by the caller into a CUDA graph, in
+ * relaxed mode, once a frame of the same scene and views was rendered directly
+ * (the tables and buffers are then in place).  A replay renders the frame as it was captured, whatever was rendered since.
+ * Up to three captured frames of a context can be alive, a further capture is
+ * refused with CURAST_ERR_CAPTURES; a frame is alive until its graph and every executable
+ * graph made from it are destroyed, and buffers that the context outgrows
+ * meanwhile stay allocated as long.  Direct frames are not limited.  Frames of
+ * one context, direct or replayed, must not overlap on the device, and none
+ * may be replayed after curast_destroy.
+ * The screen passes (curast_resolve and the like) over at most sixteen
+ * instances keep matrices and mesh buffers as they were captured. */
 
 /* Fills a visibility buffer with 0xFF..FF (device, n words). */
 curast_status curast_clear(uint64_t *vis, uint64_t n, curast_stream stream);

@@ -21,7 +21,7 @@ STATUS_NAMES = {
     0: "CURAST_OK", -1: "CURAST_ERR_INVALID_ARG", -2: "CURAST_ERR_OUT_OF_MEMORY", -3: "CURAST_ERR_ID_SPACE_OVERFLOW",
     -4: "CURAST_ERR_INDEX_OUT_OF_RANGE", -5: "CURAST_ERR_DEVICE_TIMEOUT", -6: "CURAST_ERR_CUDA",
     -7: "CURAST_ERR_NOT_AFFINE", -8: "CURAST_ERR_BAD_CAMERA", -9: "CURAST_ERR_NOT_BUILT",
-    -10: "CURAST_ERR_TOO_LARGE",
+    -10: "CURAST_ERR_TOO_LARGE", -11: "CURAST_ERR_CAPTURES",
 }
 STATIC_MAX_INSTANCES = 32
 EXPORTS = ["curast_create", "curast_destroy", "curast_status_string", "curast_get_config", "curast_set_config",

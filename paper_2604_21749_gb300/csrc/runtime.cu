@@ -6,9 +6,11 @@
 // exclusive prefix sum of triangle counts for the global ids, and a copy of
 // all of it to the GPU; then the stage kernels are enqueued.
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <new>
 #include <vector>
 
@@ -211,13 +213,13 @@ struct curast_ctx {
 
     // frame tables: [hdr | views | segs | pairs], one device copy and a ring of pinned ones, so that the host
     // can prepare frames while earlier ones run (ev_tab: the frame that read the slot is done, or its copy).
-    // A frame captured by the caller keeps its slot, which replays read again, and with it every device buffer
-    // that is outgrown later.
+    // A frame captured by the caller keeps its slot, which replays read again, as long as its graph lives
+    // (kept: true until then), and with it every device buffer that is outgrown meanwhile.
     DevBuf<unsigned char> d_tab;
     static constexpr int kSlots = 4;
     PinBuf<unsigned char> h_tab[kSlots];
     cudaEvent_t ev_tab[kSlots] = {nullptr, nullptr, nullptr, nullptr};
-    bool kept[kSlots] = {false, false, false, false};
+    std::shared_ptr<std::atomic<bool>> kept[kSlots];
     std::vector<void *> outgrown;
     int slot = 0;
     size_t cap_views = 0, cap_segs = 0, cap_pairs = 0;
@@ -284,7 +286,7 @@ void invalidate_graph(curast_ctx *c) {
     c->gkey.clear();
 }
 
-bool is_kept(const curast_ctx *c, int slot) { return c->kept[slot]; }
+bool is_kept(const curast_ctx *c, int slot) { return c->kept[slot] && c->kept[slot]->load(std::memory_order_acquire); }
 
 // Where buffers that a captured frame may name go when they are outgrown: null where there is no such frame.
 std::vector<void *> *keep(curast_ctx *c) {
@@ -296,6 +298,37 @@ std::vector<void *> *keep(curast_ctx *c) {
 void free_outgrown(curast_ctx *c) {
     for (void *p : c->outgrown) cudaFree(p);
     c->outgrown.clear();
+}
+
+void CUDART_CB graph_gone(void *p) {
+    auto *alive = static_cast<std::shared_ptr<std::atomic<bool>> *>(p);
+    (*alive)->store(false, std::memory_order_release);
+    delete alive;
+}
+
+// Ties the slot to the graph that s is being captured into: the runtime calls
+// graph_gone once the graph and everything instantiated from it are destroyed
+// (also where the capture fails or is given up).
+curast_status keep_slot(curast_ctx *c, int slot, cudaStream_t s) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaGraph_t graph = nullptr;
+    CU(cudaStreamGetCaptureInfo(s, &cap, nullptr, &graph));
+    if (cap != cudaStreamCaptureStatusActive) return CURAST_ERR_CUDA;
+    auto alive = std::make_shared<std::atomic<bool>>(true);
+    auto *own = new std::shared_ptr<std::atomic<bool>>(alive);
+    cudaUserObject_t obj = nullptr;
+    const cudaError_t e = cudaUserObjectCreate(&obj, own, graph_gone, 1, cudaUserObjectNoDestructorSync);
+    if (e != cudaSuccess) {
+        delete own;
+        return cuda_status(e);
+    }
+    const cudaError_t r = cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove);
+    if (r != cudaSuccess) {
+        cudaUserObjectRelease(obj, 1);
+        return cuda_status(r);
+    }
+    c->kept[slot] = alive;
+    return CURAST_OK;
 }
 
 MeshDev mesh_dev(const MeshRec &r) {
@@ -508,7 +541,7 @@ size_t tab_bytes(const curast_ctx *c) { return off_pairs(c) + c->cap_pairs * siz
 // Fills the next pinned copy of the frame's tables; the frame's first kernel
 // reads it in place.  Three of the copies may belong to captured frames: one is
 // always left for the others.
-curast_status stage_frame(curast_ctx *c, bool capturing) {
+curast_status stage_frame(curast_ctx *c, bool capturing, cudaStream_t s) {
     if (c->hv.size() > c->cap_views || c->hs.size() > c->cap_segs || c->hp.size() > c->cap_pairs) {
         for (cudaEvent_t e : c->ev_tab) CU(cudaEventSynchronize(e));
         c->cap_views = std::max<size_t>(c->hv.size(), std::max<size_t>(2 * c->cap_views, 8));
@@ -531,13 +564,16 @@ curast_status stage_frame(curast_ctx *c, bool capturing) {
             CU(c->h_tab[k].reserve(tab_bytes(c)));
         }
     }
-    if (capturing && left == 1) return CURAST_ERR_CUDA;
+    if (capturing && left == 1) return CURAST_ERR_CAPTURES;
     int slot = (c->slot + 1) % curast_ctx::kSlots;
     while (is_kept(c, slot)) slot = (slot + 1) % curast_ctx::kSlots;
     // the slot may still feed the frame of four calls ago
     CU(cudaEventSynchronize(c->ev_tab[slot]));
+    if (capturing) {
+        const curast_status st = keep_slot(c, slot, s);
+        if (st != CURAST_OK) return st;
+    }
     c->slot = slot;
-    c->kept[slot] = capturing;
     unsigned char *h = c->h_tab[c->slot].p;
     std::memcpy(h, &c->hdr, sizeof(FrameHdr));
     std::memcpy(h + kRoundsOff, c->rounds.data(), c->rounds.size() * sizeof(RoundDev));
@@ -654,7 +690,8 @@ curast_status render_views(curast_ctx *c, const curast_view *views, int nv, long
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     CU(cudaStreamIsCapturing(s, &cap));
     const bool capturing = cap != cudaStreamCaptureStatusNone;
-    st = stage_frame(c, capturing);
+    if (!capturing && !c->outgrown.empty() && !keep(c)) free_outgrown(c);
+    st = stage_frame(c, capturing, s);
     if (st != CURAST_OK) return st;
     if (!graph) {
         st = enqueue_stages(c, clear, capturing ? Frame::captured : Frame::direct, s);
@@ -882,6 +919,7 @@ const char *curast_status_string(curast_status s) {
     case CURAST_ERR_NOT_AFFINE: return "matrix is not affine";
     case CURAST_ERR_BAD_CAMERA: return "projection is not a symmetric perspective matrix";
     case CURAST_ERR_NOT_BUILT: return "no kernel image for this device";
+    case CURAST_ERR_CAPTURES: return "three captured frames of the context are alive";
     case CURAST_ERR_TOO_LARGE: return "exceeds a fixed capacity of the no-allocation render";
     default: return "unknown status";
     }

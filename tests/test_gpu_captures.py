@@ -1,5 +1,9 @@
-"""A context with captured frames alive renders whatever it rendered without
-them: larger tables, bitmaps and queues among it."""
+"""Frames captured by the caller give back what they hold when their graph is
+gone, and a context with captured frames alive renders whatever it rendered
+without them: larger tables, bitmaps and queues among it."""
+import gc
+import time
+
 import numpy as np
 import pytest
 import torch
@@ -29,19 +33,55 @@ def _view(k=0):
             97 + 16 * k, 61 + 8 * k)
 
 
-def _capture(r, view, vis):
+def _capture(api, r, view, vis, status=None):
+    """The captured frame, or None where it was refused (with `status`, if one is expected)."""
     g = torch.cuda.CUDAGraph()
+    ok = True
     with torch.cuda.stream(torch.cuda.Stream()):
         g.capture_begin(capture_error_mode="relaxed")
-        r.render(*view, vis=vis)
+        try:
+            r.render(*view, vis=vis)
+        except api.CurastError as e:
+            ok = False
+            assert status is None or e.status == status
         g.capture_end()
-    return g
+    return g if ok else None
 
 
 def _replay(g):
     torch.cuda.synchronize()
     g.replay()
     torch.cuda.synchronize()
+
+
+@pytest.mark.filterwarnings("ignore:The CUDA Graph is empty")
+def test_slots_come_back(api, scene):
+    """Three are alive at a time, a fourth is refused by name, and any number
+    one after the other is taken (the runtime tells of a graph's end a moment
+    after it)."""
+    r = api.Renderer()
+    keep = upload(r, scene, with_colour=False)
+    want = r.render(*_view())
+    r.sync()
+    vis = torch.zeros_like(want)
+    graphs = [_capture(api, r, _view(), vis) for _ in range(3)]
+    assert all(graphs)
+    assert _capture(api, r, _view(), vis, status=-11) is None
+    for _ in range(8):
+        graphs.pop(0).reset()
+        gc.collect()
+        deadline = time.time() + 10.0
+        g = None
+        while g is None and time.time() < deadline:
+            g = _capture(api, r, _view(), vis, status=-11)
+            if g is None:
+                time.sleep(0.01)
+        assert g is not None, "the slot of a destroyed graph did not come back"
+        graphs.append(g)
+        vis.zero_()
+        _replay(g)
+        assert_vis_equal(vis, u64(want), "captured frame")
+    del keep
 
 
 def test_a_context_grows_beside_captured_frames(api, scene):
@@ -53,7 +93,8 @@ def test_a_context_grows_beside_captured_frames(api, scene):
     want = r.render(*_view())
     r.sync()
     vis = torch.zeros_like(want)
-    graph = _capture(r, _view(), vis)
+    graph = _capture(api, r, _view(), vis)
+    assert graph
     rng = np.random.default_rng(2)
     for step in range(3):
         for _ in range(400):
