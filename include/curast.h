@@ -129,7 +129,9 @@ typedef struct {
     uint64_t triangles_in;       /* triangle x (instance, view) pairs entering stage 1 */
     uint64_t culled_clip;        /* whole triangle beyond one clip plane               */
     uint64_t culled_backface;    /* area <= 0 after snapping (stage 1)                 */
-    uint64_t culled_tiny;        /* bbox holds no pixel centre (stage 1)               */
+    uint64_t culled_tiny;        /* bbox holds no pixel centre, or dropped by the conservative
+                                    cull as beyond the near plane (stage 1).  A triangle that is
+                                    this and a back face as well is counted once, in either      */
     uint64_t stage1_rasterized;
     uint64_t queued_stage2;
     uint64_t stage2_rasterized;  /* sub-triangles rasterized by stage 2                */

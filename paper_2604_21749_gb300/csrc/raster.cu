@@ -550,23 +550,26 @@ __global__ void k_aabb_final(const float *part, int n, float *out) {
 }
 
 // -------------------------------------------------------------- launchers --
-template <bool INST, bool COMP, bool NEAR>
+template <bool INST, bool COMP, bool NEAR, bool STATS = false>
 cudaError_t stage1_shape(int *blocks) {
     const size_t sm = stage1_smem_bytes<INST>();
-    cudaError_t e = cudaFuncSetAttribute(k_stage1<INST, COMP, NEAR>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    const auto k = k_stage1<INST, COMP, NEAR, STATS>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     if (e != cudaSuccess) return e;
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k_stage1<INST, COMP, NEAR>, s1::kThreads, sm);
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks, k, s1::kThreads, sm);
 }
 
 cudaError_t query_launch_shape(LaunchShape *o, int device) {
     cudaError_t e = cudaDeviceGetAttribute(&o->num_sms, cudaDevAttrMultiProcessorCount, device);
     if (e != cudaSuccess) return e;
-    {   // the forms without the near-plane test run at the same shape
+    {   // the forms without the near-plane test and those that count run at the same shape
         int b = 0;
         if ((e = stage1_shape<false, false, false>(&b)) != cudaSuccess) return e;
         if ((e = stage1_shape<false, true, false>(&b)) != cudaSuccess) return e;
         if ((e = stage1_shape<true, false, false>(&b)) != cudaSuccess) return e;
         if ((e = stage1_shape<true, true, false>(&b)) != cudaSuccess) return e;
+        if ((e = stage1_shape<true, false, true, true>(&b)) != cudaSuccess) return e;
+        if ((e = stage1_shape<true, true, true, true>(&b)) != cudaSuccess) return e;
     }
     if ((e = stage1_shape<false, false, true>(&o->stage1_blocks_per_sm[0][0])) != cudaSuccess) return e;
     if ((e = stage1_shape<false, true, true>(&o->stage1_blocks_per_sm[0][1])) != cudaSuccess) return e;
@@ -624,17 +627,16 @@ cudaError_t launch_stage1(const FrameDev &f, bool instanced, int variant, uint32
                           cudaStream_t s) {
     const size_t s0 = stage1_smem_bytes<false>(), si = stage1_smem_bytes<true>();
     const bool p = f.pdl != 0;
-    if (instanced) {
-        if (variant == 1 && near) return launch_stage(p, k_stage1<true, true, true>, blocks, s1::kThreads, si, s, f, r);
-        if (variant == 1) return launch_stage(p, k_stage1<true, true, false>, blocks, s1::kThreads, si, s, f, r);
-        if (near) return launch_stage(p, k_stage1<true, false, true>, blocks, s1::kThreads, si, s, f, r);
-        return launch_stage(p, k_stage1<true, false, false>, blocks, s1::kThreads, si, s, f, r);
+    if (instanced) {                                  // (frames that count test for the near plane, needed or not)
+        const auto k = f.stats ? (variant == 1 ? k_stage1<true, true, true, true> : k_stage1<true, false, true, true>)
+                       : near  ? (variant == 1 ? k_stage1<true, true, true, false> : k_stage1<true, false, true, false>)
+                               : (variant == 1 ? k_stage1<true, true, false, false> : k_stage1<true, false, false, false>);
+        return launch_stage(p, k, blocks, s1::kThreads, si, s, f, r);
     }
-    if (variant == 2) return launch_stage(p, k_stage1_win, blocks, s1::kThreads, stage1_win_smem_bytes(), s, f, r);
-    if (variant == 1 && near) return launch_stage(p, k_stage1<false, true, true>, blocks, s1::kThreads, s0, s, f, r);
-    if (variant == 1) return launch_stage(p, k_stage1<false, true, false>, blocks, s1::kThreads, s0, s, f, r);
-    if (near) return launch_stage(p, k_stage1<false, false, true>, blocks, s1::kThreads, s0, s, f, r);
-    return launch_stage(p, k_stage1<false, false, false>, blocks, s1::kThreads, s0, s, f, r);
+    const auto k = variant == 2 ? k_stage1_win
+                   : near       ? (variant == 1 ? k_stage1<false, true, true, false> : k_stage1<false, false, true, false>)
+                                : (variant == 1 ? k_stage1<false, true, false, false> : k_stage1<false, false, false, false>);
+    return launch_stage(p, k, blocks, s1::kThreads, variant == 2 ? stage1_win_smem_bytes() : s0, s, f, r);
 }
 
 cudaError_t launch_stage1_exact(const FrameDev &f, bool comp, uint32_t r, int blocks, cudaStream_t s) {
