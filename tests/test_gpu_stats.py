@@ -10,6 +10,7 @@ from synthetic.scenes import Camera, Instance, Mesh, Scene
 from test_cull_bounds import _exact
 
 from gpu_util import upload
+from test_gpu_stage1_exact import _slivers
 
 pytestmark = pytest.mark.gpu
 
@@ -74,3 +75,14 @@ def test_back_faces_and_tiny_triangles(api, order, copies, group):
         assert st["culled_backface"] + st["culled_tiny"] == back + none - both
         assert back - both <= st["culled_backface"] <= back, (st, back, both)
         assert none - both <= st["culled_tiny"] <= none, (st, none, both)
+
+
+HEAVY = [(32, 32), (31, 33), (1024, 1), (40, 25)]
+
+
+def test_handed_over_triangles_are_counted_once(api):
+    """Batches of up to 96 x 1024 pixels, part of which stage 1 hands to stage 2:
+    each triangle is stage 1's or stage 2's."""
+    st = _stats(api, _slivers(700, 1100, 1060, seed=5, shapes=HEAVY), stage1_max_pixels=1024, stage1_exact_all=1)
+    assert st["queue1_overflow"] == 0 and st["stage1_rasterized"] > 0 and st["queued_stage3"] == 0
+    assert st["stage2_rasterized"] == st["queued_stage2"] > 100, st
