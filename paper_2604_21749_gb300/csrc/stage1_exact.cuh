@@ -482,7 +482,11 @@ __global__ void __launch_bounds__(32 * s1::kExactWarps, 1)
             if (lane == 0) atomicAdd(&f.ctr->q1_px, (unsigned long long)px);
             base = __shfl_sync(0xffffffffu, base, 0) + __popc(all & lt_mask);
             if (f.stats && lane == 0) stat_add(f, kStatS1, 0ull - (unsigned long long)__popc(all));   // now stage 2's
-            if (!want || base >= f.q1_cap) return false;
+            if (!want) return false;
+            if (base >= f.q1_cap) {
+                atomicAdd(&f.ctr->overflow1, 1ull);
+                return false;
+            }
             const uint2 e = S.e[slot];
             f.q1[base] = Q1Entry{f.pairs[e.y].base + e.x, e.y, 1u};
             return true;

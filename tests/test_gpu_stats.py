@@ -86,3 +86,13 @@ def test_handed_over_triangles_are_counted_once(api):
     st = _stats(api, _slivers(700, 1100, 1060, seed=5, shapes=HEAVY), stage1_max_pixels=1024, stage1_exact_all=1)
     assert st["queue1_overflow"] == 0 and st["stage1_rasterized"] > 0 and st["queued_stage3"] == 0
     assert st["stage2_rasterized"] == st["queued_stage2"] > 100, st
+
+
+@pytest.mark.parametrize("capacity", [1, 50, 300])
+def test_hand_over_to_a_full_queue_is_an_overflow(api, capacity):
+    """What the first queue has no room for is rasterized in place and counted as
+    that, wherever it was to be queued from; the rest is stage 2's."""
+    st = _stats(api, _slivers(700, 1100, 1060, seed=5, shapes=HEAVY), stage1_max_pixels=1024, stage1_exact_all=1,
+                queue1_capacity=capacity)
+    assert st["queue1_overflow"] == st["queued_stage2"] - capacity > 0, st
+    assert st["stage2_rasterized"] == capacity and st["queued_stage3"] == 0, st
