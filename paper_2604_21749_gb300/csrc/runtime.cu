@@ -543,7 +543,8 @@ size_t tab_bytes(const curast_ctx *c) { return off_pairs(c) + c->cap_pairs * siz
 // always left for the others.
 curast_status stage_frame(curast_ctx *c, bool capturing, cudaStream_t s) {
     if (c->hv.size() > c->cap_views || c->hs.size() > c->cap_segs || c->hp.size() > c->cap_pairs) {
-        for (cudaEvent_t e : c->ev_tab) CU(cudaEventSynchronize(e));
+        if (c->d_tab.p)
+            for (cudaEvent_t e : c->ev_tab) CU(cudaEventSynchronize(e));
         c->cap_views = std::max<size_t>(c->hv.size(), std::max<size_t>(2 * c->cap_views, 8));
         c->cap_segs = std::max<size_t>(c->hs.size(), std::max<size_t>(2 * c->cap_segs, 256));
         c->cap_pairs = std::max<size_t>(c->hp.size(), std::max<size_t>(2 * c->cap_pairs, 256));
@@ -560,7 +561,7 @@ curast_status stage_frame(curast_ctx *c, bool capturing, cudaStream_t s) {
         if (is_kept(c, k)) continue;
         ++left;
         if (c->h_tab[k].cap < tab_bytes(c)) {
-            CU(cudaEventSynchronize(c->ev_tab[k]));
+            if (c->h_tab[k].p) CU(cudaEventSynchronize(c->ev_tab[k]));
             CU(c->h_tab[k].reserve(tab_bytes(c)));
         }
     }
