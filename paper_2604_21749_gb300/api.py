@@ -171,7 +171,10 @@ def _ptr(t: Optional[torch.Tensor]):
 def _stream(stream=None):
     if stream is not None:
         return stream.cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    try:
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    except AttributeError:                       # (private to torch: a version without them)
+        return torch.cuda.current_stream().cuda_stream
 
 
 def _need(t: torch.Tensor, dtype, what: str, device):
