@@ -228,16 +228,18 @@ curast_status curast_clear_instances(curast_ctx *ctx);
 
 /* ------------------------------------------------------------ render --- */
 
-/* Stream capture.  curast_render, curast_render_mesh and curast_render_batch
- * with use_graph = 0 may be captured by the caller into a CUDA graph, in
- * relaxed mode, once a frame of the same scene and views was rendered directly
- * (the tables and buffers are then in place).  A replay renders the frame as it was captured, whatever was rendered since.
- * Up to three captured frames of a context can be alive, a further capture is
- * refused with CURAST_ERR_CAPTURES; a frame is alive until its graph and every executable
- * graph made from it are destroyed, and buffers that the context outgrows
- * meanwhile stay allocated as long.  Direct frames are not limited.  Frames of
- * one context, direct or replayed, must not overlap on the device, and none
- * may be replayed after curast_destroy.
+/* Stream capture. curast_render, curast_render_mesh and
+ * curast_render_batch with use_graph = 0 may be captured by the caller
+ * into a CUDA graph, in relaxed mode, once a frame of the same scene and
+ * views was rendered directly (the tables and buffers are then in place).
+ * A replay renders the frame as it was captured, whatever was rendered
+ * since. Up to three captured frames of a context can be alive, a further
+ * capture is refused with CURAST_ERR_CAPTURES; a frame is alive until its
+ * graph and every executable graph made from it are destroyed, and buffers
+ * that the context outgrows meanwhile stay allocated as long. Direct
+ * frames are not limited. Frames of one context, direct or replayed, must
+ * not overlap on the device, and none may be replayed after
+ * curast_destroy.
  * The screen passes (curast_resolve and the like) over at most sixteen
  * instances keep matrices and mesh buffers as they were captured. */
 

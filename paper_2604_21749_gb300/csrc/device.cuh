@@ -117,8 +117,6 @@ struct MeshDev {
     int32_t tex_log2, pad2;
 };
 
-__device__ __forceinline__ bool compressed(const MeshDev &m) { return m.cidx != nullptr; }
-
 // Index word k (= 3 t + corner) of a mesh, decoded when compressed.
 __device__ __forceinline__ uint32_t mesh_index(const MeshDev &m, uint64_t k) {
     if (!m.cidx) return __ldg(m.idx + k);
@@ -419,11 +417,12 @@ __device__ __forceinline__ uint64_t frag_key(int64_t E0, int64_t E1, int64_t E2,
 }
 
 // Section 3.1: the closest fragment wins by a 64-bit atomic minimum, a
-// reduction that needs no answer, issued directly in every stage.  (Stages 2
-// and 3 once read the stored word first, to skip the atomic behind nearer
-// pixels: every pixel then waited for the read.  A 4K frame of triangles of
-// 1900 pixels each: stage 2 297 us with the reads, four in flight, 216 us
-// without, stage 3 41 and 33 us.)
+// reduction that needs no answer, issued directly in every stage.  Reading the
+// stored word first, to skip the atomic behind nearer pixels, makes every pixel
+// wait for the read, and does not pay under any overdraw either: 32 layers that
+// fill 3840 x 2160, front to back, back to front and mixed, us with the read and
+// without: triangles of 60 pixels a side 2875 2951 2876 for 2067 2067 2075,
+// of 400 1296 1307 1304 for 1025 1024 1027.
 __device__ __forceinline__ void depth_min(uint64_t *vis, size_t pix, uint64_t key) {
     atomicMin(reinterpret_cast<unsigned long long *>(vis + pix), (unsigned long long)key);
 }

@@ -14,7 +14,6 @@
 // nearly every step for a lane or two.
 #pragma once
 
-
 namespace s1 {
 constexpr int kExactWarps = 20;                      // one block an SM, 96 registers a thread
 constexpr int kExactK = 3;                           // survivors a lane gathers together
@@ -24,25 +23,20 @@ constexpr uint32_t kUnitSurvivors = 128;             // survivors of a unit, abo
 constexpr int kDenseBits = 12;                       // words with as many survivors are unpacked by the whole warp
 constexpr uint32_t kSegPx = 1024;                    // pixels whose triangle starts are marked at once
 
-// A small triangle ready for the pixel loop, 48 bytes: eight lanes' 16-byte
-// loads of neighbouring records touch every bank once.
-struct __align__(16) SmallTri {
-    int e0, e1, A;             // edge functions 0 and 1 at the centre of pixel (x0, y0); their sum with edge 2
-    int c0, c1;                // edges 0 (vertex 1 to 2) and 1 (2 to 0): dx + 65536 dy, in subpixels.  The sign
-                               // is that of dy, or of dx where dy is 0: negative for a top-left edge.
-    float iz[3];               // 1/depth of the vertices
-    uint32_t id;               // global id, low word
-    uint32_t idh;              // its 4 high bits | view << 8
-    uint32_t at;               // x0 | y0 << 16 of the pixel range
-    uint32_t shape;            // its width w | ceil(2^20 / w) << 11
-};
-static_assert(sizeof(SmallTri) == 3 * sizeof(uint4), "a record is three 16-byte words");
+// A small triangle ready for the pixel loop is three 16-byte words (eight lanes'
+// 16-byte loads of neighbouring records touch every bank once):
+//   e0, e1, A, c0     edge functions 0 and 1 at the centre of pixel (x0, y0); the sum of all three;
+//   c1, iz[3]         c0, c1: edges 0 (vertex 1 to 2) and 1 (2 to 0) as dx + 65536 dy, in subpixels.  The
+//                     sign is that of dy, or of dx where dy is 0: negative for a top-left edge.
+//                     iz: 1/depth of the vertices
+//   id, idh, at, sh   the global id's low word; its 4 high bits | view << 8; x0 | y0 << 16 of the pixel
+//                     range; its width w | ceil(2^20 / w) << 11
 
 // Up to 32 K small triangles of one warp, K a lane, and the pixel loop's marks.
 template <int K>
 struct SmallBatch {
-    uint4 t[32 * K][3];        // the SmallTri of each slot
-    uint32_t npx[32 * K];    // pixels of its range (0: nothing to rasterize)
+    uint4 t[32 * K][3];        // the record of each slot
+    uint32_t npx[32 * K];      // pixels of its range (0: nothing to rasterize)
     uint32_t list[32 * K];     // triangles with pixels: first pixel of the batch | slot << 20
     uint32_t starts[kSegPx / 32];   // bit i: pixel i of the segment is a triangle's first
 };
@@ -279,7 +273,7 @@ size_t exact_smem_bytes() { return sizeof(s1::ExactWarp) * s1::kExactWarps; }
 // bitmap in units of 1 .. 128 words, a word, two or four for each lane:
 // survivors come in clusters where the view looks closely, and a fixed deal of
 // 32-word chunks to warps left some SMs with twice the average (the full-HD
-// view of a 4.2 M-triangle mesh: 179 us, 105 us now).  A unit in a cluster
+// view of a 4.2 M-triangle mesh: 179 us, 108 now).  A unit in a cluster
 // holds some 128 survivors: with 64 the fetches cost more than the balance gains (75 M
 // triangles compressed: 671 us against 621), with 512 single units last too
 // long (the full-HD view 147 us, a clustered 100 M-triangle view 537 against
@@ -471,9 +465,10 @@ __global__ void __launch_bounds__(32 * s1::kExactWarps, 1)
             exact_setup<RAY>(f, S, lane + 32 * u, lane + 32 * u < n);
         __syncwarp();
         // a batch of heavy triangles (a near surface, up to 128 pixels each) would keep its warp long after
-        // the others: what starts past kSegPx pixels goes to stage 2, which deals triangles out finely (a
-        // close 4K view of a 100 M-triangle scan: exact kernel and stage 2 521 + 67 us, 453 + 41 us with it
-        // past 2048 pixels; past 1024 or 2048, 349 + 68 and 385 + 46; past 512, 322 + 116)
+        // the others: of a batch of more than 2 kSegPx pixels, the triangles that start past pixel kSegPx go
+        // to stage 2, which deals them out finely.  Exact kernel + stage 2, us, of a close 4K view of a 100 M-
+        // triangle scan and of the full-HD view: none handed over 439 + 29, 110 + 11; kSegPx 2048 351 + 38,
+        // 111 + 12; 1024 303 + 67, 108 + 12; 512 305 + 115, 94 + 17
         small_raster<kExactK>(f, S, lane, [&](bool want, int slot) -> bool {
             unsigned long long base = 0;
             const unsigned all = __ballot_sync(0xffffffffu, want);

@@ -26,7 +26,9 @@ constexpr uint64_t kStaticQ2 = 1ull << 14;    // queue-2 tile parts (64 B each);
 constexpr int kBoundBlocks = 304;             // partial bounds of the positions
 constexpr uint64_t kItem = 1024;              // triangles of a stage-1 work item
 // A frame of fewer (triangle, instance)s than this takes the exact path for all of them: finding the mesh's
-// bounds would take longer than it saves.
+// bounds, a pass over the positions whose end the set-up waits for, costs 11 us.  Terrain seen as a whole at
+// 1280 x 720, us with the bounds and without: 2^15 64 / 53, 2^17 54 / 43, 2^19 65 / 53, 2^21 84 / 78, and of
+// four instances 2^20 77 / 67, 2^22 109 / 131, 2^23 133 / 225: for such views the line could lie at 2^21.
 constexpr uint64_t kCullFrom = 1ull << 17;
 
 constexpr size_t al(size_t x) { return (x + 255) / 256 * 256; }
