@@ -379,7 +379,14 @@ __global__ void __launch_bounds__(32 * s1::kExactWarps, 1)
                 const uint64_t at = rd.w0 + word;
                 w_next = fetch();
                 if (m | m1 | m2 | m3) {
-                    while (seg + 1 < n_segs && f.segs[seg + 1].word0 <= at) ++seg;
+                    // the run's segment: strides doubled forward, then halved (20,000 meshes of one instance
+                    // each walked one by one: exact kernel 14.8 ms, 0.20 so)
+                    int stride = 1;
+                    for (; seg + stride < n_segs && f.segs[seg + stride].word0 <= at; stride <<= 1) seg += stride;
+                    while (stride > 1) {
+                        stride >>= 1;
+                        if (seg + stride < n_segs && f.segs[seg + stride].word0 <= at) seg += stride;
+                    }
                     const SegDev &sg = f.segs[seg];
                     const uint64_t local = at - sg.word0;
                     const uint32_t per = sg.npairs * G;         // words per item (<= 64 * 32)
