@@ -107,6 +107,7 @@ struct ShadeArgs {
     const MeshDev *meshes;
     int n_inst;
     int rows;                   // pixel rows a thread walks (set by the launchers)
+    uint64_t tris;              // triangles of all instances
     // resolve
     float *rgba_f32;
     uint8_t *rgba8;

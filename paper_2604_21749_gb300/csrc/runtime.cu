@@ -779,6 +779,7 @@ curast_status shade_setup(curast_ctx *c, const float *view, const float *proj, i
     a->inst = c->d_inst.p;
     a->meshes = c->d_meshes.p;
     a->n_inst = (int)n;
+    a->tris = c->base[n];
     return CURAST_OK;
 }
 

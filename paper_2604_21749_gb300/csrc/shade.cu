@@ -634,10 +634,15 @@ __global__ void __launch_bounds__(32 * kBwdWarps) k_interp_bwd(const __grid_cons
 // 2, 4 rows: 213, 146, 134 us; at 1920 x 1080: 47.0, 42.5, 43.7; at 300 x 200:
 // 4.3, 4.9, 7.2 (one row a thread and every ray for itself: 174, 46, 5.0).
 // (With the instances as parameters: 3840 x 2160 with 4 rows 123, 1920 x 1080
-// with 2 rows 37.)
-static int rows_of(int W, int H) {
-    const long long px = (long long)W * H;
-    return px >= 4000000 ? 4 : px >= 300000 ? 2 : 1;
+// with 2 rows 37.)  Where many triangles fall to a pixel, the gathers of a
+// column share nothing and four rows only spread a block's addresses: with 36
+// triangles a pixel at 3840 x 2160 4, 2, 1 rows took 334, 311, 320 us, with 121
+// 516, 492, 488, with 259 642, 615, 597 (one row a thread and every ray for
+// itself: 340, 496, 602).  Nothing here tells a close view of such a scene,
+// which likes four rows (12 triangles a pixel, close: 126, 148, 185; 219 so).
+static int rows_of(const ShadeArgs &a) {
+    const uint64_t px = (uint64_t)a.W * (uint64_t)a.H;
+    return px >= 4000000 ? (a.tris < 64 * px ? 4 : 1) : px >= 300000 ? 2 : 1;
 }
 
 static dim3 pixel_grid(int W, int H, int rows) { return dim3((unsigned)((W + 31) / 32), (unsigned)((H + 8 * rows - 1) / (8 * rows))); }
@@ -651,7 +656,7 @@ cudaError_t launch_resolve_ss(const ShadeArgs &a, int W, int H, cudaStream_t s) 
 }
 
 cudaError_t launch_resolve(ShadeArgs &a, cudaStream_t s) {
-    a.rows = rows_of(a.W, a.H);
+    a.rows = rows_of(a);
     const dim3 grid = pixel_grid(a.W, a.H, a.rows);
     if (a.n_inst <= kFew) k_resolve<true><<<grid, 256, 0, s>>>(a);
     else k_resolve<false><<<grid, 256, 0, s>>>(a);
@@ -659,7 +664,7 @@ cudaError_t launch_resolve(ShadeArgs &a, cudaStream_t s) {
 }
 
 cudaError_t launch_resolve_textured(ShadeArgs &a, cudaStream_t s) {
-    a.rows = rows_of(a.W, a.H);
+    a.rows = rows_of(a);
     const dim3 grid = pixel_grid(a.W, a.H, a.rows);
     if (a.n_inst <= kFew) k_resolve_tex<true><<<grid, 256, 0, s>>>(a);
     else k_resolve_tex<false><<<grid, 256, 0, s>>>(a);
@@ -675,7 +680,7 @@ static void interp_fwd(const ShadeArgs &a, dim3 grid, cudaStream_t s) {
 }
 
 cudaError_t launch_interpolate(ShadeArgs &a, cudaStream_t s) {
-    a.rows = rows_of(a.W, a.H);
+    a.rows = rows_of(a);
     const dim3 grid = pixel_grid(a.W, a.H, a.rows);
     if (a.n_inst <= kFew) interp_fwd<true>(a, grid, s);
     else interp_fwd<false>(a, grid, s);
