@@ -182,7 +182,8 @@ curast_status curast_set_config(curast_ctx *ctx, const curast_config *cfg);
  * Every stage then renders the decoded positions fma(q, step, lo) in FP32,
  * step = (float)((hi - lo) / 65535), and the decoded indices.  Meshes whose
  * indices reach V are rejected with CURAST_ERR_INDEX_OUT_OF_RANGE.  A
- * compressed mesh cannot be updated and has no differentiable path. */
+ * compressed mesh takes other colours, but no other positions or indices
+ * (curast_update_mesh), and has no differentiable path. */
 #define CURAST_MESH_COMPRESSED 1u
 curast_status curast_upload_mesh(curast_ctx *ctx, const float *pos, uint64_t V, const uint32_t *idx,
                                  uint64_t T, const uint8_t *rgba8, uint32_t flags, uint32_t *mesh_id);

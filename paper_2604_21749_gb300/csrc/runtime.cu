@@ -1048,8 +1048,10 @@ curast_status curast_update_mesh(curast_ctx *c, uint32_t mesh_id, const float *p
     if (pos) m.pos = pos;
     if (idx) m.idx = idx;
     if (rgba8) m.rgba = rgba8;
-    curast_status st = compute_bounds(c, m);
-    if (st != CURAST_OK) return st;
+    if (!m.comp) {                                   // (a compressed mesh has no positions of its own, nor other bounds)
+        const curast_status st = compute_bounds(c, m);
+        if (st != CURAST_OK) return st;
+    }
     c->meshes_dirty = true;
     return CURAST_OK;
 }
